@@ -167,7 +167,9 @@ double dev_norm(Ctx& c, int64_t n, const double* v, double* slot) {
   return h;
 }
 
-void check_status(Ctx& c) {
+// Throws for the errors of the kernels since the last call; true when only the
+// merged coarse inverse has to be redone by the banded LU.
+bool check_status(Ctx& c) {
   int32_t st[ST_COUNT];
   ck(cudaMemcpyAsync(st, c.status, sizeof(st), cudaMemcpyDeviceToHost, c.stream), "D2H status");
   sync(c);
@@ -180,11 +182,62 @@ void check_status(Ctx& c) {
   if (st[ST_TANGLED]) throw ApiError(FSI_E_MESH_TANGLED, "det F <= 0 at a quadrature point");
   if (st[ST_NONFINITE]) throw ApiError(FSI_E_NONFINITE, "non-finite values");
   if (st[ST_SINGULAR]) throw ApiError(FSI_E_SINGULAR, "zero or non-finite pivot in a Schwarz block or coarse LU");
+  return st[ST_COARSE_RETRY] != 0;
 }
 
 // ---------------------------------------------------------------------------
 // build
 // ---------------------------------------------------------------------------
+// Merge tree of the 2D coarse inverse over the slabs of an ordering: ranges
+// are halved.  Null when there are no slabs or they do not fit the kernel's
+// shared memory.
+std::shared_ptr<CoarseTree> make_tree(const HostLevel& H, int* max_leaf, int* max_s) {
+  const int K = (int)H.free_slab_off.size() - 1, p = H.free_p;
+  if (H.dim != 2 || K < 1 || K > kMaxLeaves) return nullptr;
+  auto t = std::make_shared<CoarseTree>();
+  t->nleaf = K;
+  for (int k = 0; k <= K; ++k) t->off[k] = (int)H.free_slab_off[k];
+  std::vector<std::vector<CoarseMerge>> lv;
+  auto split = [&](auto&& self, int lo, int hi) -> int {   // returns the height of [lo, hi)
+    if (hi - lo == 1) return 0;
+    const int mid = (lo + hi) / 2;
+    const int h = std::max(self(self, lo, mid), self(self, mid, hi));
+    if ((int)lv.size() <= h) lv.resize(h + 1);
+    lv[h].push_back({t->off[lo], t->off[mid], t->off[hi], t->off[mid + 1] - t->off[mid]});
+    return h + 1;
+  };
+  split(split, 0, K);
+  t->nlev = (int)lv.size();
+  int n = 0;
+  for (size_t h = 0; h < lv.size(); ++h) {
+    t->level[h] = n;
+    for (const CoarseMerge& m : lv[h]) t->merge[n++] = m;
+  }
+  t->level[lv.size()] = n;
+  *max_leaf = *max_s = 0;
+  for (int k = 0; k < K; ++k) *max_leaf = std::max(*max_leaf, t->off[k + 1] - t->off[k]);
+  for (int i = 0; i < n; ++i) *max_s = std::max(*max_s, t->merge[i].s);
+  return coarse_merge_fits(*max_leaf, p, *max_s) ? t : nullptr;
+}
+
+// sizes of the slab-blocked solve of an ordering
+void slab_sizes(CoarseOrder& o) {
+  const int K = (int)o.slab_off.size() - 1;
+  o.sinv_off.assign(K + 1, 0);
+  for (int k = 0; k < K; ++k) {
+    const int64_t m = o.slab_off[k + 1] - o.slab_off[k];
+    o.mmax = std::max<int>(o.mmax, (int)m);
+    o.sinv_off[k + 1] = o.sinv_off[k] + m * m;
+  }
+}
+
+// doubles of its scratch: left factors, coupling blocks, two p x p matrices per merge of a level
+size_t tree_gh_doubles(const CoarseTree& t, int p) {
+  int most = 0;
+  for (int l = 0; l < t.nlev; ++l) most = std::max(most, t.level[l + 1] - t.level[l]);
+  return (size_t)most * 2 * p * p;
+}
+
 void build_device(Ctx& c) {
   const int L = (int)c.hl.size();
   c.dl.assign(L, DevLevel());
@@ -356,44 +409,55 @@ void build_device(Ctx& c) {
   c.dense_ws = dalloc<double>(c, c.mixed ? ((size_t)c.dense_ws_len + 1) / 2 : (size_t)c.dense_ws_len);
   // coarse dense operator
   const int64_t n0 = c.hl[0].Ni;
-  c.c_A = dalloc<double>(c, (size_t)n0 * n0);   // banded LU in dense column-major storage
+  c.c_A = dalloc<double>(c, (size_t)n0 * n0);   // dense operator / banded LU, column-major
   c.c_B = dalloc<double>(c, (size_t)2 * n0);   // reciprocal pivots of the coarse LU
   c.c_piv = dalloc<int32_t>(c, n0);
-  c.coarse_slab = c.dim == 3 && !c.hl[0].slab_off.empty();
-  if (!c.coarse_slab) {
-    c.c_inv = dalloc<double>(c, (size_t)n0 * n0);   // column-major inverse
-    c.c_part = dalloc<double>(c, (size_t)((n0 + 31) / 32) * n0);   // coarse GEMV chunk partials
-  } else {
-    // block-tridiagonal slab factorisation: inverse Schur complements Sinv_k
-    const HostLevel& H0 = c.hl[0];
-    c.slab_off = H0.slab_off;
-    c.slab_p = H0.slab_p;
-    const int K = (int)c.slab_off.size() - 1;
-    c.sinv_off.assign(K + 1, 0);
-    for (int k = 0; k < K; ++k) {
-      const int64_t m = c.slab_off[k + 1] - c.slab_off[k];
-      c.slab_mmax = std::max<int>(c.slab_mmax, (int)m);
-      c.sinv_off[k + 1] = c.sinv_off[k] + m * m;
-    }
-    const int64_t mm = c.slab_mmax;
-    c.c_sinv = dalloc<double>(c, (size_t)c.sinv_off[K]);
-    c.c_S = dalloc<double>(c, (size_t)mm * mm);
-    c.c_T = dalloc<double>(c, (size_t)c.slab_p * mm);
-    c.c_zb = dalloc<double>(c, n0);
-    c.c_xb = dalloc<double>(c, n0);
-    c.c_tp = dalloc<double>(c, c.slab_p);
-    c.c_part = dalloc<double>(c, (size_t)((mm + 31) / 32) * mm);
-    std::vector<int32_t> iota(mm);
-    std::iota(iota.begin(), iota.end(), 0);
-    c.c_iota = upload(c, iota);
-  }
+  c.c_rhs = dalloc<double>(c, n0);
+  c.c_dr = dalloc<double>(c, n0);
   {
     const HostLevel& H0 = c.hl[0];
-    std::vector<int32_t> pinv(H0.Ni);
-    for (int64_t i = 0; i < H0.Ni; ++i) pinv[H0.coarse_perm[i]] = (int32_t)i;
-    c.coarse_perm = upload(c, H0.coarse_perm);
-    c.coarse_pinv = upload(c, pinv);
-    c.coarse_bw = H0.coarse_bw;
+    std::vector<int32_t> inv(n0), iota(n0);
+    for (int64_t i = 0; i < n0; ++i) inv[H0.coarse_perm[i]] = (int32_t)i;
+    std::iota(iota.begin(), iota.end(), 0);
+    c.c_iota = upload(c, iota);
+    CoarseOrder &fr = c.co[0], &all = c.co[1];
+    fr.n = (int64_t)H0.free_map.size();
+    fr.pos = upload(c, H0.free_pos);
+    fr.map = upload(c, H0.free_map);
+    fr.bw = H0.free_bw;
+    fr.p = H0.free_p;
+    fr.slab_off = H0.free_slab_off;
+    all.n = n0;
+    all.pos = upload(c, H0.coarse_perm);
+    all.map = upload(c, inv);
+    all.bw = H0.coarse_bw;
+    all.p = H0.slab_p;
+    all.slab_off = H0.slab_off;
+    for (CoarseOrder& o : c.co) {
+      o.slab = c.dim == 3 && !o.slab_off.empty();
+      if (o.slab) slab_sizes(o);
+    }
+    if (fr.slab != all.slab) fr = all;
+    if (c.dim == 2) fr.tree = make_tree(H0, &fr.tree_leaf, &fr.tree_s);
+    if (fr.tree) {
+      c.c_L = dalloc<double>(c, (size_t)fr.n * fr.p);
+      c.c_Bp = dalloc<double>(c, (size_t)fr.n * fr.p);
+      c.c_gh = dalloc<double>(c, tree_gh_doubles(*fr.tree, fr.p));
+    }
+    if (!all.slab) {
+      c.c_inv = dalloc<double>(c, (size_t)n0 * n0);   // column-major inverse
+      c.c_part = dalloc<double>(c, (size_t)((n0 + 31) / 32) * n0);   // coarse GEMV chunk partials
+    } else {
+      // block-tridiagonal slab factorisation: inverse Schur complements Sinv_k
+      const int64_t mm = all.mmax;
+      c.c_sinv = dalloc<double>(c, (size_t)all.sinv_off.back());
+      c.c_S = dalloc<double>(c, (size_t)mm * mm);
+      c.c_T = dalloc<double>(c, (size_t)all.p * mm);
+      c.c_zb = dalloc<double>(c, n0);
+      c.c_xb = dalloc<double>(c, n0);
+      c.c_tp = dalloc<double>(c, all.p);
+      c.c_part = dalloc<double>(c, (size_t)((mm + 31) / 32) * mm);
+    }
   }
   c.status = dalloc<int32_t>(c, ST_COUNT);
   ck(cudaMemsetAsync(c.status, 0, ST_COUNT * sizeof(int32_t), c.stream), "memset");
@@ -426,6 +490,7 @@ void assemble(Ctx& c, bool want_res) {
 }
 
 void assemble_impl(Ctx& c) {
+  c.coarse_imported = false;
   const int L = (int)c.dl.size();
   const int B = c.B;
   DevLevel& F = c.dl[L - 1];
@@ -526,32 +591,39 @@ void assemble_impl(Ctx& c) {
 // only on the last x-plane P of slab k-1, the update is
 // A_{k,k-1}[:,P] (S_{k-1}^{-1}[P,P] A_{k-1,k}[P,:]).
 // ---------------------------------------------------------------------------
-void coarse_factor_slab(Ctx& c) {
+void coarse_gather(Ctx& c) {
   DevLevel& C = c.dl[0];
-  const int64_t n0 = C.Ni;
-  const int K = (int)c.slab_off.size() - 1;
-  const int p = c.slab_p;
+  const CoarseOrder& o = c.ord();
+  const int npad = o.n == C.Ni ? c.n_coarse_pads : 0;
+  launch_dense_gather(c.B, C.nb, C.rowptr, C.col, C.val, c.coarse_pad_list, npad, o.pos, o.n, c.c_dr, c.c_A,
+                      c.stream);
+  counted(c, npad > 0 ? 3 : 2);
+}
+
+void coarse_factor_slab(Ctx& c) {
+  const CoarseOrder& co = c.ord();
+  const int64_t n0 = co.n;
+  const int K = (int)co.slab_off.size() - 1;
+  const int p = co.p;
   double flops = 0.0, bytes = (double)n0 * n0 * 8.0;
   for (int k = 0; k < K; ++k) {
-    const double m = (double)(c.slab_off[k + 1] - c.slab_off[k]);
+    const double m = (double)(co.slab_off[k + 1] - co.slab_off[k]);
     flops += 2.0 * m * m * m * (2.0 / 3.0 + 1.0);   // LU + inverse columns
     if (k > 0) flops += 2.0 * p * (double)p * m + 2.0 * m * p * m;
     bytes += 3.0 * m * m * 8.0;
   }
-  Prof pr(c, FSI_K_COARSE_FACTOR, bytes, flops, (c.n_coarse_pads > 0 ? 2 : 1) + 3 * K + 2 * (K - 1));
-  launch_dense_gather(c.B, C.nb, C.rowptr, C.col, C.val, c.coarse_pad_list, c.n_coarse_pads, c.coarse_perm, n0,
-                      c.c_A, c.stream);
-  counted(c, c.n_coarse_pads > 0 ? 2 : 1);
+  Prof pr(c, FSI_K_COARSE_FACTOR, bytes, flops, 1 + 3 * K + 2 * (K - 1));
+  coarse_gather(c);
   for (int k = 0; k < K; ++k) {
-    const int64_t o = c.slab_off[k];
-    const int m = (int)(c.slab_off[k + 1] - o);
+    const int64_t o = co.slab_off[k];
+    const int m = (int)(co.slab_off[k + 1] - o);
     double* Akk = c.c_A + o * n0 + o;
     launch_copy2d(m, m, Akk, n0, c.c_S, m, c.stream);
     counted(c);
     if (k > 0) {
-      const int64_t op = c.slab_off[k - 1];
+      const int64_t op = co.slab_off[k - 1];
       const int mp = (int)(o - op);
-      const double* Sp = c.c_sinv + c.sinv_off[k - 1];
+      const double* Sp = c.c_sinv + co.sinv_off[k - 1];
       // T = S_{k-1}^{-1}[P,P] A_{k-1,k}[P,:]   (p x m)
       launch_dgemm_nn(p, m, p, 1.0, Sp + (int64_t)(mp - p) * mp + (mp - p), mp, c.c_A + o * n0 + (o - p), n0, 0.0,
                       c.c_T, p, c.stream);
@@ -559,56 +631,82 @@ void coarse_factor_slab(Ctx& c) {
       launch_dgemm_nn(m, m, p, -1.0, c.c_A + (o - p) * n0 + o, n0, c.c_T, p, 1.0, c.c_S, m, c.stream);
       counted(c, 2);
     }
-    const int rc = launch_coarse_lu_inverse(m, m - 1, m - 1, c.c_S, c.c_B, c.c_sinv + c.sinv_off[k], c.c_piv,
+    const int rc = launch_coarse_lu_inverse(m, m - 1, m - 1, c.c_S, c.c_B, c.c_sinv + co.sinv_off[k], c.c_piv,
                                             c.c_iota, c.c_iota, c.status, c.sm_count, c.stream);
     if (rc != 0) throw ApiError(FSI_E_CUDA, "slab LU launch failed (" + std::to_string(rc) + ")");
     counted(c, 2);
   }
 }
 
-// x = A_0^{-1} b (internal ordering, FP64): forward block elimination
-// w_k = b_k - A_{k,k-1}[:,P] (S_{k-1}^{-1}[P,:] w_{k-1}), then back
+// x = A_0^{-1} b over the ordering (FP64, b in c_zb, x in c_xb): forward block
+// elimination w_k = b_k - A_{k,k-1}[:,P] (S_{k-1}^{-1}[P,:] w_{k-1}), then back
 // substitution x_k = S_k^{-1} (w_k - A_{k,k+1} x_{k+1}) with A_{k,k+1}
 // nonzero in the rows P of slab k only.
-void coarse_apply_slab(Ctx& c, const double* b, double* x) {
-  const int64_t n0 = c.dl[0].Ni;
-  const int K = (int)c.slab_off.size() - 1;
-  const int p = c.slab_p;
-  launch_gather(n0, c.coarse_pinv, b, c.c_zb, c.stream);
-  counted(c);
+void coarse_apply_slab(Ctx& c) {
+  const CoarseOrder& co = c.ord();
+  const int64_t n0 = co.n;
+  const int K = (int)co.slab_off.size() - 1;
+  const int p = co.p;
   for (int k = 1; k < K; ++k) {
-    const int64_t o = c.slab_off[k], op = c.slab_off[k - 1];
-    const int m = (int)(c.slab_off[k + 1] - o), mp = (int)(o - op);
-    const double* Sp = c.c_sinv + c.sinv_off[k - 1];
+    const int64_t o = co.slab_off[k], op = co.slab_off[k - 1];
+    const int m = (int)(co.slab_off[k + 1] - o), mp = (int)(o - op);
+    const double* Sp = c.c_sinv + co.sinv_off[k - 1];
     launch_gemv_sub(p, mp, 1.0, Sp + (mp - p), mp, c.c_zb + op, 0.0, c.c_tp, c.c_part, c.stream);
     launch_gemv_sub(m, p, -1.0, c.c_A + (o - p) * n0 + o, n0, c.c_tp, 1.0, c.c_zb + o, c.c_part, c.stream);
     counted(c, 4);
   }
   for (int k = K - 1; k >= 0; --k) {
-    const int64_t o = c.slab_off[k];
-    const int m = (int)(c.slab_off[k + 1] - o);
+    const int64_t o = co.slab_off[k];
+    const int m = (int)(co.slab_off[k + 1] - o);
     if (k < K - 1) {
-      const int64_t on = c.slab_off[k + 1];
-      const int mn = (int)(c.slab_off[k + 2] - on);
+      const int64_t on = co.slab_off[k + 1];
+      const int mn = (int)(co.slab_off[k + 2] - on);
       launch_gemv_sub(p, mn, -1.0, c.c_A + on * n0 + (on - p), n0, c.c_xb + on, 1.0, c.c_zb + (on - p), c.c_part,
                       c.stream);
       counted(c, 2);
     }
-    launch_gemv_sub(m, m, 1.0, c.c_sinv + c.sinv_off[k], m, c.c_zb + o, 0.0, c.c_xb + o, c.c_part, c.stream);
+    launch_gemv_sub(m, m, 1.0, c.c_sinv + co.sinv_off[k], m, c.c_zb + o, 0.0, c.c_xb + o, c.c_part, c.stream);
     counted(c, 2);
   }
-  launch_gather(n0, c.coarse_perm, c.c_xb, x, c.stream);
-  counted(c);
 }
 
 double coarse_slab_apply_bytes(const Ctx& c) {
-  const int K = (int)c.slab_off.size() - 1;
+  const CoarseOrder& co = c.ord();
+  const int K = (int)co.slab_off.size() - 1;
   double b = 0.0;
   for (int k = 0; k < K; ++k) {
-    const double m = (double)(c.slab_off[k + 1] - c.slab_off[k]);
-    b += m * m * 8.0 + (k > 0 ? 2.0 * c.slab_p * m * 8.0 : 0.0);
+    const double m = (double)(co.slab_off[k + 1] - co.slab_off[k]);
+    b += m * m * 8.0 + (k > 0 ? 2.0 * co.p * m * 8.0 : 0.0);
   }
   return b;
+}
+
+// x = J_0^{-1} b, internal layout, FP64 inverse and accumulation; TB the type
+// of both vectors.  Unknowns that the ordering leaves out are identity rows
+// (x = b); their columns move to the right-hand side on a one-level instance,
+// where J_0 is the assembled operator (a Galerkin operator has none: the grid
+// transfers drop them).
+template <typename TB>
+void coarse_solve(Ctx& c, const TB* b, TB* x, double* part) {
+  DevLevel& C = c.dl[0];
+  const CoarseOrder& o = c.ord();
+  const bool shift = c.dl.size() == 1 && o.n < C.Ni;
+  if (shift) {
+    launch_coarse_rhs<TB>(c.B, C.nb, C.rowptr, C.col, C.val, o.pos, b, c.c_rhs, c.stream);
+    counted(c);
+  }
+  if (o.slab) {
+    if (shift) launch_coarse_pick<double>(o.n, o.map, c.c_dr, c.c_rhs, c.c_zb, c.stream);
+    else launch_coarse_pick<TB>(o.n, o.map, c.c_dr, b, c.c_zb, c.stream);
+    counted(c);
+    coarse_apply_slab(c);
+    launch_coarse_scatter<TB, TB>(C.Ni, o.pos, c.c_xb, b, x, c.stream);
+    counted(c);
+  } else {
+    if (shift) launch_gemv<double, TB>(C.Ni, o.n, c.c_inv, o.pos, o.map, c.c_dr, c.c_rhs, x, part, c.stream);
+    else launch_gemv<TB, TB>(C.Ni, o.n, c.c_inv, o.pos, o.map, c.c_dr, b, x, part, c.stream);
+    counted(c, 2);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -737,24 +835,67 @@ void schwarz_factor(Ctx& c) {
   }
 }
 
+// 2D, any band: banded LU and the inverse's columns by triangular solves
+void coarse_factor_banded(Ctx& c) {
+  const CoarseOrder& o = c.ord();
+  const double nn = (double)o.n;
+  // banded LU (2 n kl (kl + ku) flops) + inverse columns (~2 n^2 (kl + ku) flops, sparsity aside)
+  const double bw = (double)o.bw;
+  Prof pr(c, FSI_K_COARSE_FACTOR, nn * nn * 8.0 * 3.0, 2.0 * nn * bw * 2.0 * bw + 2.0 * nn * nn * 2.0 * bw, 4);
+  coarse_gather(c);
+  const int rc = launch_coarse_lu_inverse(o.n, o.bw, o.bw, c.c_A, c.c_B, c.c_inv, c.c_piv, c.c_iota, c.c_iota,
+                                          c.status, c.sm_count, c.stream);
+  if (rc != 0) throw ApiError(FSI_E_CUDA, "banded coarse LU launch failed (" + std::to_string(rc) + ")");
+  counted(c, 2);
+}
+
+// The merged inverse needs nonsingular slab ranges, which the LU's pivoting
+// across slabs does not; its result is therefore checked on one vector (rows
+// of A x - v against |A| |x| + |v|; both inverses measure below 1e-10 there, a
+// breakdown order 1), and factor() falls back to the LU when that fails.
+constexpr double kCoarseCheckTol = 1e-6;
+
+void drop_vcycle_graph(Ctx& c) {
+  if (c.vc_exec) cudaGraphExecDestroy(c.vc_exec);
+  if (c.vc_graph) cudaGraphDestroy(c.vc_graph);
+  c.vc_exec = nullptr;
+  c.vc_graph = nullptr;
+  c.vc_graph_failed = false;
+}
+
+// The Dirichlet rows of J_0 are identity rows, so its solve is one over the
+// free unknowns (2D 16 x 4 cells: 1,074 of 1,444; 3D 16 x 4 x 4: 10,200 of
+// 17,574, in slabs of 652 instead of 1,068), unless level 0 was imported.
 void coarse_factor(Ctx& c) {
-  const int B = c.B;
   DevLevel& C = c.dl[0];
-  const int64_t n0 = C.Ni;
-  if (c.coarse_slab) {
+  const int which = c.coarse_imported ? 1 : 0;
+  if (which != c.co_now) {
+    c.co_now = which;
+    drop_vcycle_graph(c);   // the recorded V-cycle solves over the other ordering
+  }
+  const CoarseOrder& o = c.ord();
+  if (o.slab) {
     coarse_factor_slab(c);
+  } else if (o.tree) {
+    double flops = 0.0;
+    const CoarseTree& t = *o.tree;
+    const double p = o.p;
+    for (int k = 0; k < t.nleaf; ++k) flops += 2.0 * std::pow((double)(t.off[k + 1] - t.off[k]), 3);
+    for (int i = 0; i < t.level[t.nlev]; ++i) {
+      const double w = t.merge[i].b - t.merge[i].a;
+      flops += 2.0 * p * w * (w + t.merge[i].s + 2.0 * p);
+    }
+    Prof pr(c, FSI_K_COARSE_FACTOR, (double)o.n * o.n * 8.0 * 3.0, flops, 6);
+    coarse_gather(c);
+    const int rc = launch_coarse_merge(t, o.n, o.p, o.tree_leaf, o.tree_s, c.c_A, c.c_L, c.c_Bp, c.c_gh, c.c_inv,
+                                       c.status, c.sm_count, c.stream);
+    if (rc != 0) throw ApiError(FSI_E_CUDA, "merged coarse inverse launch failed (" + std::to_string(rc) + ")");
+    launch_coarse_probe(C.Ni, o.pos, C.b, c.stream);
+    launch_gemv<double, double>(C.Ni, o.n, c.c_inv, o.pos, o.map, c.c_dr, C.b, C.x, c.c_part, c.stream);
+    launch_coarse_check(c.B, C.nb, C.rowptr, C.col, C.val, C.b, C.x, kCoarseCheckTol, o.pos, c.status, c.stream);
+    counted(c, 5);
   } else {
-    const double nn = (double)n0;
-    // banded LU (2 n kl (kl + ku) flops) + inverse columns (~2 n^2 (kl + ku) flops, sparsity aside)
-    const double bw = (double)c.coarse_bw;
-    Prof pr(c, FSI_K_COARSE_FACTOR, nn * nn * 8.0 * 3.0, 2.0 * nn * bw * 2.0 * bw + 2.0 * nn * nn * 2.0 * bw, 4);
-    launch_dense_gather(B, C.nb, C.rowptr, C.col, C.val, c.coarse_pad_list, c.n_coarse_pads, c.coarse_perm, n0,
-                        c.c_A, c.stream);
-    counted(c, c.n_coarse_pads > 0 ? 2 : 1);
-    const int rc = launch_coarse_lu_inverse(n0, c.coarse_bw, c.coarse_bw, c.c_A, c.c_B, c.c_inv, c.c_piv,
-                                            c.coarse_perm, c.coarse_pinv, c.status, c.sm_count, c.stream);
-    if (rc != 0) throw ApiError(FSI_E_CUDA, "banded coarse LU launch failed (" + std::to_string(rc) + ")");
-    counted(c, 2);
+    coarse_factor_banded(c);
   }
 }
 
@@ -806,7 +947,10 @@ void factor(Ctx& c) {
   schwarz_factor(c);
   if (fork) cudaStreamWaitEvent(c.stream, c.ev_join, 0);
   else coarse_factor(c);
-  check_status(c);
+  if (check_status(c)) {
+    coarse_factor_banded(c);
+    check_status(c);
+  }
   c.factored = true;
   c.b_factor = c.alg_bytes - b0;
 }
@@ -819,6 +963,16 @@ void spmv(Ctx& c, int l, const double* x, const double* b, double* y, int kind =
   Prof pr(c, kind, D.spmv_bytes - (b ? 0.0 : D.Ni * 8.0), D.spmv_flops);
   launch_bsr_residual(c.B, D.nb, D.rowptr, D.col, D.val, x, b, y, c.stream);
   counted(c);
+}
+
+// coarsest-grid solve of the V-cycle
+template <typename T>
+void coarse_grid(Ctx& c, const T* b, T* x) {
+  const CoarseOrder& o = c.ord();
+  const double n = (double)o.n, io = 2.0 * (double)c.dl[0].Ni * sizeof(T);
+  const double by = o.slab ? coarse_slab_apply_bytes(c) : n * n * 8.0;
+  Prof pr(c, FSI_K_TRANSFER, by + io, by / 4.0, o.slab ? 2 + 8 * ((int)o.slab_off.size() - 1) : 2);
+  coarse_solve<T>(c, b, x, c.c_part);
 }
 
 // Level data of the V-cycle in precision T (double: FP64 path, float: mixed).
@@ -848,18 +1002,7 @@ template <> struct VC<double> {
     launch_csr_spmv(D.Ni, D.P_ptr, D.P_col, D.P_val, xc, x, true, c.stream);
     counted(c);
   }
-  static void coarse(Ctx& c, const double* b, double* x) {
-    const double n0 = (double)c.dl[0].Ni;
-    if (c.coarse_slab) {
-      const double by = coarse_slab_apply_bytes(c);
-      Prof pr(c, FSI_K_TRANSFER, by + 4.0 * n0 * 8.0, by / 4.0, 2 + 8 * ((int)c.slab_off.size() - 1));
-      coarse_apply_slab(c, b, x);
-      return;
-    }
-    Prof pr(c, FSI_K_TRANSFER, n0 * n0 * 8.0 + 2.0 * n0 * 8.0, 2.0 * n0 * n0);
-    launch_gemv(c.dl[0].Ni, c.c_inv, b, x, c.c_part, c.stream);
-    counted(c, 2);
-  }
+  static void coarse(Ctx& c, const double* b, double* x) { coarse_grid<double>(c, b, x); }
 };
 template <> struct VC<float> {
   static float* x(DevLevel& D) { return D.x32; }
@@ -901,23 +1044,8 @@ template <> struct VC<float> {
     launch_csr_spmv_f32(D.Ni, D.P_ptr, D.P_col, D.P_val32, xc, x, true, c.stream);
     counted(c);
   }
-  static void coarse(Ctx& c, const float* b, float* x) {
-    // the coarsest-grid solve stays FP64 (FP64 inverse, FP64 accumulation)
-    const double n0 = (double)c.dl[0].Ni;
-    if (c.coarse_slab) {
-      const double by = coarse_slab_apply_bytes(c);
-      Prof pr(c, FSI_K_TRANSFER, by + 4.0 * n0 * 8.0 + 2.0 * n0 * 4.0, by / 4.0, 4 + 8 * ((int)c.slab_off.size() - 1));
-      launch_to_f64(c.dl[0].Ni, b, c.c_xb, c.stream);
-      counted(c);
-      coarse_apply_slab(c, c.c_xb, c.c_zb);   // both buffers are free again when it writes its result
-      launch_to_f32(c.dl[0].Ni, c.c_zb, x, c.stream);
-      counted(c);
-      return;
-    }
-    Prof pr(c, FSI_K_TRANSFER, n0 * n0 * 8.0 + 2.0 * n0 * 4.0, 2.0 * n0 * n0);
-    launch_gemv_f32io(c.dl[0].Ni, c.c_inv, b, x, c.c_part, c.stream);
-    counted(c, 2);
-  }
+  // the coarsest-grid solve stays FP64 (FP64 inverse, FP64 accumulation)
+  static void coarse(Ctx& c, const float* b, float* x) { coarse_grid<float>(c, b, x); }
 };
 
 template <typename T>
@@ -1362,7 +1490,9 @@ static int64_t estimate_device_bytes(const Ctx& c) {
   double sum_dense = 0.0;
   for (size_t l = 1; l < L; ++l) sum_dense += (double)c.hl[l].dense_total;
   b += (mixed ? sum_dense : max_dense) * fs + F.n_elem * (double)nd * 8.0 + 1e6;
-  const std::vector<int64_t>& so = c.hl[0].slab_off;
+  const HostLevel& H0 = c.hl[0];
+  const std::vector<int64_t>& so = H0.slab_off;
+  b += 2.0 * n0 * 8.0 + H0.free_map.size() * 4.0 + n0 * 4.0;   // right-hand side, row scales, free ordering
   if (c.dim == 3 && !so.empty()) {
     // dense banded-order operator + Sinv_k blocks + LU scratch + vectors
     double mm = 0.0, sum = 0.0;
@@ -1371,9 +1501,12 @@ static int64_t estimate_device_bytes(const Ctx& c) {
       mm = std::max(mm, m);
       sum += m * m;
     }
-    b += n0 * n0 * 8.0 + (sum + mm * mm + c.hl[0].slab_p * mm + mm * mm / 32.0 + mm) * 8.0 + 6.0 * n0 * 8.0;
+    b += n0 * n0 * 8.0 + (sum + mm * mm + H0.slab_p * mm + mm * mm / 32.0 + mm) * 8.0 + 6.0 * n0 * 8.0;
   } else {
     b += 2.0 * n0 * n0 * 8.0 + (n0 / 32.0 + 1.0) * n0 * 8.0 + 2.0 * n0 * 8.0;
+    int leaf = 0, s = 0;
+    if (const auto t = make_tree(H0, &leaf, &s))
+      b += (2.0 * H0.free_map.size() * H0.free_p + (double)tree_gh_doubles(*t, H0.free_p)) * 8.0;
   }
   return (int64_t)b;
 }
@@ -1765,7 +1898,10 @@ int fsi_factor_schwarz_batch(fsi_ctx* const* ctxs, int n) {
     const float ms = elapsed(*c0);
     for (int i = 0; i < n; ++i) {
       Ctx& c = *ctxs[i];
-      check_status(c);
+      if (check_status(c)) {
+        coarse_factor_banded(c);
+        check_status(c);
+      }
       c.factored = true;
       c.t_factor = ms;
       double by = 0.0;   // the Schwarz gathers and inverses (the coarse LU is in the level-0 estimate)
@@ -1936,6 +2072,20 @@ int fsi_import_csr(fsi_ctx* c, int level, const double* val) {
         }
     }
     ck(cudaMemcpyAsync(D.val, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream), "H2D");
+    if (level == 0) {
+      // the coarse solve leaves Dirichlet unknowns out when their rows are
+      // identity rows (and, below other levels, nothing couples to them)
+      bool identity = true;
+      const bool cols = c->dl.size() > 1;
+      for (int64_t br = 0; br < H.nb && identity; ++br)
+        for (int32_t k = H.rowptr[br]; k < H.rowptr[br + 1]; ++k)
+          for (int e = 0; e < B * B; ++e) {
+            const int64_t i = br * B + e / B, j = (int64_t)H.col[k] * B + e % B;
+            const double x = v[(size_t)k * B * B + e];
+            if (H.dir[i] ? x != (i == j ? 1.0 : 0.0) : cols && H.dir[j] && x != 0.0) identity = false;
+          }
+      c->coarse_imported = !identity;
+    }
     if (c->mixed && level >= 1) {
       launch_to_f32((int64_t)v.size(), D.val, D.val32, c->stream);
       counted(*c);
@@ -2102,7 +2252,7 @@ int fsi_coarse_solve_static(fsi_ctx* c, const double* b, double* x) {
   return guard(c, [&] {
     need_device(*c);
     if (!b || !x) throw ApiError(FSI_E_INVALID, "null pointer");
-    if (c->coarse_slab)
+    if (c->ord().slab)
       throw ApiError(FSI_E_INVALID, "fsi_coarse_solve_static: the slab-blocked (3D) coarse LU is not supported");
     DevLevel& C = c->dl[0];
     const int64_t n0 = C.Ni;
@@ -2120,8 +2270,7 @@ int fsi_coarse_solve_static(fsi_ctx* c, const double* b, double* x) {
                                         ") is not the device the ctx was built on (" + std::to_string(c->device) + ")");
     double* part = static_part(dev);
     to_internal(*c, 0, b, C.b);
-    launch_gemv(n0, c->c_inv, C.b, C.x, part, c->stream);
-    counted(*c, 2);
+    coarse_solve<double>(*c, C.b, C.x, part);
     to_canonical(*c, 0, C.x, x);
     sync(*c);
   });
@@ -2191,14 +2340,6 @@ int fsi_set_profiling(fsi_ctx* c, int on) {
 // ---------------------------------------------------------------------------
 // launch parameters (autotuner)
 // ---------------------------------------------------------------------------
-static void drop_vcycle_graph(Ctx& c) {
-  if (c.vc_exec) cudaGraphExecDestroy(c.vc_exec);
-  if (c.vc_graph) cudaGraphDestroy(c.vc_graph);
-  c.vc_exec = nullptr;
-  c.vc_graph = nullptr;
-  c.vc_graph_failed = false;
-}
-
 int fsi_set_launch_params(fsi_ctx* c, int level, const fsi_launch_params* p) {
   return guard(c, [&] {
     need_device(*c);

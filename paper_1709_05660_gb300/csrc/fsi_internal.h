@@ -11,6 +11,7 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -89,6 +90,12 @@ struct HostLevel {
   // and k runs only through the last slab_p positions of slab k-1
   std::vector<int64_t> slab_off;
   int slab_p = 0;
+  // the banded ordering restricted to the free unknowns (Dirichlet rows are
+  // identity rows; padding slots): internal unknown -> position or -1, its
+  // inverse, half-bandwidth, slabs and free unknowns per interface plane
+  std::vector<int32_t> free_pos, free_map;
+  int free_bw = 0, free_p = 0;
+  std::vector<int64_t> free_slab_off;
 };
 
 bool build_host_hierarchy(const fsi_problem_desc& d, const fsi_solver_opts& o,
@@ -152,6 +159,19 @@ struct DevLevel {
   double factor_bytes = 0, factor_flops = 0, R_bytes = 0, P_bytes = 0;
 };
 
+struct CoarseTree;   // kernels.h
+
+// One ordering of the coarse unknowns and the solver that it takes
+struct CoarseOrder {
+  int64_t n = 0;
+  int32_t *pos = nullptr, *map = nullptr;   // internal unknown -> position (-1: left out) and back
+  int bw = 0, p = 0, mmax = 0;              // half-bandwidth, interface plane, largest slab
+  std::vector<int64_t> slab_off, sinv_off;
+  bool slab = false;                        // slab-blocked LU (3D)
+  std::shared_ptr<CoarseTree> tree;         // merged inverse (2D, slabs small enough)
+  int tree_leaf = 0, tree_s = 0;            // largest leaf; largest first leaf of a right part
+};
+
 struct Ctx {
   fsi_problem_desc desc;
   fsi_solver_opts opts;
@@ -194,14 +214,17 @@ struct Ctx {
   bool have_history = false;
   bool factored = false;   // fsi_factor_schwarz has run at least once
   int32_t* coarse_pad_list = nullptr;     // padding slots of the coarse dense operator
-  int32_t* coarse_perm = nullptr;         // internal unknown -> banded position
-  int32_t* coarse_pinv = nullptr;         // banded position -> internal unknown
-  int coarse_bw = 0;
   int n_coarse_pads = 0;
+  // orderings of the coarse solve: 0 = free unknowns only (Dirichlet rows are
+  // identity rows), 1 = all of them (an imported operator may have any rows)
+  CoarseOrder co[2];
+  int co_now = 0;                         // ordering of the last factorisation
+  bool coarse_imported = false;           // level 0 was imported since the last assembly
+  const CoarseOrder& ord() const { return co[co_now]; }
+  double *c_L = nullptr, *c_Bp = nullptr, *c_gh = nullptr;   // scratch of the merged inverse
+  double* c_dr = nullptr;                 // row scales of the coarse operator
+  double* c_rhs = nullptr;                // right-hand side less the Dirichlet columns (one level)
   // slab-blocked coarse solve (3D): Sinv_k blocks, LU scratch, vectors
-  bool coarse_slab = false;
-  std::vector<int64_t> slab_off, sinv_off;
-  int slab_p = 0, slab_mmax = 0;
   double *c_sinv = nullptr, *c_S = nullptr, *c_T = nullptr, *c_zb = nullptr, *c_xb = nullptr, *c_tp = nullptr;
   int32_t* c_iota = nullptr;
   float t_assemble = 0.f, t_factor = 0.f, t_solve = 0.f;
@@ -235,6 +258,8 @@ struct Ctx {
 };
 
 // status flag slots
-enum { ST_SINGULAR = 0, ST_TANGLED = 1, ST_NONFINITE = 2, ST_TIMEOUT = 3, ST_COUNT = 4 };
+// (ST_COARSE_RETRY: the merged coarse inverse broke down or failed its check;
+// the host then factors the coarse operator by the banded LU)
+enum { ST_SINGULAR = 0, ST_TANGLED = 1, ST_NONFINITE = 2, ST_TIMEOUT = 3, ST_COARSE_RETRY = 4, ST_COUNT = 5 };
 
 }  // namespace fsi

@@ -506,6 +506,44 @@ void build_coarse_ordering(HostLevel& L) {
     }
   }
   if (!ok) L.slab_off.clear();   // no slab structure: the banded solve is used
+
+  // the same ordering without the Dirichlet unknowns, whose rows are identity
+  // rows, and the padding slots: positions of the free unknowns in it
+  std::vector<int32_t> order_f(L.Ni, -1);
+  for (int64_t i = 0; i < L.Ni; ++i)
+    if (L.canon_of_int[i] >= 0 && !L.dir[i]) order_f[L.coarse_perm[i]] = (int32_t)i;
+  L.free_pos.assign(L.Ni, -1);
+  L.free_map.clear();
+  std::vector<int64_t> before(L.Ni + 1, 0);   // free unknowns before a banded position
+  for (int64_t q = 0; q < L.Ni; ++q) {
+    before[q + 1] = before[q] + (order_f[q] >= 0);
+    if (order_f[q] >= 0) {
+      L.free_pos[order_f[q]] = (int32_t)L.free_map.size();
+      L.free_map.push_back(order_f[q]);
+    }
+  }
+  int64_t fw = 0;
+  for (int64_t b = 0; b < nb; ++b) {
+    const int64_t b0 = before[pos[b] * (int64_t)L.B], b1 = before[(pos[b] + 1) * (int64_t)L.B];
+    for (int32_t k = L.rowptr[b]; k < L.rowptr[b + 1] && b1 > b0; ++k) {
+      const int64_t c0 = before[pos[L.col[k]] * (int64_t)L.B], c1 = before[(pos[L.col[k]] + 1) * (int64_t)L.B];
+      if (c1 > c0) fw = std::max(fw, std::max(b1 - 1 - c0, c1 - 1 - b0));
+    }
+  }
+  L.free_bw = (int)fw;
+  L.free_slab_off.clear();
+  L.free_p = 2;
+  if (!L.slab_off.empty()) {
+    bool same = true;
+    for (int k = 0; k <= K; ++k) L.free_slab_off.push_back(before[L.slab_off[k]]);
+    for (int k = 0; k + 1 < K; ++k) {   // interface planes: all with the same number of free unknowns
+      const int64_t q = L.slab_off[k + 1], p = before[q] - before[q - L.slab_p];
+      if (k == 0) L.free_p = (int)p;
+      same = same && p == L.free_p && p > 0;
+    }
+    for (int k = 0; k < K; ++k) same = same && L.free_slab_off[k + 1] > L.free_slab_off[k];
+    if (!same) L.free_slab_off.clear();
+  }
 }
 
 }  // namespace

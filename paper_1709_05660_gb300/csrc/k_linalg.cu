@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "bounds.cuh"
+#include "fp64_util.cuh"
 #include "kernels.h"
 
 namespace cg = cooperative_groups;
@@ -19,8 +20,6 @@ namespace cg = cooperative_groups;
 namespace fsi {
 
 namespace {
-constexpr int kWarp = 32;
-
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -49,17 +48,6 @@ __device__ double block_sum(double v, double* scratch) {
 // integer (NaN mapped to 0) picks the row a floating-point comparison would,
 // while keeping the comparisons off the FP64 pipe, which on GB300 retires two
 // operations per SM and cycle.
-// a != 0.0 (either sign of zero fails) as an integer test, off the FP64 pipe
-__device__ __forceinline__ bool nonzero(double a) {
-  return ((unsigned long long)__double_as_longlong(a) << 1) != 0ull;
-}
-__device__ __forceinline__ unsigned long long abs_key(double a) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
-  return b > 0x7FF0000000000000ull ? 0ull : b;   // NaN -> 0; +inf stays the largest
-}
-__device__ __forceinline__ bool key_wins(unsigned long long ok, int oi, unsigned long long k, int i) {
-  return (oi >= 0 && i < 0) || (oi >= 0 && (ok > k || (ok == k && oi < i)));
-}
 __device__ int block_argmax_key(unsigned long long v, int idx, unsigned long long* sv, int* si) {
   const int lane = threadIdx.x % kWarp, wid = threadIdx.x / kWarp;
 #pragma unroll
@@ -508,11 +496,33 @@ void launch_nonfinite_check(int64_t n, const double* v, int32_t* status, cudaStr
 // ---------------------------------------------------------------------------
 // coarse level
 // ---------------------------------------------------------------------------
-// Dense coarse operator in the banded ordering, column-major:
-// A[perm[col] * n + perm[row]] (padding slots get 1 on the diagonal).
+// Power-of-two row scales of the coarse operator over an ordering: row maxima
+// (kept columns) to [1, 2).  Momentum, kinematic and mass rows differ by 1e12 in
+// scale, which makes pivot choices by magnitude arbitrary; the exact scaling is
+// undone on the right-hand side of the coarse solve (explicit inverses of the
+// 5 x 4 to 24 x 6 grids: backward error 1e-10 to 1e-7 without, 1e-12 with it).
+__global__ void k_coarse_row_scale(int B, int64_t nb, const int32_t* __restrict__ rowptr,
+                                   const int32_t* __restrict__ col, const double* __restrict__ val,
+                                   const int32_t* __restrict__ perm, int64_t n, double* __restrict__ dr) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nb * B || perm[i] < 0 || !FSI_IN(perm[i], n, FSI_SITE(2))) return;
+  const int64_t br = i / B;
+  const int ci = (int)(i % B);
+  uint32_t top = 0u;   // largest exponent field
+  for (int32_t k = rowptr[br]; k < rowptr[br + 1]; ++k)
+    for (int c = 0; c < B; ++c)
+      if (perm[(int64_t)col[k] * B + c] >= 0)
+        top = max(top, (uint32_t)(abs_key(val[((int64_t)k * B + ci) * B + c]) >> 52));
+  // 2^(1023 - e) for e = 1 .. 2045 as a bit pattern; zero, tiny and non-finite rows keep their scale
+  dr[perm[i]] = top >= 1u && top <= 2045u ? __longlong_as_double((long long)(2046u - top) << 52) : 1.0;
+}
+
+// Dense coarse operator in the banded ordering, rows scaled by dr, column-major:
+// A[perm[col] * n + perm[row]]; unknowns with perm < 0 are left out (padding
+// slots in the list, where they are part of it, get 1 on the diagonal).
 __global__ void k_dense_gather(int B, int64_t nb, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                                const double* __restrict__ val, const int32_t* __restrict__ perm, int64_t n,
-                               double* __restrict__ A) {
+                               const double* __restrict__ dr, double* __restrict__ A) {
   const int64_t br = blockIdx.x;
   if (br >= nb) return;
   const int BB = B * B;
@@ -521,7 +531,7 @@ __global__ void k_dense_gather(int B, int64_t nb, const int32_t* __restrict__ ro
       const int ci = e / B, cj = e % B;
       if (!FSI_IN(col[k], nb, FSI_SITE(2))) continue;
       const int64_t r = perm[br * B + ci], c = perm[(int64_t)col[k] * B + cj];
-      if (FSI_IN(r, n, FSI_SITE(2)) && FSI_IN(c, n, FSI_SITE(2))) A[c * n + r] = val[(int64_t)k * BB + e];
+      if (r >= 0 && c >= 0 && FSI_IN(r, n, FSI_SITE(2)) && FSI_IN(c, n, FSI_SITE(2))) A[c * n + r] = dr[r] * val[(int64_t)k * BB + e];
     }
 }
 
@@ -535,10 +545,11 @@ __global__ void k_set_diag(const int32_t* __restrict__ list, int cnt, const int3
 }
 
 void launch_dense_gather(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
-                         const int32_t* pad_list, int npad, const int32_t* perm, int64_t n, double* A,
+                         const int32_t* pad_list, int npad, const int32_t* perm, int64_t n, double* dr, double* A,
                          cudaStream_t st) {
   cudaMemsetAsync(A, 0, (size_t)n * n * sizeof(double), st);
-  k_dense_gather<<<(unsigned)nb, 64, 0, st>>>(B, nb, rowptr, col, val, perm, n, A);
+  k_coarse_row_scale<<<(unsigned)((nb * B + 127) / 128), 128, 0, st>>>(B, nb, rowptr, col, val, perm, n, dr);
+  k_dense_gather<<<(unsigned)nb, 64, 0, st>>>(B, nb, rowptr, col, val, perm, n, dr, A);
   if (npad > 0) k_set_diag<<<(npad + 255) / 256, 256, 0, st>>>(pad_list, npad, perm, n, A);
 }
 
@@ -923,49 +934,122 @@ int launch_coarse_lu_inverse(int64_t n, int kl, int ku, double* M, double* rdiag
   return 0;
 }
 
-// y = A x with A column-major FP64 (n x n).  Stage 1: block (rb, cb) forms
-// the partial product of rows [256 rb, 256 rb + 256) over the column chunk
-// cb (kGemvChunk columns), one thread per row, coalesced column reads;
-// stage 2 adds the chunk partials in a fixed order.
+// y = A x with A column-major FP64 (n x n) over the unknowns of a coarse
+// ordering: column c reads x[map[c]] (times its row scale dr[c]), row pos[i] gives y[i], and unknowns that
+// the ordering leaves out (pos < 0: identity rows) get y[i] = x[i].  Stage 1:
+// block (rb, cb) forms the partial product of rows [256 rb, 256 rb + 256)
+// over the column chunk cb (kGemvChunk columns), one thread per row, coalesced
+// column reads; stage 2 adds the chunk partials in a fixed order.
 constexpr int kGemvChunk = 32;
 
 template <typename TX>
 __global__ void __launch_bounds__(256) k_gemv_cm_part(int64_t n, const double* __restrict__ A,
+                                                      const int32_t* __restrict__ map, const double* __restrict__ dr,
                                                       const TX* __restrict__ x, double* __restrict__ part) {
+  __shared__ double xs[kGemvChunk];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t c0 = (int64_t)blockIdx.y * kGemvChunk;
   const int64_t c1 = min(n, c0 + kGemvChunk);
+  if (threadIdx.x < c1 - c0) xs[threadIdx.x] = (double)x[map[c0 + threadIdx.x]] * dr[c0 + threadIdx.x];
+  __syncthreads();
   if (i >= n) return;
   double a0 = 0.0, a1 = 0.0;
   int64_t c = c0;
   for (; c + 1 < c1; c += 2) {
-    a0 += A[c * n + i] * (double)x[c];
-    a1 += A[(c + 1) * n + i] * (double)x[c + 1];
+    a0 += A[c * n + i] * xs[c - c0];
+    a1 += A[(c + 1) * n + i] * xs[c + 1 - c0];
   }
-  if (c < c1) a0 += A[c * n + i] * (double)x[c];
+  if (c < c1) a0 += A[c * n + i] * xs[c - c0];
   part[(int64_t)blockIdx.y * n + i] = a0 + a1;
 }
 
-template <typename TY>
-__global__ void k_gemv_cm_sum(int64_t n, int nchunk, const double* __restrict__ part, TY* __restrict__ y) {
+template <typename TX, typename TY>
+__global__ void k_gemv_cm_sum(int64_t ni, int64_t n, int nchunk, const double* __restrict__ part,
+                              const int32_t* __restrict__ pos, const TX* __restrict__ x, TY* __restrict__ y) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= ni) return;
+  const int64_t r = pos[i];
   double s = 0.0;
-  for (int q = 0; q < nchunk; ++q) s += part[(int64_t)q * n + i];
+  if (r < 0) s = (double)x[i];
+  else
+    for (int q = 0; q < nchunk; ++q) s += part[(int64_t)q * n + r];
   y[i] = TY(s);
 }
 
-void launch_gemv(int64_t n, const double* A, const double* x, double* y, double* part, cudaStream_t st) {
+template <typename TX, typename TY>
+void launch_gemv(int64_t ni, int64_t n, const double* A, const int32_t* pos, const int32_t* map, const double* dr,
+                 const TX* x, TY* y, double* part, cudaStream_t st) {
   const int nchunk = (int)((n + kGemvChunk - 1) / kGemvChunk);
-  k_gemv_cm_part<double><<<dim3((unsigned)((n + 255) / 256), nchunk), 256, 0, st>>>(n, A, x, part);
-  k_gemv_cm_sum<double><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, nchunk, part, y);
+  k_gemv_cm_part<TX><<<dim3((unsigned)((n + 255) / 256), nchunk), 256, 0, st>>>(n, A, map, dr, x, part);
+  k_gemv_cm_sum<TX, TY><<<(unsigned)((ni + 255) / 256), 256, 0, st>>>(ni, n, nchunk, part, pos, x, y);
+}
+template void launch_gemv<double, double>(int64_t, int64_t, const double*, const int32_t*, const int32_t*, const double*,
+                                          const double*, double*, double*, cudaStream_t);
+template void launch_gemv<double, float>(int64_t, int64_t, const double*, const int32_t*, const int32_t*, const double*,
+                                         const double*, float*, double*, cudaStream_t);
+template void launch_gemv<float, float>(int64_t, int64_t, const double*, const int32_t*, const int32_t*, const double*, const float*,
+                                        float*, double*, cudaStream_t);
+
+// Right-hand side of the free unknowns: out = b - A[:, D] b_D with D the
+// unknowns that the ordering leaves out; out_D = b_D.
+template <typename TX>
+__global__ void k_coarse_rhs(int B, int64_t nb, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                             const double* __restrict__ val, const int32_t* __restrict__ pos,
+                             const TX* __restrict__ b, double* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nb * B) return;
+  double s = (double)b[i];
+  if (pos[i] >= 0) {
+    const int64_t br = i / B;
+    const int ci = (int)(i % B);
+    for (int32_t k = rowptr[br]; k < rowptr[br + 1]; ++k)
+      for (int c = 0; c < B; ++c) {
+        const int64_t j = (int64_t)col[k] * B + c;
+        if (FSI_IN(j, nb * B, FSI_SITE(2)) && pos[j] < 0) s -= val[((int64_t)k * B + ci) * B + c] * (double)b[j];
+      }
+  }
+  out[i] = s;
 }
 
-void launch_gemv_f32io(int64_t n, const double* A, const float* x, float* y, double* part, cudaStream_t st) {
-  const int nchunk = (int)((n + kGemvChunk - 1) / kGemvChunk);
-  k_gemv_cm_part<float><<<dim3((unsigned)((n + 255) / 256), nchunk), 256, 0, st>>>(n, A, x, part);
-  k_gemv_cm_sum<float><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, nchunk, part, y);
+template <typename TX>
+void launch_coarse_rhs(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
+                       const int32_t* pos, const TX* b, double* out, cudaStream_t st) {
+  k_coarse_rhs<TX><<<(unsigned)((nb * B + 255) / 256), 256, 0, st>>>(B, nb, rowptr, col, val, pos, b, out);
 }
+template void launch_coarse_rhs<double>(int, int64_t, const int32_t*, const int32_t*, const double*, const int32_t*,
+                                        const double*, double*, cudaStream_t);
+template void launch_coarse_rhs<float>(int, int64_t, const int32_t*, const int32_t*, const double*, const int32_t*,
+                                       const float*, double*, cudaStream_t);
+
+// y[i] = x[pos[i]], or b[i] where the ordering leaves i out
+template <typename TB, typename TY>
+__global__ void k_coarse_scatter(int64_t ni, const int32_t* __restrict__ pos, const double* __restrict__ x,
+                                 const TB* __restrict__ b, TY* __restrict__ y) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < ni) y[i] = TY(pos[i] >= 0 ? x[pos[i]] : (double)b[i]);
+}
+template <typename TB>
+__global__ void k_coarse_pick(int64_t n, const int32_t* __restrict__ map, const double* __restrict__ dr,
+                              const TB* __restrict__ b, double* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = (double)b[map[i]] * dr[i];
+}
+template <typename TB, typename TY>
+void launch_coarse_scatter(int64_t ni, const int32_t* pos, const double* x, const TB* b, TY* y, cudaStream_t st) {
+  k_coarse_scatter<TB, TY><<<(unsigned)((ni + 255) / 256), 256, 0, st>>>(ni, pos, x, b, y);
+}
+template <typename TB>
+void launch_coarse_pick(int64_t n, const int32_t* map, const double* dr, const TB* b, double* out, cudaStream_t st) {
+  k_coarse_pick<TB><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, map, dr, b, out);
+}
+template void launch_coarse_scatter<double, double>(int64_t, const int32_t*, const double*, const double*, double*,
+                                                    cudaStream_t);
+template void launch_coarse_scatter<double, float>(int64_t, const int32_t*, const double*, const double*, float*,
+                                                   cudaStream_t);
+template void launch_coarse_scatter<float, float>(int64_t, const int32_t*, const double*, const float*, float*,
+                                                  cudaStream_t);
+template void launch_coarse_pick<double>(int64_t, const int32_t*, const double*, const double*, double*, cudaStream_t);
+template void launch_coarse_pick<float>(int64_t, const int32_t*, const double*, const float*, double*, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // slab-blocked coarse solve (3D): dense FP64 building blocks on column-major

@@ -172,14 +172,48 @@ struct ApplyShape { int kind, slices, vps, groups; };
 ApplyShape apply_shape(int np, int max_nown, int vec_width, int sm_count, int want_slices, int want_groups);
 
 void launch_dense_gather(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
-                         const int32_t* pad_list, int npad, const int32_t* perm, int64_t n, double* A,
+                         const int32_t* pad_list, int npad, const int32_t* perm, int64_t n, double* dr, double* A,
                          cudaStream_t st);
 int launch_coarse_lu_inverse(int64_t n, int kl, int ku, double* M, double* rdiag, double* Ainv, int32_t* piv,
                              const int32_t* perm, const int32_t* pinv, int32_t* status, int sm_count,
                              cudaStream_t st);
-// coarse apply: part holds ceil(n / 32) * n doubles of scratch
-void launch_gemv(int64_t n, const double* A, const double* x, double* y, double* part, cudaStream_t st);
-void launch_gemv_f32io(int64_t n, const double* A, const float* x, float* y, double* part, cudaStream_t st);
+// k_coarse.cu: explicit inverse of the block-tridiagonal 2D coarse operator by
+// merging the inverses of its slab ranges.  off: leaves; merge i joins [a, m)
+// and [m, b), s = size of the first leaf right of m; level[l] .. level[l + 1]
+// are the merges of one level
+constexpr int kMaxLeaves = FSI_MAX_BREAKS + 1;
+struct CoarseMerge { int a, m, b, s; };
+struct CoarseTree {
+  int nleaf, nlev;
+  int off[kMaxLeaves + 1];
+  CoarseMerge merge[kMaxLeaves];
+  int level[9];
+};
+bool coarse_merge_fits(int max_leaf, int p, int max_s);
+// A: the dense operator in the banded ordering (overwritten); Lbuf, Bbuf: n p
+// doubles each; gh: 2 p p doubles per merge of the widest level.  0 or an
+// error; a breakdown raises ST_COARSE_RETRY
+int launch_coarse_merge(const CoarseTree& tr, int64_t n, int p, int max_leaf, int max_s, double* A, double* Lbuf,
+                        double* Bbuf, double* gh, double* Ainv, int32_t* status, int sm_count, cudaStream_t st);
+// test vector on the unknowns with pos >= 0, zero elsewhere
+void launch_coarse_probe(int64_t ni, const int32_t* pos, double* v, cudaStream_t st);
+void launch_coarse_check(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
+                         const double* v, const double* x, double tol, const int32_t* pos, int32_t* status,
+                         cudaStream_t st);
+
+// coarse apply over an ordering of n of the ni unknowns (the others are
+// identity rows), dr its row scales: part holds ceil(n / 32) * n doubles of scratch
+template <typename TX, typename TY>
+void launch_gemv(int64_t ni, int64_t n, const double* A, const int32_t* pos, const int32_t* map, const double* dr,
+                 const TX* x, TY* y, double* part, cudaStream_t st);
+// b less the columns of the unknowns that the ordering leaves out
+template <typename TX>
+void launch_coarse_rhs(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
+                       const int32_t* pos, const TX* b, double* out, cudaStream_t st);
+template <typename TB>
+void launch_coarse_pick(int64_t n, const int32_t* map, const double* dr, const TB* b, double* out, cudaStream_t st);
+template <typename TB, typename TY>
+void launch_coarse_scatter(int64_t ni, const int32_t* pos, const double* x, const TB* b, TY* y, cudaStream_t st);
 // slab-blocked coarse solve: column-major FP64 sub-matrices with leading dimensions
 void launch_dgemm_nn(int m, int n, int k, double alpha, const double* A, int64_t lda, const double* Bm, int64_t ldb,
                      double beta, double* C, int64_t ldc, cudaStream_t st);
