@@ -17,13 +17,13 @@
 #include <type_traits>
 
 #include "bounds.cuh"
+#include "gj_smem.cuh"
 #include "kernels.h"
 #include "tc_util.cuh"
 
 namespace fsi {
 
 namespace {
-constexpr int kWarp = 32;
 
 // Owned inverse rows are stored column-major with the owned count padded to a
 // multiple of 4 (pad rows are zero), so each thread of the apply streams 4
@@ -328,6 +328,56 @@ k_patch_gj_t(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown
   if (threadIdx.x == 0 && s_sing) atomicExch(&status[ST_SINGULAR], 1);
 }
 
+// FP64 blocks of at most kGjSmemMax unknowns: the whole block in shared memory
+// (transposed on the way in: columns contiguous), gj_inverse_smem.  Two thread
+// blocks share an SM up to about 110 unknowns, so one's pivot chain runs beside
+// the other's updates.  GB300, 3-level channel (2 x 2-element blocks of 112
+// unknowns): 3.3 -> 1.58 ms against the sweep that updates every
+// element in every step.
+constexpr int kGjPad = 1;   // column stride n + 1: conflict-free transposed stores
+__global__ void __launch_bounds__(512)
+k_patch_gj_small(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown,
+                 const int64_t* __restrict__ dense_off, const int64_t* __restrict__ own_off,
+                 const int32_t* __restrict__ own, const int64_t* __restrict__ inv_off,
+                 const double* __restrict__ dense, double* __restrict__ invT, int32_t* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ GjStep step;
+  const int p = blockIdx.x;
+  const int n = p_n[p], ld = n + kGjPad;
+  double* M = reinterpret_cast<double*>(smem_raw);
+  double* f = M + (size_t)n * ld;
+  double* rd = f + 2 * n;
+  int* piv = reinterpret_cast<int*>(rd + n);
+  int* qinv = piv + n;
+  uint8_t* isown = reinterpret_cast<uint8_t*>(qinv + n);
+  const int nown = p_nown[p];
+  const int32_t* ow = own + own_off[p];
+  const double* Mg = dense + dense_off[p];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) isown[i] = 0;
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) M[(t % n) * ld + t / n] = Mg[t];
+  __syncthreads();
+  for (int o = threadIdx.x; o < nown; o += blockDim.x)
+    if (FSI_IN(ow[o], n, FSI_SITE(1))) isown[ow[o]] = 1;
+  __syncthreads();
+  const bool ok = gj_inverse_smem(M, n, ld, f, rd, piv, qinv, step, isown);
+  double* out = invT + inv_off[p];
+  const int opad = own_pad(nown);
+  for (int t = threadIdx.x; t < n * opad; t += blockDim.x) {
+    const int c = t / opad, o = t - c * opad;
+    double v = 0.0;
+    if (o < nown && FSI_IN(ow[o], n, FSI_SITE(1))) {
+      const int r = piv[ow[o]];
+      v = rd[r] * M[r + qinv[c] * ld];
+    }
+    out[t] = v;
+  }
+  if (threadIdx.x == 0 && !ok) atomicExch(&status[ST_SINGULAR], 1);
+}
+
+size_t gj_small_smem(int n) {
+  return ((size_t)n * (n + kGjPad) + 3 * n) * sizeof(double) + 2 * (size_t)n * sizeof(int) + n;
+}
+
 // Panel-blocked form of the same in-place Gauss-Jordan sweep.  For a panel of
 // W columns K = [k0, k0+W): (1) the n x W panel G = M[:, K] is swept in shared
 // memory (pivot search and rank-1 updates touch only panel columns); (2) the
@@ -336,110 +386,201 @@ k_patch_gj_t(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown
 // composite transform of the W steps, M[:, rest] += (G - E_P) R[:, rest],
 // with E_P the identity columns at the pivot rows - a rank-W update that reads
 // and writes each block once per panel instead of once per pivot step.
+//
+// In FP64 the pipe bounds it on GB300 (a warp-wide operation every 64 cycles
+// and sub-partition, however many lanes it has), so it issues as few of them as
+// it can: rows stay unscaled until the output (row r holds 1 / rd[r] of its
+// value), the panel is stored by columns so that lanes run over rows, pivot
+// search and zero tests are integer tests, and three kinds of work are left out:
+// rows with no multiplier in the panel, groups of 32 columns that the pivot
+// rows do not reach yet (a block is sparse until its elimination has filled
+// it), and rows of the inverse that the restricted update never reads (the
+// pivot rows of non-owned unknowns).  A 4 x 4-element block (372 unknowns, 304
+// owned) needs 0.52 of n^3 fused multiply-adds, against 0.98.  As in
+// gj_inverse_smem, warp 0 runs one pivot step ahead of the other warps.  Panels of
+// 16 columns leave room for two thread blocks per SM, whose panels and
+// updates overlap.  5-level channel (1,364 blocks): 171 -> 93.8 ms.
+template <typename T>
+__device__ __forceinline__ unsigned long long gj_key(T a) { return abs_key((double)a); }
+template <typename T>
+__device__ __forceinline__ bool gj_nonzero(T a) { return nonzero((double)a); }
+template <>
+__device__ __forceinline__ bool gj_nonzero<float>(float a) { return (__float_as_uint(a) << 1) != 0u; }
+
 template <typename T, int W>
 __global__ void __launch_bounds__(512)
 k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown,
                const int64_t* __restrict__ dense_off, const int64_t* __restrict__ own_off,
                const int32_t* __restrict__ own, const int64_t* __restrict__ inv_off, T* __restrict__ dense,
                T* __restrict__ invT, int32_t* __restrict__ status, int max_n) {
-  constexpr int GS = W + 1;   // padded panel row stride (bank conflicts)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int p = blockIdx.x;
   const int n = p_n[p];
   // regions sized for the largest block of the launch (max_n), so the output
-  // tile (32 x 33, placed in G; the host checks max_n * GS >= 32 * 33) never
+  // tile (32 x 33, placed in G; the host checks max_n * W >= 32 * 33) never
   // overlaps the pivot arrays, whatever this block's n
-  T* G = reinterpret_cast<T*>(smem_raw);              // max_n * GS
-  T* R = G + (size_t)max_n * GS;                      // W * max_n
-  T* pcol = R + (size_t)W * max_n;                    // max_n
-  T* prow = pcol + max_n;                             // W
-  int* piv = reinterpret_cast<int*>(prow + W);        // max_n
+  const int gs = max_n | 1;                           // odd column stride of the panel (bank conflicts)
+  T* G = reinterpret_cast<T*>(smem_raw);              // W * gs, by columns
+  T* R = G + (size_t)W * gs;                          // W * max_n
+  T* f = R + (size_t)W * max_n;                       // 2 * max_n multipliers
+  T* rd = f + 2 * max_n;                              // max_n reciprocal pivots by row
+  int* piv = reinterpret_cast<int*>(rd + max_n);      // max_n
   int* qinv = piv + max_n;                            // max_n
-  uint8_t* used = reinterpret_cast<uint8_t*>(qinv + max_n);   // max_n
-  uint8_t* live = used + max_n;                       // max_n: row touched by this panel
-  __shared__ double sv[32];
-  __shared__ int si[32];
-  __shared__ int s_sing;
+  uint8_t* used = reinterpret_cast<uint8_t*>(qinv + max_n);   // max_n: 1 used, 2 used and not needed any more
+  uint8_t* isown = used + max_n;                      // max_n
+  uint8_t* live = isown + max_n;                      // max_n: row touched by this panel
+  const int nch = (n + kWarp - 1) / kWarp, mch = (max_n + kWarp - 1) / kWarp;
+  uint8_t* fl = live + max_n;                         // 2 * mch: rows 32 u ..: a multiplier is not zero
+  uint8_t* cl = fl + 2 * mch;                         // mch: columns 32 u ..: a pivot-row entry is not zero
+  __shared__ int s_row[2], s_sing;
   T* M = dense + dense_off[p];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) used[i] = 0;
+  const int nown = p_nown[p];
+  const int32_t* ow = own + own_off[p];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) { used[i] = 0; isown[i] = 0; }
   if (threadIdx.x == 0) s_sing = 0;
   __syncthreads();
+  for (int o = threadIdx.x; o < nown; o += blockDim.x)
+    if (FSI_IN(ow[o], n, FSI_SITE(1))) isown[ow[o]] = 1;
   const int lane = threadIdx.x % kWarp, wid = threadIdx.x / kWarp, nw = blockDim.x / kWarp;
-  for (int k0 = 0; k0 < n; k0 += W) {
-    const int wp = min(W, n - k0);
-    for (int i = wid; i < n; i += nw)
-      for (int m = lane; m < W; m += kWarp) G[i * GS + m] = m < wp ? M[(int64_t)i * n + k0 + m] : T(0);
-    __syncthreads();
-    for (int m = 0; m < wp; ++m) {
-      double best = -1.0;
-      int bi = -1;
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        if (used[i]) continue;
-        double a = fabs((double)G[i * GS + m]);
-        if (!(a >= 0.0)) a = 0.0;
-        if (a > best) { best = a; bi = i; }
+  // panel column m: G[r][c] -= f[r] G[pr][c] of one step
+  auto update = [&](int c, int pr, const T* fk, const uint8_t* flk) {
+    T* Gc = G + (size_t)c * gs;
+    const T t = Gc[pr];
+    if (!gj_nonzero(t)) return;
+    for (int u = 0; u < nch; ++u) {
+      if (!flk[u]) continue;
+      const int i = u * kWarp + lane;
+      if (i < n) Gc[i] = Gc[i] - fk[i] * t;
+    }
+  };
+  // warp 0: pivot search of panel column m (largest |a| of the unused rows,
+  // ties to the lowest row) and the multipliers of its step
+  auto prepare = [&](int m, int k) {
+    const T* Gm = G + (size_t)m * gs;
+    T* fk = f + (m & 1) * max_n;
+    unsigned long long best = 0ull;
+    uint32_t row = 0xffffffffu;
+    for (int i = lane; i < n; i += kWarp)
+      if (!used[i]) {
+        const unsigned long long a = gj_key<T>(Gm[i]);
+        if (row == 0xffffffffu || a > best) { best = a; row = i; }
       }
-      const int pr = block_argmax_abs(best, bi, sv, si);
-      for (int i = threadIdx.x; i < n; i += blockDim.x) pcol[i] = G[i * GS + m];
-      if (threadIdx.x < W) prow[threadIdx.x] = G[pr * GS + threadIdx.x];
-      if (threadIdx.x == 0) { used[pr] = 1; piv[k0 + m] = pr; }
-      __syncthreads();
-      T pv = prow[m];
-      if (!(fabs((double)pv) > 0.0) || !isfinite((double)pv)) {
-        if (threadIdx.x == 0) s_sing = 1;
+    const bool has = row != 0xffffffffu;
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, has ? (uint32_t)(best >> 32) : 0u);
+    const bool in = has && (uint32_t)(best >> 32) == hi;
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, in ? (uint32_t)best : 0u);
+    const int pr = (int)__reduce_min_sync(0xffffffffu, in && (uint32_t)best == lo ? row : 0xffffffffu);
+    T rp = T(0);
+    if (lane == 0) {
+      const unsigned long long top = ((unsigned long long)hi << 32) | lo;
+      T pv = Gm[pr];
+      if (top == 0ull || top >= 0x7FF0000000000000ull) {
+        s_sing = 1;
         pv = T(1);
       }
-      const T rp = T(1) / pv;
-      for (int i = wid; i < n; i += nw) {
-        if (lane >= wp) continue;
-        T* Gi = G + i * GS;
-        if (i == pr) {
-          Gi[lane] = (lane == m) ? rp : prow[lane] * rp;
-        } else {
-          const T f = pcol[i] * rp;
-          if (f != T(0)) Gi[lane] = (lane == m) ? -f : Gi[lane] - f * prow[lane];
+      rp = T(1) / pv;
+      rd[pr] = rp;
+      s_row[m & 1] = pr;
+      piv[k] = pr;
+    }
+    rp = __shfl_sync(0xffffffffu, rp, 0);
+    for (int u = 0; u < nch; ++u) {
+      const int i = u * kWarp + lane;
+      T v = T(0);
+      if (i < n && i != pr && used[i] != 2) v = Gm[i];
+      const bool any = __any_sync(0xffffffffu, gj_nonzero(v));
+      if (any) v *= rp;
+      if (i < n) fk[i] = v;
+      if (lane == 0) fl[(m & 1) * mch + u] = any;
+    }
+    __syncwarp();
+    if (lane == 0) used[pr] = isown[k] ? 1 : 2;
+    __syncwarp();
+  };
+  for (int k0 = 0; k0 < n; k0 += W) {
+    const int wp = min(W, n - k0);
+    for (int t = threadIdx.x; t < n * W; t += blockDim.x) {
+      const int i = t / W, m = t % W;
+      if (m < wp) G[m * gs + i] = M[(int64_t)i * n + k0 + m];
+    }
+    __syncthreads();
+    if (wid == 0) prepare(0, k0);
+    for (int m = 0; m < wp; ++m) {
+      __syncthreads();
+      const int pr = s_row[m & 1];
+      const T* fk = f + (m & 1) * max_n;
+      const uint8_t* flk = fl + (m & 1) * mch;
+      if (wid == 0) {
+        if (m + 1 < wp) {
+          update(m + 1, pr, fk, flk);
+          __syncwarp();
+          prepare(m + 1, k0 + m + 1);
+        }
+      } else {
+        // column m itself becomes -f (1 at the pivot row); the rest are updated
+        for (int c = wid - 1; c < wp; c += nw - 1) {
+          if (c == m) {
+            for (int i = lane; i < n; i += kWarp) G[m * gs + i] = i == pr ? T(1) : -fk[i];
+          } else if (c != m + 1) {
+            update(c, pr, fk, flk);
+          }
         }
       }
-      __syncthreads();
     }
-    // old pivot rows, panel write-back, G - E_P, live rows
+    __syncthreads();
+    // old pivot rows, the column groups they reach, panel write-back
     for (int m = wid; m < wp; m += nw) {
       const T* Mp = M + (int64_t)piv[k0 + m] * n;
-      for (int j = lane; j < n; j += kWarp) R[m * n + j] = Mp[j];
+      for (int j = lane; j < n; j += kWarp) R[m * max_n + j] = Mp[j];
     }
-    for (int i = wid; i < n; i += nw)
-      if (lane < wp) M[(int64_t)i * n + k0 + lane] = G[i * GS + lane];
     __syncthreads();
-    if (threadIdx.x < wp) G[piv[k0 + threadIdx.x] * GS + threadIdx.x] -= T(1);
-    __syncthreads();
-    for (int i = wid; i < n; i += nw) {
-      const bool nz = lane < wp && G[i * GS + lane] != T(0);
+    for (int u = wid; u < nch; u += nw) {
+      const int j = u * kWarp + lane;
+      bool nz = false;
+      if (j < n && !(j >= k0 && j < k0 + wp))
+        for (int m = 0; m < wp; ++m) nz |= gj_nonzero(R[m * max_n + j]);
       const unsigned any = __ballot_sync(0xffffffffu, nz);
-      if (lane == 0) live[i] = any != 0u;
+      if (lane == 0) cl[u] = any != 0u;
+    }
+    for (int t = threadIdx.x; t < n * W; t += blockDim.x) {
+      const int i = t / W, m = t % W;
+      if (m < wp) M[(int64_t)i * n + k0 + m] = G[m * gs + i];
+    }
+    __syncthreads();
+    // G - E_P and the rows that it changes
+    if (threadIdx.x < wp) G[threadIdx.x * gs + piv[k0 + threadIdx.x]] -= T(1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      bool nz = false;
+      if (used[i] != 2)
+        for (int m = 0; m < wp; ++m) nz |= gj_nonzero(G[m * gs + i]);
+      live[i] = nz;
     }
     __syncthreads();
     // trailing rank-wp update, 4 rows per warp pass sharing each R load
-    // (the FP64 pipe, not shared memory, bounds this loop on this part)
     for (int g = wid; 4 * g < n; g += nw) {
       const int i0 = 4 * g;
-      bool any = false;
+      bool on[4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) any |= (i0 + r < n) && live[i0 + r];
-      if (!any) continue;
-      for (int j = lane; j < n; j += kWarp) {
-        if (j >= k0 && j < k0 + wp) continue;
+      for (int r = 0; r < 4; ++r) on[r] = i0 + r < n && live[i0 + r];
+      if (!(on[0] || on[1] || on[2] || on[3])) continue;
+      const T* Gr = G + i0;   // entries past row n - 1 are other columns' or R's: their sums are not stored
+      for (int u = 0; u < nch; ++u) {
+        if (!cl[u]) continue;
+        const int j = u * kWarp + lane;
+        if (j >= n || (j >= k0 && j < k0 + wp)) continue;
         T acc[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[r] = T(0);
+        for (int r = 0; r < 4; ++r) acc[r] = on[r] ? M[(int64_t)(i0 + r) * n + j] : T(0);
+#pragma unroll 4
         for (int m = 0; m < wp; ++m) {
-          const T rv = R[m * n + j];
+          const T rv = R[m * max_n + j];
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
-            if (i0 + r < n) acc[r] += G[(i0 + r) * GS + m] * rv;
+          for (int r = 0; r < 4; ++r) acc[r] += Gr[m * gs + r] * rv;
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-          if (i0 + r < n && live[i0 + r]) M[(int64_t)(i0 + r) * n + j] += acc[r];
+          if (on[r]) M[(int64_t)(i0 + r) * n + j] = acc[r];
       }
     }
     __syncthreads();
@@ -449,16 +590,16 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
   __syncthreads();
   // owned rows of the inverse, transposed through a shared tile (reuses G)
   T* tile = G;   // 32 x 33
-  const int nown = p_nown[p];
-  const int32_t* ow = own + own_off[p];
   T* out = invT + inv_off[p];
   for (int o0 = 0; o0 < own_pad(nown); o0 += 32) {
     for (int c0 = 0; c0 < n; c0 += 32) {
       for (int t = threadIdx.x; t < 32 * 32; t += blockDim.x) {
         const int oo = t / 32, cc = t % 32;
         const int o = o0 + oo, c = c0 + cc;
-        if (o < nown && c < n && FSI_IN(ow[o], n, FSI_SITE(1)))
-          tile[oo * 33 + cc] = M[(int64_t)piv[ow[o]] * n + qinv[c]];
+        if (o < nown && c < n && FSI_IN(ow[o], n, FSI_SITE(1))) {
+          const int r = piv[ow[o]];
+          tile[oo * 33 + cc] = rd[r] * M[(int64_t)r * n + qinv[c]];
+        }
       }
       __syncthreads();
       for (int t = threadIdx.x; t < 32 * 32; t += blockDim.x) {
@@ -1093,8 +1234,8 @@ bool launch_patch_gj_tc_levels(const GjLevels& lv, int nblocks, int max_n, int32
 
 template <typename T, int W>
 size_t gj_blk_smem(int n) {
-  return (size_t)n * (W + 1) * sizeof(T) + (size_t)W * n * sizeof(T) + (size_t)n * sizeof(T) + W * sizeof(T) +
-         2 * (size_t)n * sizeof(int) + 2 * (size_t)n + 64;
+  return ((size_t)W * (n | 1) + (size_t)W * n + 3 * (size_t)n) * sizeof(T) + 2 * (size_t)n * sizeof(int) +
+         3 * (size_t)n + 3 * ((size_t)n / kWarp + 1) + 64;
 }
 
 // owned-row vectors of the apply: 4 rows per thread in FP32, 2 in FP64
@@ -1237,7 +1378,7 @@ bool try_gj_blk(int np, int max_n, const int32_t* p_n, const int32_t* p_nown, co
                 const int64_t* own_off, const int32_t* own, const int64_t* inv_off, T* dense, T* invT,
                 int32_t* status, cudaStream_t st) {
   const size_t smem = gj_blk_smem<T, W>(max_n);
-  if (smem > 220 * 1024 || (size_t)32 * 33 > (size_t)max_n * (W + 1)) return false;
+  if (smem > 220 * 1024 || (size_t)32 * 33 > (size_t)max_n * W) return false;
   cudaFuncSetAttribute(k_patch_gj_blk<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_patch_gj_blk<T, W><<<np, 512, smem, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status,
                                                max_n);
@@ -1249,6 +1390,14 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
                        const int64_t* own_off, const int32_t* own, const int64_t* inv_off, T* dense, T* invT,
                        int32_t* status, bool n_mult4, cudaStream_t st) {
   if (np <= 0) return;
+  if (std::is_same<T, double>::value && max_n <= kGjSmemMax) {
+    const size_t smem = gj_small_smem(max_n);
+    cudaFuncSetAttribute(k_patch_gj_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_patch_gj_small<<<np, 512, smem, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off,
+                                            reinterpret_cast<const double*>(dense),
+                                            reinterpret_cast<double*>(invT), status);
+    return;
+  }
   // small blocks: the whole matrix fits in shared memory (unblocked sweep)
   const size_t base = (size_t)max_n * (2 * sizeof(T) + 2 * sizeof(int)) + ((max_n + 15) / 16) * 16;
   const size_t with_m = base + (size_t)max_n * max_n * sizeof(T);
@@ -1270,7 +1419,8 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
     if (try_gj_f32<32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, st)) return;
     if (try_gj_f32<16>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, st)) return;
   }
-  if (try_gj_blk<T, 32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
+  if (std::is_same<T, float>::value &&
+      try_gj_blk<T, 32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
   if (try_gj_blk<T, 16>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
   if (try_gj_blk<T, 8>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
   cudaFuncSetAttribute(k_patch_gj_t<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
