@@ -649,12 +649,10 @@ __device__ __forceinline__ int row_kind3(int cls, int slot) {
 // only through the fields (grad d 9, grad u 9, u 3, d 3, p 1: 25 directions
 // against 166 unknowns).  k_flux_3d evaluates them along the 25 directions in
 // dual arithmetic (27 x 25 = 675 evaluations per element) and stores the
-// derivatives and values of the 22 flux outputs; k_assemble_3d then builds
-// column j of the exact element Jacobian by the chain rule through the basis
-// coefficients of unknown j (its value and three gradient components, or psi
-// for a pressure unknown) and the test functions.  The 166 x 166 element
-// matrix fills shared memory, so the flux derivatives (119 KB per element)
-// pass through a global scratch, one chunk of elements at a time.
+// derivatives and values of the 22 flux outputs; k_assemble_3d contracts them
+// with the trial and test basis to the exact element Jacobian.  The flux
+// derivatives (119 KB per element) pass through a global scratch, one chunk of
+// elements at a time.
 namespace {
 constexpr int k3Q = 27;
 constexpr int k3NF = 25;   // differentiated fields (fv indices 0..24)
@@ -663,8 +661,6 @@ constexpr int k3NO = 22;   // outputs: 0..8 T_ck (3 c + k) | 9..11 convection / 
 constexpr size_t k3FluxDoubles = (size_t)k3Q * k3NF * k3NO + (size_t)k3Q * k3NO;   // per element
 constexpr int k3Chunk = 1024;                                                      // elements per pass
 }  // namespace
-
-size_t assemble_3d_smem() { return ((size_t)k3Ndofe * k3Ndofe + k3Nloc * 4) * sizeof(double); }
 
 size_t assemble_3d_scratch_doubles(int max_ne) {
   return (size_t)std::min(max_ne, k3Chunk) * k3FluxDoubles;
@@ -977,123 +973,268 @@ k_flux_3d(const int32_t* __restrict__ elems, const double* __restrict__ y, const
   if (tangled) atomicExch(&status[ST_TANGLED], 1);
 }
 
-// One thread block per element; thread j < 166 owns column j of the 166 x 166
-// element Jacobian, accumulated in shared memory (no two threads write the
-// same entry), and the value of residual row j.
+// Element matrix from the flux derivatives, one thread block per element, by
+// sum factorisation.  Every momentum entry is a sum over the 27 points of
+// (test kind: value or a gradient component) x coefficient x (trial kind), and
+// the Q2 basis is a product of 1D ones, so the points are contracted one
+// axis at a time (z, y, x), carrying 13, 9 and 4 coefficient combinations: 18.5
+// thousand fused multiply-adds per pair of components instead of the 98
+// thousand of a sum over points for every entry - which is what bounds the
+// kernel, as the FP64 pipe of GB300 retires two per SM and cycle.  One test
+// component at a time with all six trial ones, so that a thread of the last stage
+// holds the six trial components of a node pair and writes them together.
+// The mesh (ALE) rows and the solid kinematic rows have constant coefficients:
+// products of 1D integrals.  908,422-unknown box (16,384 elements), this kernel
+// and the flux derivatives: 155.6 -> 28.6 ms on GB300.
+namespace {
+constexpr int kSfThreads = 256;
+constexpr int kSfPP = 3 * 4 * 3 * 9;              // [axis][kind][point][3 a + b]: products of 1D bases
+constexpr int kSfI = 3 * 4 * 9;                   // their integrals
+constexpr int kSfC = k3Q * 24 * 4;                // [point][field][T_c0..2, body_c]
+constexpr int kSfG = 6 * 9 * 9 * 9;               // [s][3 tx + rx][qx + 3 qy][zp]
+constexpr int kSfH = 6 * 4 * 3 * 81;              // [s][2 tx + rx][qx][9 zp + yp]
+}  // namespace
+
+size_t assemble_3d_smem() { return (size_t)(kSfPP + kSfI + kSfC + kSfG + kSfH) * sizeof(double); }
+
+// cu, cd: coefficients of u and d in the solid kinematic equation
 template <bool SOLID>
-__global__ void __launch_bounds__(192)
+__global__ void __launch_bounds__(kSfThreads, 2)
 k_assemble_3d(const int32_t* __restrict__ elems, const int32_t* __restrict__ elem_nodes,
               const uint8_t* __restrict__ node_class, const double* __restrict__ elem_geo,
-              const double* __restrict__ Dg, double* __restrict__ Ke, double* __restrict__ Re) {
+              const double* __restrict__ Dg, int ale_op, double cu, double cd, double* __restrict__ Ke,
+              double* __restrict__ Re) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* K = reinterpret_cast<double*>(smem_raw);   // [i][j]
-  double* bt = K + k3Ndofe * k3Ndofe;                 // per node: N, Gx, Gy, Gz
-  __shared__ double geo[2 * k3Dim];
+  double* PP = reinterpret_cast<double*>(smem_raw);
+  double* I1 = PP + kSfPP;
+  double* C = I1 + kSfI;
+  double* G = C + kSfC;
+  double* H = G + kSfG;
+  __shared__ double V1[3][3][3][2];   // [axis][point][node]: 1D basis, derivative times 2 / h
   __shared__ unsigned s_iface;
   const int e = elems[blockIdx.x];
-  const int j = threadIdx.x;
-  for (int t = threadIdx.x; t < k3Ndofe * k3Ndofe; t += blockDim.x) K[t] = 0.0;
-  if (threadIdx.x < 2 * k3Dim) geo[threadIdx.x] = elem_geo[(int64_t)e * 2 * k3Dim + threadIdx.x];
-  if (threadIdx.x == 0) {
+  const int tid = threadIdx.x;
+  const double* geo = elem_geo + (int64_t)e * 2 * k3Dim + k3Dim;
+  if (tid < 27) {
+    const int ax = tid / 9, q = (tid / 3) % 3, a = tid % 3;
+    V1[ax][q][a][0] = L1(a, gp(q));
+    V1[ax][q][a][1] = dL1(a, gp(q)) * (2.0 / geo[ax]);
+  }
+  if (tid == 32) {
     unsigned m = 0;
     for (int a = 0; a < k3Nloc; ++a)
       if (node_class[elem_nodes[(int64_t)e * k3Nloc + a]] == kIface) m |= 1u << a;
     s_iface = m;
   }
   __syncthreads();
-  const double hx = geo[3], hy = geo[4], hz = geo[5];
+  // kinds: bit 1 the test (a) side is a derivative, bit 0 the trial (b) side
+  for (int t = tid; t < kSfPP; t += kSfThreads) {
+    const int ab = t % 9, q = (t / 9) % 3, kind = (t / 27) % 4, ax = t / 108;
+    PP[t] = V1[ax][q][ab / 3][kind >> 1] * V1[ax][q][ab % 3][kind & 1];
+  }
+  __syncthreads();
+  for (int t = tid; t < kSfI; t += kSfThreads) {
+    const int ab = t % 9, kind = (t / 9) % 4, ax = t / 36;
+    const double* p = PP + (ax * 4 + kind) * 27 + ab;
+    const double hh = 0.5 * geo[ax];
+    I1[t] = p[0] * (gw(0) * hh) + p[9] * (gw(1) * hh) + p[18] * (gw(2) * hh);
+  }
   const unsigned iface = s_iface;
-  const bool act = j < k3Ndofe;
-  const int aj = (act && j < k3NN) ? j / k3B : -1;
-  const int sj = (act && j < k3NN) ? j % k3B : -1;
-  const int pk = (act && j >= k3NN) ? j - k3NN : -1;
-  // the fields unknown j moves: value and gradient of its component, or p
-  const int ci = sj >= 3 ? sj - 3 : sj;
-  const int f_val = sj < 0 ? 24 : (sj < 3 ? 21 + ci : 18 + ci);
-  const int f_grad = sj < 3 ? 3 * ci : 9 + 3 * ci;
   const double* De = Dg + (size_t)blockIdx.x * k3FluxDoubles;
   const double* Ve = De + (size_t)k3Q * k3NF * k3NO;
-  double vj = 0.0;
-  for (int q = 0; q < k3Q; ++q) {
-    const double xi = gp(q % 3), eta = gp((q / 3) % 3), zeta = gp(q / 9);
-    if (threadIdx.x < k3Nloc) {
-      const int a = threadIdx.x, ia = a % 3, ja = (a / 3) % 3, ka = a / 9;
-      const double lx = L1(ia, xi), ly = L1(ja, eta), lz = L1(ka, zeta);
-      bt[a * 4 + 0] = lx * ly * lz;
-      bt[a * 4 + 1] = dL1(ia, xi) * ly * lz * (2.0 / hx);
-      bt[a * 4 + 2] = lx * dL1(ja, eta) * lz * (2.0 / hy);
-      bt[a * 4 + 3] = lx * ly * dL1(ka, zeta) * (2.0 / hz);
+  double* Kg = Ke + (int64_t)e * k3Ndofe * k3Ndofe;
+  const double *PX = PP, *PY = PP + 108, *PZ = PP + 216;
+
+  for (int c = 0; c < 3; ++c) {
+    for (int t = tid; t < kSfC; t += kSfThreads) {
+      const int o = t % 4, f = (t / 4) % 24, q = t / 96;
+      C[t] = De[((size_t)q * k3NF + f) * k3NO + (o < 3 ? 3 * c + o : 9 + c)];
     }
     __syncthreads();
-    if (act) {
-      const double* dq = De + (size_t)q * k3NF * k3NO;
-      const double* vq = Ve + (size_t)q * k3NO;
-      double dj[k3NO];
-      double nj = 0.0, g0 = 0.0, g1 = 0.0, g2 = 0.0;
-      if (pk < 0) {
-        nj = bt[aj * 4];
-        g0 = bt[aj * 4 + 1];
-        g1 = bt[aj * 4 + 2];
-        g2 = bt[aj * 4 + 3];
-        const double* d0 = dq + f_val * k3NO;
-        const double* d1 = dq + f_grad * k3NO;
-        const double* d2 = d1 + k3NO;
-        const double* d3 = d2 + k3NO;
+    // z: item = (trial component s, point (qx, qy), z pair)
+    for (int t = tid; t < 6 * 81; t += kSfThreads) {
+      const int zp = t % 9, qxy = (t / 9) % 9, s = t / 81;
+      const int fv = s < 3 ? 21 + s : 15 + s, fg = 3 * s;   // value and first gradient field of s
+      double g[9] = {};
 #pragma unroll
-        for (int o = 0; o < k3NO; ++o) dj[o] = d0[o] * nj + d1[o] * g0 + d2[o] * g1 + d3[o] * g2;
-      } else {
-        const double ps = pk == 0 ? 1.0 : (pk == 1 ? xi : (pk == 2 ? eta : zeta));
-        const double* d0 = dq + 24 * k3NO;
-#pragma unroll
-        for (int o = 0; o < k3NO; ++o) dj[o] = d0[o] * ps;
+      for (int qz = 0; qz < 3; ++qz) {
+        const double vv = PZ[qz * 9 + zp], vd = PZ[27 + qz * 9 + zp], dv = PZ[54 + qz * 9 + zp],
+                     dd = PZ[81 + qz * 9 + zp];
+        const double* cq = C + (size_t)(qxy + 9 * qz) * 96;
+        const double *cx = cq + fg * 4, *cy = cx + 4, *cz = cx + 8, *c0 = cq + fv * 4;
+        g[0] = fma(cx[0], vv, g[0]);
+        g[1] = fma(cy[0], vv, g[1]);
+        g[2] = fma(cz[0], vd, g[2]);
+        g[3] = fma(cx[1], vv, g[3]);
+        g[4] = fma(cy[1], vv, g[4]);
+        g[5] = fma(cz[1], vd, g[5]);
+        g[6] = fma(cx[2], dv, fma(cx[3], vv, g[6]));
+        g[7] = fma(cy[2], dv, fma(cy[3], vv, g[7]));
+        g[8] = fma(cz[2], dd, fma(cz[3], vd, fma(c0[3], vv, g[8])));
       }
-      for (int a = 0; a < k3Nloc; ++a) {
-        const double Na = bt[a * 4], G0 = bt[a * 4 + 1], G1 = bt[a * 4 + 2], G2 = bt[a * 4 + 3];
-        const bool ifc = (iface >> a) & 1u;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const double md = dj[3 * c] * G0 + dj[3 * c + 1] * G1 + dj[3 * c + 2] * G2 + dj[9 + c] * Na;
-          const int rd = a * k3B + c, ru = a * k3B + 3 + c;
-          if (SOLID) {
-            K[rd * k3Ndofe + j] += md;
-            K[ru * k3Ndofe + j] += dj[12 + c] * Na;
-          } else if (ifc) {
-            // interface node: momentum in the d-row, no ALE row (psi = 0 on the interface)
-            K[rd * k3Ndofe + j] += md;
-          } else {
-            // fluid node: ALE in the d-row, momentum in the u-row
-            K[rd * k3Ndofe + j] += dj[12 + 3 * c] * G0 + dj[13 + 3 * c] * G1 + dj[14 + 3 * c] * G2;
-            K[ru * k3Ndofe + j] += md;
-          }
+      for (int k = 0; k < 9; ++k) G[((s * 9 + k) * 9 + qxy) * 9 + zp] = g[k];
+    }
+    __syncthreads();
+    // y: item = (s, qx, z pair, y pair)
+    for (int t = tid; t < 6 * 3 * 81; t += kSfThreads) {
+      const int zy = t % 81, yp = zy % 9, zp = zy / 9, qx = (t / 81) % 3, s = t / 243;
+      double h[4] = {};
+#pragma unroll
+      for (int qy = 0; qy < 3; ++qy) {
+        const double vv = PY[qy * 9 + yp], vd = PY[27 + qy * 9 + yp], dv = PY[54 + qy * 9 + yp],
+                     dd = PY[81 + qy * 9 + yp];
+        const double* gq = G + ((size_t)s * 81 + qx + 3 * qy) * 9 + zp;   // + 81 k: combination k
+        h[0] = fma(gq[0], vv, h[0]);
+        h[1] = fma(gq[81], vd, fma(gq[162], vv, h[1]));
+        h[2] = fma(gq[243], dv, fma(gq[486], vv, h[2]));
+        h[3] = fma(gq[324], dd, fma(gq[405], dv, fma(gq[567], vd, fma(gq[648], vv, h[3]))));
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) H[((s * 4 + k) * 3 + qx) * 81 + zy] = h[k];
+    }
+    __syncthreads();
+    // x: item = (z pair, y pair, x pair) = node pair (a, b)
+    for (int t = tid; t < 729; t += kSfThreads) {
+      const int xp = t % 9, zy = t / 9, yp = zy % 9, zp = zy / 9;
+      const int a = xp / 3 + 3 * (yp / 3) + 9 * (zp / 3), b = xp % 3 + 3 * (yp % 3) + 9 * (zp % 3);
+      double k[6] = {};
+#pragma unroll
+      for (int qx = 0; qx < 3; ++qx) {
+        const double vv = PX[qx * 9 + xp], vd = PX[27 + qx * 9 + xp], dv = PX[54 + qx * 9 + xp],
+                     dd = PX[81 + qx * 9 + xp];
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+          const double* hq = H + (s * 12 + qx) * 81 + zy;   // + 243 k: combination k
+          k[s] = fma(hq[0], dd, fma(hq[243], dv, fma(hq[486], vd, fma(hq[729], vv, k[s]))));
         }
       }
-      K[k3NN * k3Ndofe + j] += dj[21];
-      K[(k3NN + 1) * k3Ndofe + j] += dj[21] * xi;
-      K[(k3NN + 2) * k3Ndofe + j] += dj[21] * eta;
-      K[(k3NN + 3) * k3Ndofe + j] += dj[21] * zeta;
-      // residual row j from the flux values
-      if (pk < 0) {
-        const bool ifc = (iface >> aj) & 1u;
+      const bool ifc = (iface >> a) & 1u;
+      // momentum sits in the d-row of solid and interface nodes, in the u-row of fluid ones
+      double2* mrow = reinterpret_cast<double2*>(Kg + (a * k3B + (SOLID || ifc ? 0 : 3) + c) * k3Ndofe + b * k3B);
+      mrow[0] = make_double2(k[0], k[1]);
+      mrow[1] = make_double2(k[2], k[3]);
+      mrow[2] = make_double2(k[4], k[5]);
+      // the node's other row: kinematic (solid), nothing (interface), ALE (fluid)
+      const double *ix = I1 + xp, *iy = I1 + 36 + yp, *iz = I1 + 72 + zp;   // + 9 kind
+      double r[6] = {};
+      if (SOLID) {
+        const double m = ix[0] * iy[0] * iz[0];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {   // unrolled select: no dynamic register-array index
-          const double mv = vq[3 * c] * g0 + vq[3 * c + 1] * g1 + vq[3 * c + 2] * g2 + vq[9 + c] * nj;
-          if (SOLID) {
-            if (sj == c) vj += mv;
-            if (sj == 3 + c) vj += vq[12 + c] * nj;
-          } else {
-            if (sj == c) vj += ifc ? mv : vq[12 + 3 * c] * g0 + vq[13 + 3 * c] * g1 + vq[14 + 3 * c] * g2;
-            if (sj == 3 + c && !ifc) vj += mv;
-          }
+        for (int s = 0; s < 3; ++s) {
+          r[s] = s == c ? m * cd : 0.0;
+          r[3 + s] = s == c ? m * cu : 0.0;
         }
-      } else {
-        vj += vq[21] * (pk == 0 ? 1.0 : (pk == 1 ? xi : (pk == 2 ? eta : zeta)));
+      } else if (!ifc) {
+        const double kale = 1.0 / (geo[0] * geo[1] * geo[2]);
+        const double lap = ix[27] * iy[0] * iz[0] + ix[0] * iy[27] * iz[0] + ix[0] * iy[0] * iz[27];
+        // the transposed term: test derivative along s, trial derivative along c
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          double v = s == c ? lap : 0.0;
+          if (ale_op == 0) {
+            const int k0 = (s == 0 ? 2 : 0) + (c == 0 ? 1 : 0), k1 = (s == 1 ? 2 : 0) + (c == 1 ? 1 : 0),
+                      k2 = (s == 2 ? 2 : 0) + (c == 2 ? 1 : 0);
+            v += ix[9 * k0] * iy[9 * k1] * iz[9 * k2];
+          }
+          r[s] = v * kale;
+        }
       }
+      double2* orow = reinterpret_cast<double2*>(Kg + (a * k3B + (SOLID || ifc ? 3 : 0) + c) * k3Ndofe + b * k3B);
+      orow[0] = make_double2(r[0], r[1]);
+      orow[1] = make_double2(r[2], r[3]);
+      orow[2] = make_double2(r[4], r[5]);
     }
     __syncthreads();
   }
-  double* Kg = Ke + (int64_t)e * k3Ndofe * k3Ndofe;
-  for (int t = threadIdx.x; t < k3Ndofe * k3Ndofe; t += blockDim.x) Kg[t] = K[t];
-  if (act) Re[(int64_t)e * k3Ndofe + j] = vj;
+  // pressure rows and columns and the residual, point by point with the nine
+  // points of a z layer per item; partial sums of the layers added afterwards
+  double* bt = G;   // [point][node]: N, d/dx, d/dy, d/dz
+  for (int t = tid; t < k3Q * k3Nloc; t += kSfThreads) {
+    const int q = t / k3Nloc, a = t % k3Nloc;
+    const double *x = V1[0][q % 3][a % 3], *y = V1[1][(q / 3) % 3][(a / 3) % 3], *z = V1[2][q / 9][a / 9];
+    const double yz = y[0] * z[0];
+    bt[t * 4] = x[0] * yz;
+    bt[t * 4 + 1] = x[1] * yz;
+    bt[t * 4 + 2] = x[0] * y[1] * z[0];
+    bt[t * 4 + 3] = x[0] * y[0] * z[1];
+  }
+  __syncthreads();
+  double *pc = H, *pr = pc + 243 * 4, *rs = pr + 486 * 4;   // partial sums: pressure columns, rows, residual
+  for (int t = tid; t < 243 + 486 + 486 + 12; t += kSfThreads) {
+    if (t < 243) {
+      const int ac = t % 81, a = ac / 3, c = ac % 3, qz = t / 81;
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      for (int q = 9 * qz; q < 9 * qz + 9; ++q) {
+        const double* d = De + ((size_t)q * k3NF + 24) * k3NO + 3 * c;
+        const double* w = bt + (q * k3Nloc + a) * 4;
+        const double v = d[0] * w[1] + d[1] * w[2] + d[2] * w[3];
+        s0 += v;
+        s1 = fma(v, gp(q % 3), s1);
+        s2 = fma(v, gp((q / 3) % 3), s2);
+      }
+      pc[t * 4] = s0;
+      pc[t * 4 + 1] = s1;
+      pc[t * 4 + 2] = s2;
+      pc[t * 4 + 3] = s0 * gp(qz);
+    } else if (t < 729) {
+      const int u = t - 243, bs = u % 162, b = bs / 6, s = bs % 6, qz = u / 162;
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+      for (int q = 9 * qz; q < 9 * qz + 9; ++q) {
+        const double* d = De + ((size_t)q * k3NF + 3 * s) * k3NO + 21;
+        const double* w = bt + (q * k3Nloc + b) * 4;
+        const double v = d[0] * w[1] + d[k3NO] * w[2] + d[2 * k3NO] * w[3];
+        s0 += v;
+        s1 = fma(v, gp(q % 3), s1);
+        s2 = fma(v, gp((q / 3) % 3), s2);
+      }
+      pr[u * 4] = s0;
+      pr[u * 4 + 1] = s1;
+      pr[u * 4 + 2] = s2;
+      pr[u * 4 + 3] = s0 * gp(qz);
+    } else if (t < 1215) {
+      const int u = t - 729, j = u % 162, a = j / 6, s = j % 6, c = s % 3, qz = u / 162;
+      const bool ifc = (iface >> a) & 1u;
+      // momentum (outputs 3 c .. with body 9 + c), ALE (12 + 3 c ..), kinematic (12 + c) or no row
+      const bool mom = SOLID || ifc ? s < 3 : s >= 3;
+      const int og = mom ? 3 * c : (!SOLID && !ifc ? 12 + 3 * c : -1);
+      const int ov = mom ? 9 + c : (SOLID ? 12 + c : -1);
+      double v = 0.0;
+      for (int q = 9 * qz; q < 9 * qz + 9; ++q) {
+        const double* d = Ve + (size_t)q * k3NO;
+        const double* w = bt + (q * k3Nloc + a) * 4;
+        if (og >= 0) v += d[og] * w[1] + d[og + 1] * w[2] + d[og + 2] * w[3];
+        if (ov >= 0) v = fma(d[ov], w[0], v);
+      }
+      rs[u] = v;
+    } else {
+      const int u = t - 1215, pk = u % 4, qz = u / 4;
+      double v = 0.0;
+      for (int q = 9 * qz; q < 9 * qz + 9; ++q)
+        v += Ve[(size_t)q * k3NO + 21] * (pk == 0 ? 1.0 : (pk == 1 ? gp(q % 3) : (pk == 2 ? gp((q / 3) % 3) : gp(qz))));
+      rs[486 + u] = v;
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < 324 + 648 + 166 + 16; t += kSfThreads) {
+    if (t < 324) {
+      const int pk = t % 4, ac = t / 4, a = ac / 3, c = ac % 3;
+      const double v = pc[ac * 4 + pk] + pc[(81 + ac) * 4 + pk] + pc[(162 + ac) * 4 + pk];
+      const int m = SOLID || ((iface >> a) & 1u) ? 0 : 3;
+      Kg[(a * k3B + m + c) * k3Ndofe + k3NN + pk] = v;
+      Kg[(a * k3B + 3 - m + c) * k3Ndofe + k3NN + pk] = 0.0;
+    } else if (t < 972) {
+      const int u = t - 324, bs = u % 162, pk = u / 162;
+      Kg[(k3NN + pk) * k3Ndofe + bs] = pr[bs * 4 + pk] + pr[(162 + bs) * 4 + pk] + pr[(324 + bs) * 4 + pk];
+    } else if (t < 1138) {
+      const int j = t - 972;
+      Re[(int64_t)e * k3Ndofe + j] = j < k3NN ? rs[j] + rs[162 + j] + rs[324 + j]
+                                              : rs[486 + j - k3NN] + rs[490 + j - k3NN] + rs[494 + j - k3NN];
+    } else {
+      const int u = t - 1138;
+      Kg[(k3NN + u / 4) * k3Ndofe + k3NN + u % 4] = 0.0;
+    }
+  }
 }
 
 // Element-wise Galerkin coarsening in 3D.  Per child: T = A_c P_c is formed
@@ -1346,12 +1487,16 @@ bool launch_assemble_3d(bool solid, const int32_t* elems, int ne, const double* 
   if (ne <= 0) return true;
   if (std::min(ne, k3Chunk) > scratch_ne) return false;   // the flux scratch holds scratch_ne elements
   const size_t smem = assemble_3d_smem();
+  // solid kinematic equation: u, u - (a0 d + history) / dt, (u + u_n) / 2 - (d - d_n) / dt
+  const double cu = pp.transient == 2 ? 0.5 : 1.0;
+  const double cd = pp.transient == 2 ? -pp.idt : (pp.transient ? -pp.a0 * pp.idt : 0.0);
   auto go = [&](auto flux, auto cols) {
     cudaFuncSetAttribute(cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     for (int e0 = 0; e0 < ne; e0 += k3Chunk) {
       const int nc = std::min(k3Chunk, ne - e0);
       flux<<<nc, 256, 0, st>>>(elems + e0, y, elem_nodes, elem_geo, n_nodes, pp, scratch, status);
-      cols<<<nc, 192, smem, st>>>(elems + e0, elem_nodes, node_class, elem_geo, scratch, Ke, Re);
+      cols<<<nc, kSfThreads, smem, st>>>(elems + e0, elem_nodes, node_class, elem_geo, scratch, pp.ale_op, cu, cd, Ke,
+                                         Re);
     }
   };
   if (solid) {
