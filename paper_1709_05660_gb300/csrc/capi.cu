@@ -437,7 +437,8 @@ void build_device(Ctx& c) {
       o.slab = c.dim == 3 && !o.slab_off.empty();
       if (o.slab) slab_sizes(o);
     }
-    if (fr.slab != all.slab) fr = all;
+    const bool same = fr.slab != all.slab;   // no slabs of equal planes among the free unknowns
+    if (same) fr = all;
     if (c.dim == 2) fr.tree = make_tree(H0, &fr.tree_leaf, &fr.tree_s);
     if (fr.tree) {
       c.c_L = dalloc<double>(c, (size_t)fr.n * fr.p);
@@ -457,6 +458,18 @@ void build_device(Ctx& c) {
       c.c_xb = dalloc<double>(c, n0);
       c.c_tp = dalloc<double>(c, all.p);
       c.c_part = dalloc<double>(c, (size_t)((mm + 31) / 32) * mm);
+      fr.twoway = fr.slab && !same && slab_gj_fits(fr.mmax, c.sm_count);
+      if (fr.twoway) {
+        const size_t m2 = fr.mmax;
+        c.s_S = dalloc<double>(c, 2 * m2 * m2);
+        c.s_T = dalloc<double>(c, 2 * slab_gj_scratch(fr.mmax));
+        c.s_Q = dalloc<double>(c, 2 * m2 * fr.p);
+        c.s_rd = dalloc<double>(c, 2 * m2);
+        c.s_u = dalloc<double>(c, 2 * m2);
+        c.s_piv = dalloc<int32_t>(c, 2 * m2);
+        c.s_flag = dalloc<int32_t>(c, 2 * (size_t)slab_gj_panels(fr.mmax));
+        ck(cudaMemsetAsync(c.s_flag, 0, 2 * (size_t)slab_gj_panels(fr.mmax) * sizeof(int32_t), c.stream), "memset");
+      }
     }
   }
   c.status = dalloc<int32_t>(c, ST_COUNT);
@@ -638,6 +651,92 @@ void coarse_factor_slab(Ctx& c) {
   }
 }
 
+// The same elimination from both ends of the chain to its middle slab (k_slab.cu).
+SlabChain slab_chain(const CoarseOrder& co) {
+  SlabChain ch{};
+  ch.K = (int)co.slab_off.size() - 1;
+  ch.mid = ch.K / 2;
+  ch.p = co.p;
+  ch.mmax = co.mmax;
+  for (int k = 0; k <= ch.K; ++k) {
+    ch.off[k] = (int)co.slab_off[k];
+    if (k < ch.K) ch.inv[k] = co.sinv_off[k];
+  }
+  return ch;
+}
+
+void coarse_factor_twoway(Ctx& c) {
+  const CoarseOrder& co = c.ord();
+  const SlabChain ch = slab_chain(co);
+  const int64_t n0 = co.n;
+  const int p = co.p, K = ch.K;
+  double flops = 0.0, bytes = (double)n0 * n0 * 8.0;
+  for (int k = 0; k < K; ++k) {
+    const double m = (double)(ch.off[k + 1] - ch.off[k]);
+    flops += 2.0 * m * m * m + (k < ch.mid ? 2.0 * p * p * m + 2.0 * m * p * m : 0.0) +
+             (k > ch.mid ? 2.0 * m * m * p + 2.0 * p * p * m : 0.0);
+    bytes += 3.0 * m * m * 8.0;
+  }
+  const int steps = std::max(ch.mid, K - 1 - ch.mid) + 1;
+  Prof pr(c, FSI_K_COARSE_FACTOR, bytes, flops, 2 + 5 * steps);
+  coarse_gather(c);
+  for (int s = 0; s < steps; ++s) {
+    // step s: slab s from the left, slab K - 1 - s from the right; the middle one last, from both
+    const bool last = s + 1 == steps;
+    int slab[2], n = 0;
+    if (last) {
+      slab[n++] = ch.mid;
+    } else {
+      if (s < ch.mid) slab[n++] = s;
+      if (K - 1 - s > ch.mid) slab[n++] = K - 1 - s;
+    }
+    SlabJobs jobs{};
+    SlabGemm one[2], two[2];
+    int ng = 0;
+    for (int i = 0; i < n; ++i) {
+      const int k = slab[i];
+      const int64_t o = ch.off[k];
+      const int m = ch.off[k + 1] - ch.off[k];
+      double* S = c.s_S + (size_t)i * co.mmax * co.mmax;
+      launch_copy2d(m, m, c.c_A + o * n0 + o, n0, S, m, c.stream);
+      counted(c);
+      auto left = [&] {    // S -= A_{k,k-1}[:,P] (S_{k-1}^{-1}[P,P] A_{k-1,k}[P,:])
+        const int mp = (int)(o - ch.off[k - 1]);
+        const double* X = c.c_sinv + ch.inv[k - 1];
+        double* Q = c.s_Q + (size_t)ng * co.mmax * p;
+        one[ng] = SlabGemm{p, m, p, 1.0, 0.0, X + (int64_t)(mp - p) * mp + (mp - p), mp, c.c_A + o * n0 + (o - p), n0, Q, p};
+        two[ng++] = SlabGemm{m, m, p, -1.0, 1.0, c.c_A + (o - p) * n0 + o, n0, Q, p, S, m};
+      };
+      auto right = [&] {   // S[P,P] -= A_{k,k+1}[P,:] (S_{k+1}^{-1} A_{k+1,k}[:,P])
+        const int64_t on = ch.off[k + 1];
+        const int mn = (int)(ch.off[k + 2] - on);
+        double* Q = c.s_Q + (size_t)ng * co.mmax * p;
+        one[ng] = SlabGemm{mn, p, mn, 1.0, 0.0, c.c_sinv + ch.inv[k + 1], mn, c.c_A + (on - p) * n0 + on, n0, Q, mn};
+        two[ng++] = SlabGemm{p, p, mn, -1.0, 1.0, c.c_A + on * n0 + (on - p), n0, Q, mn,
+                             S + (int64_t)(m - p) * m + (m - p), m};
+      };
+      if (k <= ch.mid && k > 0) left();
+      if (k >= ch.mid && k + 1 < K) right();
+      jobs.j[jobs.n++] = SlabJob{S, c.s_T + (size_t)i * slab_gj_scratch(co.mmax), c.c_sinv + ch.inv[k], m,
+                                 c.s_piv + (size_t)i * co.mmax, c.s_rd + (size_t)i * co.mmax,
+                                 c.s_flag + (size_t)i * slab_gj_panels(co.mmax)};
+    }
+    if (ng > 0) {
+      launch_slab_gemm(one, ng, c.stream);
+      if (last && ng == 2) {   // both corrections of the middle slab add to its plane P
+        launch_slab_gemm(two, 1, c.stream);
+        launch_slab_gemm(two + 1, 1, c.stream);
+      } else {
+        launch_slab_gemm(two, ng, c.stream);
+      }
+      counted(c, last && ng == 2 ? 3 : 2);
+    }
+    const int rc = launch_slab_gj(jobs, ++c.s_epoch, c.status, c.sm_count, c.stream);
+    if (rc != 0) throw ApiError(FSI_E_CUDA, "slab inverse launch failed (" + std::to_string(rc) + ")");
+    counted(c);
+  }
+}
+
 // x = A_0^{-1} b over the ordering (FP64, b in c_zb, x in c_xb): forward block
 // elimination w_k = b_k - A_{k,k-1}[:,P] (S_{k-1}^{-1}[P,:] w_{k-1}), then back
 // substitution x_k = S_k^{-1} (w_k - A_{k,k+1} x_{k+1}) with A_{k,k+1}
@@ -699,7 +798,13 @@ void coarse_solve(Ctx& c, const TB* b, TB* x, double* part) {
     if (shift) launch_coarse_pick<double>(o.n, o.map, c.c_dr, c.c_rhs, c.c_zb, c.stream);
     else launch_coarse_pick<TB>(o.n, o.map, c.c_dr, b, c.c_zb, c.stream);
     counted(c);
-    coarse_apply_slab(c);
+    if (o.twoway) {
+      if (launch_slab_solve(slab_chain(o), c.c_A, o.n, c.c_sinv, c.c_zb, c.c_xb, c.s_u, c.sm_count, c.stream) != 0)
+        throw ApiError(FSI_E_CUDA, "slab solve launch failed");
+      counted(c);
+    } else {
+      coarse_apply_slab(c);
+    }
     launch_coarse_scatter<TB, TB>(C.Ni, o.pos, c.c_xb, b, x, c.stream);
     counted(c);
   } else {
@@ -875,7 +980,8 @@ void coarse_factor(Ctx& c) {
   }
   const CoarseOrder& o = c.ord();
   if (o.slab) {
-    coarse_factor_slab(c);
+    if (o.twoway) coarse_factor_twoway(c);
+    else coarse_factor_slab(c);
   } else if (o.tree) {
     double flops = 0.0;
     const CoarseTree& t = *o.tree;
@@ -971,7 +1077,7 @@ void coarse_grid(Ctx& c, const T* b, T* x) {
   const CoarseOrder& o = c.ord();
   const double n = (double)o.n, io = 2.0 * (double)c.dl[0].Ni * sizeof(T);
   const double by = o.slab ? coarse_slab_apply_bytes(c) : n * n * 8.0;
-  Prof pr(c, FSI_K_TRANSFER, by + io, by / 4.0, o.slab ? 2 + 8 * ((int)o.slab_off.size() - 1) : 2);
+  Prof pr(c, FSI_K_TRANSFER, by + io, by / 4.0, o.twoway ? 3 : (o.slab ? 2 + 8 * ((int)o.slab_off.size() - 1) : 2));
   coarse_solve<T>(c, b, x, c.c_part);
 }
 
@@ -1502,6 +1608,10 @@ static int64_t estimate_device_bytes(const Ctx& c) {
       sum += m * m;
     }
     b += n0 * n0 * 8.0 + (sum + mm * mm + H0.slab_p * mm + mm * mm / 32.0 + mm) * 8.0 + 6.0 * n0 * 8.0;
+    double fm = 0.0;   // elimination from both ends: two slabs' complements, transforms, products, vectors
+    for (size_t k = 0; k + 1 < H0.free_slab_off.size(); ++k)
+      fm = std::max(fm, (double)(H0.free_slab_off[k + 1] - H0.free_slab_off[k]));
+    if (fm <= 1024.0) b += (4.0 * fm * fm + 2.0 * H0.free_p * fm + 16.0 * fm) * 8.0;
   } else {
     b += 2.0 * n0 * n0 * 8.0 + (n0 / 32.0 + 1.0) * n0 * 8.0 + 2.0 * n0 * 8.0;
     int leaf = 0, s = 0;

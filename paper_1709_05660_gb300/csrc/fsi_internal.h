@@ -168,6 +168,7 @@ struct CoarseOrder {
   int bw = 0, p = 0, mmax = 0;              // half-bandwidth, interface plane, largest slab
   std::vector<int64_t> slab_off, sinv_off;
   bool slab = false;                        // slab-blocked LU (3D)
+  bool twoway = false;                      // eliminated from both ends (k_slab.cu)
   std::shared_ptr<CoarseTree> tree;         // merged inverse (2D, slabs small enough)
   int tree_leaf = 0, tree_s = 0;            // largest leaf; largest first leaf of a right part
 };
@@ -227,6 +228,10 @@ struct Ctx {
   // slab-blocked coarse solve (3D): Sinv_k blocks, LU scratch, vectors
   double *c_sinv = nullptr, *c_S = nullptr, *c_T = nullptr, *c_zb = nullptr, *c_xb = nullptr, *c_tp = nullptr;
   int32_t* c_iota = nullptr;
+  // the same from both ends: complements, panel transforms, products, pivots, flags, solve scratch of two slabs
+  double *s_S = nullptr, *s_T = nullptr, *s_Q = nullptr, *s_rd = nullptr, *s_u = nullptr;
+  int32_t *s_piv = nullptr, *s_flag = nullptr;
+  int s_epoch = 0;
   float t_assemble = 0.f, t_factor = 0.f, t_solve = 0.f;
   int red_blocks = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;

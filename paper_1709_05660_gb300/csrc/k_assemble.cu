@@ -32,13 +32,8 @@ __device__ __forceinline__ Dual operator-(Dual a) { return {-a.v, -a.d}; }
 __device__ __forceinline__ Dual operator*(Dual a, Dual b) { return {a.v * b.v, a.d * b.v + a.v * b.d}; }
 __device__ __forceinline__ Dual operator*(Dual a, double s) { return {a.v * s, a.d * s}; }
 __device__ __forceinline__ Dual operator+(Dual a, double s) { return {a.v + s, a.d}; }
-__device__ __forceinline__ Dual operator/(Dual a, Dual b) {
-  const double inv = 1.0 / b.v;
-  const double q = a.v * inv;
-  return {q, (a.d - b.d * q) * inv};
-}
-// a / b given inv = 1 / b.v (the same arithmetic as operator/, with the one
-// reciprocal shared by several quotients of the same divisor)
+// a / b given inv = 1 / b.v (one reciprocal shared by several quotients of the
+// same divisor)
 __device__ __forceinline__ Dual div_inv(Dual a, Dual b, double inv) {
   const double q = a.v * inv;
   return {q, (a.d - b.d * q) * inv};

@@ -1,0 +1,510 @@
+// Slab-blocked coarse solve in 3D from both ends (Sec. 3, 4.1): the coarse
+// operator is block tridiagonal over x-slabs, and slabs k - 1 and k couple
+// through the last node plane P of slab k - 1 only.  Block elimination runs from
+// the first slab to the middle one and from the last slab to the middle one at
+// the same time,
+//     left   S_k = A_kk - A_{k,k-1}[:,P] (S_{k-1}^{-1}[P,P] A_{k-1,k}[P,:]),
+//     right  S_k = A_kk - E_P (A_{k,k+1}[P,:] S_{k+1}^{-1} A_{k+1,k}[:,P]) E_P^T,
+// which halves the chain of dependent slab inverses; the middle slab takes both
+// corrections.  The slab complements are inverted by Gauss-Jordan with
+// partial pivoting, spread over half of the SMs per side (k_slab_gj), and the
+// solve (k_slab_solve) is one launch.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "bounds.cuh"
+#include "fp64_util.cuh"
+#include "kernels.h"
+
+namespace cg = cooperative_groups;
+
+namespace fsi {
+
+namespace {
+constexpr int kSlabThreads = 512;
+constexpr int kSlabRows = 2;                 // rows per thread: slabs of at most 1,024 unknowns
+constexpr int kSlabW = 4;                    // panel width
+constexpr int kSlabWarps = kSlabThreads / kWarp;
+constexpr long long kSlabWait = 1LL << 21;   // iteration limit of a wait for a panel
+
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(int* p, int v) {
+  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+}  // namespace
+
+// In-place Gauss-Jordan inverses of up to two m x m matrices (S, column-major),
+// `ng` thread blocks each.  Panels of kSlabW columns are dealt to the blocks in
+// turn and stay in shared memory.  The owner of panel k factors it and
+// publishes the composite transform T_k = G - E_P of its steps (m x kSlabW) and
+// its pivot rows; every block applies T_0, T_1, ... to its panels as they are
+// published, the next owner to its own next panel first, so that it factors
+// panel k + 1 while the others still apply T_k.  Rows stay unscaled (as in
+// gj_inverse_smem).
+//
+// The chain of one block's panel work bounds it: per panel kSlabW pivot steps
+// over m rows and the transform of the previous panel, both on one SM's FP64 pipe
+// (two fused multiply-adds per cycle), and the hand-over.  Their cost per column
+// is m (kSlabW + kSlabW) / 2 cycles plus (hand-over) / kSlabW, hence narrow
+// panels: 4 columns.  Nine rounds of two slabs of 652
+// unknowns with their products: 28.4 ms against 88 one after the other by the
+// banded LU kernels.
+//
+// The launch is cooperative (all blocks resident), the waits are bounded: a
+// block whose wait runs out raises ST_TIMEOUT and returns, and so do those
+// that wait for it.
+__global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int ng, int epoch,
+                                                             int32_t* __restrict__ status) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const SlabJob& J = jobs.j[blockIdx.x / ng];
+  const int m = J.m, g = blockIdx.x % ng;
+  const int np = (m + kSlabW - 1) / kSlabW;
+  const int slots = g < np ? (np - g + ng - 1) / ng : 0;      // panels g, g + ng, ...
+  const int ms = (m + 1) & ~1;
+  double* T = reinterpret_cast<double*>(smem_raw);            // [2][kSlabW][ms]
+  double* X = T + 2 * kSlabW * (size_t)ms;                    // [slots * kSlabW][ms]
+  __shared__ double s_R[64 * kSlabW], s_prow[2][kSlabW], s_rp;
+  __shared__ unsigned long long s_key[2][kSlabWarps];
+  __shared__ int s_row[2][kSlabWarps], s_piv[2][kSlabW], s_abort, s_sing;
+  __shared__ uint8_t s_used[kSlabThreads * kSlabRows];
+  const int tid = threadIdx.x, lane = tid % kWarp, wid = tid / kWarp;
+  for (int i = tid; i < m; i += kSlabThreads) s_used[i] = 0;
+  if (tid == 0) { s_abort = 0; s_sing = 0; }
+  for (int c = wid; c < slots * kSlabW; c += kSlabWarps) {
+    const int col = ((c / kSlabW) * ng + g) * kSlabW + c % kSlabW;
+    for (int i = lane; i < m; i += kWarp) X[(size_t)c * ms + i] = col < m ? J.S[(size_t)col * m + i] : 0.0;
+  }
+  __syncthreads();
+
+  // T of buffer b (pivot rows s_piv[b]) on the columns [c0, c1) of the block
+  auto apply = [&](int b, int c0, int c1) {
+    const double* Tb = T + (size_t)b * kSlabW * ms;
+    __syncthreads();
+    for (int t = tid; t < (c1 - c0) * kSlabW; t += kSlabThreads)
+      s_R[t] = X[(size_t)(c0 + t / kSlabW) * ms + s_piv[b][t % kSlabW]];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSlabRows; ++r) {
+      const int i = tid + r * kSlabThreads;
+      if (r * kSlabThreads + wid * kWarp >= m) break;
+      if (i >= m) continue;
+      double t[kSlabW];
+#pragma unroll
+      for (int w = 0; w < kSlabW; ++w) t[w] = Tb[w * ms + i];
+      for (int c = c0; c < c1; ++c) {
+        const double* R = s_R + (c - c0) * kSlabW;
+        double x = X[(size_t)c * ms + i];
+#pragma unroll
+        for (int w = 0; w < kSlabW; ++w) x = fma(t[w], R[w], x);
+        X[(size_t)c * ms + i] = x;
+      }
+    }
+  };
+
+  // Factors the panel in the columns c0 .. c0 + kSlabW of the block (wp of them
+  // real): buffer b gets T and its pivot rows, the columns their final values.
+  auto factor = [&](int k, int b, int c0, int wp) {
+    double a[kSlabRows][kSlabW];
+    bool used[kSlabRows];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSlabRows; ++r) {
+      const int i = tid + r * kSlabThreads;
+      used[r] = i >= m || s_used[i] != 0;
+#pragma unroll
+      for (int w = 0; w < kSlabW; ++w) a[r][w] = i < m ? X[(size_t)(c0 + w) * ms + i] : 0.0;
+    }
+    // the block's candidate of panel column w: key and row of each warp's best unused row
+    auto offer = [&](int w) {
+      unsigned long long best = 0ull;
+      uint32_t row = 0xffffffffu;
+#pragma unroll
+      for (int r = 0; r < kSlabRows; ++r)
+        if (!used[r]) {
+          unsigned long long key = 0ull;
+#pragma unroll
+          for (int v = 0; v < kSlabW; ++v)
+            if (v == w) key = abs_key(a[r][v]);
+          if (row == 0xffffffffu || key > best) { best = key; row = tid + r * kSlabThreads; }
+        }
+      const bool has = row != 0xffffffffu;
+      const uint32_t hi = __reduce_max_sync(0xffffffffu, has ? (uint32_t)(best >> 32) : 0u);
+      const bool in = has && (uint32_t)(best >> 32) == hi;
+      const uint32_t lo = __reduce_max_sync(0xffffffffu, in ? (uint32_t)best : 0u);
+      const uint32_t win = __reduce_min_sync(0xffffffffu, in && (uint32_t)best == lo ? row : 0xffffffffu);
+      if (lane == 0) {
+        s_key[w & 1][wid] = ((unsigned long long)hi << 32) | lo;
+        s_row[w & 1][wid] = (int)win;   // -1: no unused row
+      }
+    };
+    // the best of the warps' candidates (every warp finds the same one)
+    auto choose = [&](int w, unsigned long long& key) {
+      const bool has = lane < kSlabWarps && s_row[w & 1][lane % kSlabWarps] >= 0;
+      const unsigned long long k0 = has ? s_key[w & 1][lane % kSlabWarps] : 0ull;
+      const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(k0 >> 32));
+      const bool in = has && (uint32_t)(k0 >> 32) == hi;
+      const uint32_t lo = __reduce_max_sync(0xffffffffu, in ? (uint32_t)k0 : 0u);
+      key = ((unsigned long long)hi << 32) | lo;
+      return (int)__reduce_min_sync(0xffffffffu,
+                                    in && (uint32_t)k0 == lo ? (uint32_t)s_row[w & 1][lane % kSlabWarps] : 0xffffffffu);
+    };
+    // reciprocal pivot (thread 0) and the pivot row's values (its owner)
+    auto publish = [&](int w, int pr, unsigned long long key) {
+#pragma unroll
+      for (int r = 0; r < kSlabRows; ++r)
+        if (tid + r * kSlabThreads == pr) {
+#pragma unroll
+          for (int v = 0; v < kSlabW; ++v) s_prow[w & 1][v] = a[r][v];
+          double pv = 1.0;
+#pragma unroll
+          for (int v = 0; v < kSlabW; ++v)
+            if (v == w) pv = a[r][v];
+          if (key == 0ull || key >= 0x7FF0000000000000ull) {
+            s_sing = 1;
+            pv = 1.0;
+          }
+          const double rp = 1.0 / pv;
+          s_rp = rp;
+          J.rd[pr] = rp;
+          J.piv[k * kSlabW + w] = pr;
+          s_piv[b][w] = pr;
+          s_used[pr] = 1;
+        }
+    };
+    offer(0);
+    __syncthreads();
+    unsigned long long key;
+    int pr = choose(0, key);
+    publish(0, pr, key);
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kSlabW; ++w) {
+      if (w >= wp) break;
+      double f[kSlabRows];
+      const double rp = s_rp;
+      double row[kSlabW];
+#pragma unroll
+      for (int v = 0; v < kSlabW; ++v) row[v] = s_prow[w & 1][v];
+      bool mine[kSlabRows];
+#pragma unroll
+      for (int r = 0; r < kSlabRows; ++r) {
+        if (r * kSlabThreads + wid * kWarp >= m) break;
+        mine[r] = tid + r * kSlabThreads == pr;
+        if (mine[r]) used[r] = true;
+        f[r] = mine[r] ? 0.0 : a[r][w] * rp;
+        if (w + 1 < kSlabW) a[r][(w + 1) % kSlabW] = fma(-f[r], row[(w + 1) % kSlabW], a[r][(w + 1) % kSlabW]);
+      }
+      const bool more = w + 1 < wp;
+      if (more) offer(w + 1);
+      __syncthreads();
+      int next = -1;
+      if (more) next = choose(w + 1, key);
+#pragma unroll
+      for (int r = 0; r < kSlabRows; ++r) {
+        if (r * kSlabThreads + wid * kWarp >= m) break;
+#pragma unroll
+        for (int v = 0; v < kSlabW; ++v)
+          if (v != w && v != w + 1) a[r][v] = fma(-f[r], row[v], a[r][v]);
+        a[r][w] = mine[r] ? 1.0 : -f[r];
+      }
+      if (more) publish(w + 1, next, key);
+      pr = next;
+      __syncthreads();
+    }
+    double* Tb = T + (size_t)b * kSlabW * ms;
+    double* Tg = J.T + (size_t)k * kSlabW * ms;
+#pragma unroll
+    for (int r = 0; r < kSlabRows; ++r) {
+      const int i = tid + r * kSlabThreads;
+      if (i >= m) continue;
+#pragma unroll
+      for (int w = 0; w < kSlabW; ++w) {
+        X[(size_t)(c0 + w) * ms + i] = a[r][w];
+        const double t = w < wp ? (i == s_piv[b][w] ? a[r][w] - 1.0 : a[r][w]) : 0.0;
+        Tb[w * ms + i] = t;
+        Tg[w * ms + i] = t;
+      }
+    }
+    if (tid < kSlabW && tid >= wp) s_piv[b][tid] = 0;   // its T column is zero
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) st_release(J.flag + k, epoch);
+  };
+
+  int ahead = -1;   // panel of this block that was factored ahead of its turn
+  for (int k = 0; k < np; ++k) {
+    const int b = k & 1;
+    if (k % ng == g) {
+      if (ahead != k) factor(k, b, (k / ng) * kSlabW, min(kSlabW, m - k * kSlabW));   // only k = 0, or one block
+    } else {
+      __syncthreads();
+      if (tid == 0) {
+        long long it = 0;
+        while (ld_acquire(J.flag + k) != epoch && it < kSlabWait) ++it;
+        if (it >= kSlabWait) s_abort = 1;
+      }
+      __syncthreads();
+      if (s_abort) {
+        if (tid == 0) atomicExch(&status[ST_TIMEOUT], 1);
+        return;
+      }
+      const double2* src = reinterpret_cast<const double2*>(J.T + (size_t)k * kSlabW * ms);
+      double2* dst = reinterpret_cast<double2*>(T + (size_t)b * kSlabW * ms);
+      for (int t = tid; t < kSlabW * ms / 2; t += kSlabThreads) dst[t] = __ldcg(src + t);
+      if (tid < kSlabW) {
+        const int pr = k * kSlabW + tid < m ? __ldcg(J.piv + k * kSlabW + tid) : 0;
+        s_piv[b][tid] = pr;
+        if (k * kSlabW + tid < m) s_used[pr] = 1;
+      }
+    }
+    // the next panel first, if it is this block's
+    const int nx = k + 1;
+    const int skip = k % ng == g ? k / ng : -1;
+    const bool next = nx < np && nx % ng == g && ng > 1;
+    if (next) {
+      apply(b, (nx / ng) * kSlabW, (nx / ng + 1) * kSlabW);
+      factor(nx, b ^ 1, (nx / ng) * kSlabW, min(kSlabW, m - nx * kSlabW));
+      ahead = nx;
+    }
+    // the block's other panels (the transform leaves its own panel's columns alone)
+    const int done = next ? nx / ng : -1;
+    for (int s = 0; s < slots; ) {
+      if (s == skip || s == done) { ++s; continue; }
+      int s1 = s;
+      while (s1 < slots && s1 != skip && s1 != done && s1 - s < 64 / kSlabW) ++s1;
+      apply(b, s * kSlabW, s1 * kSlabW);
+      s = s1;
+    }
+  }
+  __syncthreads();
+  // inverse[r][c] = rd[piv[r]] M[piv[r]][j], c the pivot row of column j: needs
+  // every panel's pivots, which this block has waited for
+  for (int c = wid; c < slots * kSlabW; c += kSlabWarps) {
+    const int col = ((c / kSlabW) * ng + g) * kSlabW + c % kSlabW;
+    if (col >= m) continue;
+    double* out = J.X + (size_t)__ldcg(J.piv + col) * m;
+    for (int r = lane; r < m; r += kWarp) {
+      const int pr = __ldcg(J.piv + r);
+      out[r] = __ldcg(J.rd + pr) * X[(size_t)c * ms + pr];
+    }
+  }
+  if (tid == 0 && s_sing) atomicExch(&status[ST_SINGULAR], 1);
+}
+
+namespace {
+size_t slab_gj_smem(int m, int ng) {
+  const size_t ms = (m + 1) & ~1, np = (m + kSlabW - 1) / kSlabW;
+  return (2 * kSlabW + (np + ng - 1) / ng * kSlabW) * ms * sizeof(double);
+}
+}  // namespace
+
+size_t slab_gj_scratch(int m) { return (size_t)((m + kSlabW - 1) / kSlabW) * kSlabW * ((m + 1) & ~1); }
+int slab_gj_panels(int m) { return (m + kSlabW - 1) / kSlabW; }
+
+bool slab_gj_fits(int m, int sm_count) {
+  return m <= kSlabThreads * kSlabRows && sm_count >= 4 && slab_gj_smem(m, sm_count / 2) <= 200 * 1024;
+}
+
+int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_count, cudaStream_t st) {
+  int ng = jobs.n == 1 ? sm_count : sm_count / 2, mmax = 0;
+  for (int i = 0; i < jobs.n; ++i) mmax = std::max(mmax, jobs.j[i].m);
+  ng = std::min(ng, slab_gj_panels(mmax));
+  const size_t smem = slab_gj_smem(mmax, ng);
+  if (cudaFuncSetAttribute(k_slab_gj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_slab_gj, kSlabThreads, smem);
+  if (per_sm < 1) return -1;
+  SlabJobs jb = jobs;
+  void* args[] = {(void*)&jb, (void*)&ng, (void*)&epoch, (void*)&status};
+  return cudaLaunchCooperativeKernel((const void*)k_slab_gj, ng * jobs.n, kSlabThreads, args, smem, st) == cudaSuccess
+             ? 0 : -2;
+}
+
+// ---------------------------------------------------------------------------
+// products of the elimination: C = beta C + alpha A B of up to two jobs in one
+// launch (column-major).  32 x 32 output tiles, so that the two sides' products
+// of 294 to 652 unknowns give every SM several tiles; the FP64 pipe bounds them.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_slab_gemm(SlabGemms jobs) {
+  __shared__ double As[16][32 + 1], Bs[16][32 + 1];
+  int t = blockIdx.x, j = 0;
+  if (t >= jobs.tiles0) { t -= jobs.tiles0; j = 1; }
+  const SlabGemm& g = jobs.g[j];
+  const int tr = (g.m + 31) / 32, r0 = (t % tr) * 32, c0 = (t / tr) * 32;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  double acc[2][2] = {};
+  for (int k0 = 0; k0 < g.k; k0 += 16) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int e = threadIdx.x + 256 * q;
+      const int r = e % 32, kk = e / 32;            // A tile: rows fastest (coalesced columns)
+      As[kk][r] = (r0 + r < g.m && k0 + kk < g.k) ? g.A[(int64_t)(k0 + kk) * g.lda + r0 + r] : 0.0;
+      const int kb = e % 16, cb = e / 16;           // B tile: k fastest (coalesced columns)
+      Bs[kb][cb] = (k0 + kb < g.k && c0 + cb < g.n) ? g.B[(int64_t)(c0 + cb) * g.ldb + k0 + kb] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < 16; ++kk) {
+      const double a0 = As[kk][tx], a1 = As[kk][tx + 16], b0 = Bs[kk][ty], b1 = Bs[kk][ty + 16];
+      acc[0][0] = fma(a0, b0, acc[0][0]);
+      acc[0][1] = fma(a0, b1, acc[0][1]);
+      acc[1][0] = fma(a1, b0, acc[1][0]);
+      acc[1][1] = fma(a1, b1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int r = r0 + tx + 16 * i, c = c0 + ty + 16 * k;
+      if (r < g.m && c < g.n) {
+        double* p = g.C + (int64_t)c * g.ldc + r;
+        *p = (g.beta == 0.0 ? 0.0 : g.beta * *p) + g.alpha * acc[i][k];
+      }
+    }
+}
+
+void launch_slab_gemm(const SlabGemm* g, int n, cudaStream_t st) {
+  SlabGemms jobs{};
+  int total = 0;
+  for (int i = 0; i < n; ++i) {
+    jobs.g[i] = g[i];
+    total += ((g[i].m + 31) / 32) * ((g[i].n + 31) / 32);
+    if (i == 0) jobs.tiles0 = total;
+  }
+  if (total > 0) k_slab_gemm<<<total, 256, 0, st>>>(jobs);
+}
+
+// ---------------------------------------------------------------------------
+// solve
+// ---------------------------------------------------------------------------
+namespace {
+constexpr int kSvThreads = 512;
+constexpr int kSvRows = 16;                            // rows of a thread block's product
+constexpr int kSvCols = kSvThreads / kSvRows;          // columns in flight
+
+// out[r0 + r] = beta y[r0 + r] + alpha sum_c A[(r0 + r) + c lda] x[c] for the
+// kSvRows rows of a thread block (the rows < nr): lanes over rows, column groups
+// over the threads, summed in a fixed order.  x is read through L2: other
+// blocks wrote it before the last grid barrier.
+__device__ __forceinline__ void block_gemv(const double* __restrict__ A, int64_t lda, int r0, int nr, int nc,
+                                           const double* x, double alpha, double beta, const double* y, double* out,
+                                           double* red) {
+  const int r = threadIdx.x % kSvRows, cgp = threadIdx.x / kSvRows;
+  const bool ok = r0 + r < nr;
+  const double* Ar = A + (ok ? r0 + r : 0);
+  double s0 = 0.0, s1 = 0.0;
+  int c = cgp;
+#pragma unroll 4
+  for (; c + kSvCols < nc; c += 2 * kSvCols) {
+    s0 = fma(__ldg(Ar + (int64_t)c * lda), __ldcg(x + c), s0);
+    s1 = fma(__ldg(Ar + (int64_t)(c + kSvCols) * lda), __ldcg(x + c + kSvCols), s1);
+  }
+  if (c < nc) s0 = fma(__ldg(Ar + (int64_t)c * lda), __ldcg(x + c), s0);
+  red[cgp * kSvRows + r] = s0 + s1;
+  __syncthreads();
+  if (threadIdx.x < kSvRows && ok) {
+    double s = 0.0;
+    for (int q = 0; q < kSvCols; ++q) s += red[q * kSvRows + threadIdx.x];
+    const double b = beta == 0.0 ? 0.0 : beta * __ldcg(y + r0 + r);
+    __stcg(out + r0 + r, fma(alpha, s, b));
+  }
+  __syncthreads();
+}
+}  // namespace
+
+// x = A^{-1} b over the slab ordering (b in w, overwritten; x in x): elimination
+// from both ends, the middle slab, back substitution to both ends; each step is
+// a product over the thread blocks followed by a grid barrier, the left
+// side's on the even blocks and the right side's on the odd ones.  Two products
+// per slab and direction; a step is bound by the barrier and one L2 round
+// trip (about 2.5 us) rather than by its 3.4 MB of matrix, so it is one launch
+// instead of 134: 0.4 ms against 1.5 for the 16 slabs of 652 unknowns.
+__global__ void __launch_bounds__(kSvThreads) k_slab_solve(SlabChain ch, const double* __restrict__ A, int64_t n,
+                                                           const double* __restrict__ sinv, double* w, double* x,
+                                                           double* u) {
+  cg::grid_group grid = cg::this_grid();
+  __shared__ double red[kSvThreads];
+  const int side = blockIdx.x & 1, b0 = blockIdx.x >> 1, nbk = gridDim.x >> 1;
+  const int K = ch.K, mid = ch.mid, p = ch.p;
+  double* us = u + (size_t)side * ch.mmax;
+  auto off = [&](int k) { return (int64_t)ch.off[k]; };
+  auto len = [&](int k) { return ch.off[k + 1] - ch.off[k]; };
+  auto inv = [&](int k) { return sinv + ch.inv[k]; };
+  // rows [0, nr) of a product over the blocks of one side
+  auto rows = [&](int nr, auto&& f) {
+    for (int r0 = b0 * kSvRows; r0 < nr; r0 += nbk * kSvRows) f(r0);
+  };
+  const int steps = max(mid, K - 1 - mid);
+  for (int s = 0; s < steps; ++s) {
+    const int kl = s + 1, kr = K - 2 - s;   // slabs that take a correction
+    if (side == 0 && kl <= mid) {
+      const int m = len(kl - 1);            // u = S_{kl-1}^{-1}[P,:] w_{kl-1}
+      rows(p, [&](int r0) { block_gemv(inv(kl - 1) + (m - p), m, r0, p, m, w + off(kl - 1), 1.0, 0.0, us, us, red); });
+    }
+    if (side == 1 && kr >= mid) {
+      const int m = len(kr + 1);            // u = S_{kr+1}^{-1} w_{kr+1}
+      rows(m, [&](int r0) { block_gemv(inv(kr + 1), m, r0, m, m, w + off(kr + 1), 1.0, 0.0, us, us, red); });
+    }
+    grid.sync();
+    // both sides correct the middle slab: the right one in the step's second half
+    const bool clash = kl == mid && kr == mid;
+    if (side == 0 && kl <= mid) {
+      const int m = len(kl);                // w_kl -= A_{kl,kl-1}[:,P] u
+      const double* B = A + (off(kl) - p) * n + off(kl);
+      rows(m, [&](int r0) { block_gemv(B, n, r0, m, p, us, -1.0, 1.0, w + off(kl), w + off(kl), red); });
+    }
+    if (clash) grid.sync();
+    if (side == 1 && kr >= mid) {
+      const int64_t o = off(kr + 1) - p;    // w_kr[P] -= A_{kr,kr+1}[P,:] u
+      rows(p, [&](int r0) {
+        block_gemv(A + off(kr + 1) * n + o, n, r0, p, len(kr + 1), us, -1.0, 1.0, w + o, w + o, red);
+      });
+    }
+    grid.sync();
+  }
+  {
+    const int m = len(mid);
+    for (int r0 = blockIdx.x * kSvRows; r0 < m; r0 += gridDim.x * kSvRows)
+      block_gemv(inv(mid), m, r0, m, m, w + off(mid), 1.0, 0.0, x + off(mid), x + off(mid), red);
+  }
+  grid.sync();
+  for (int s = 0; s < steps; ++s) {
+    const int kl = mid - 1 - s, kr = mid + 1 + s;
+    if (side == 0 && kl >= 0) {
+      const int64_t o = off(kl + 1) - p;    // w_kl[P] -= A_{kl,kl+1}[P,:] x_{kl+1}
+      rows(p, [&](int r0) {
+        block_gemv(A + off(kl + 1) * n + o, n, r0, p, len(kl + 1), x + off(kl + 1), -1.0, 1.0, w + o, w + o, red);
+      });
+    }
+    if (side == 1 && kr < K) {
+      const int m = len(kr);                // w_kr -= A_{kr,kr-1}[:,P] x_{kr-1}[P]
+      const double* B = A + (off(kr) - p) * n + off(kr);
+      rows(m, [&](int r0) { block_gemv(B, n, r0, m, p, x + off(kr) - p, -1.0, 1.0, w + off(kr), w + off(kr), red); });
+    }
+    grid.sync();
+    const int k = side == 0 ? kl : kr;
+    if (k >= 0 && k < K) {
+      const int m = len(k);
+      rows(m, [&](int r0) { block_gemv(inv(k), m, r0, m, m, w + off(k), 1.0, 0.0, x + off(k), x + off(k), red); });
+    }
+    grid.sync();
+  }
+}
+
+int launch_slab_solve(const SlabChain& ch, const double* A, int64_t n, const double* sinv, double* w, double* x,
+                      double* u, int sm_count, cudaStream_t st) {
+  // a block per 16 rows of a side's slab; more would only lengthen the barriers
+  const int grid = std::max(2, std::min(sm_count & ~1, 2 * ((ch.mmax + kSvRows - 1) / kSvRows)));
+  SlabChain c = ch;
+  void* args[] = {(void*)&c, (void*)&A, (void*)&n, (void*)&sinv, (void*)&w, (void*)&x, (void*)&u};
+  return cudaLaunchCooperativeKernel((const void*)k_slab_solve, grid, kSvThreads, args, 0, st) == cudaSuccess ? 0 : -2;
+}
+
+}  // namespace fsi

@@ -201,6 +201,44 @@ void launch_coarse_check(int B, int64_t nb, const int32_t* rowptr, const int32_t
                          const double* v, const double* x, double tol, const int32_t* pos, int32_t* status,
                          cudaStream_t st);
 
+// k_slab.cu: 3D coarse factorisation and solve from both ends of the slab chain
+struct SlabJob {
+  const double* S;   // m x m, column-major
+  double* T;         // slab_gj_scratch(m) doubles
+  double* X;         // its inverse
+  int m;
+  int32_t* piv;      // m
+  double* rd;        // m
+  int* flag;         // slab_gj_panels(m); never equal to a coming epoch
+};
+struct SlabJobs { int n; SlabJob j[2]; };
+struct SlabGemm {
+  int m, n, k;
+  double alpha, beta;
+  const double* A;
+  int64_t lda;
+  const double* B;
+  int64_t ldb;
+  double* C;
+  int64_t ldc;
+};
+struct SlabGemms { int tiles0; SlabGemm g[2]; };
+struct SlabChain {
+  int K, mid, p, mmax;
+  int off[FSI_MAX_BREAKS];        // slab k = positions off[k] .. off[k + 1] - 1
+  int64_t inv[FSI_MAX_BREAKS];    // its inverse's offset
+};
+size_t slab_gj_scratch(int m);
+int slab_gj_panels(int m);
+bool slab_gj_fits(int m, int sm_count);
+// inverses of up to two slab complements at once; epoch: another one on every call with the same flags.
+// A zero pivot raises ST_SINGULAR, a wait that ran out ST_TIMEOUT
+int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_count, cudaStream_t st);
+void launch_slab_gemm(const SlabGemm* g, int n, cudaStream_t st);   // n <= 2 products
+// x = A^{-1} w (w is overwritten); u: 2 mmax doubles
+int launch_slab_solve(const SlabChain& ch, const double* A, int64_t n, const double* sinv, double* w, double* x,
+                      double* u, int sm_count, cudaStream_t st);
+
 // coarse apply over an ordering of n of the ni unknowns (the others are
 // identity rows), dr its row scales: part holds ceil(n / 32) * n doubles of scratch
 template <typename TX, typename TY>
