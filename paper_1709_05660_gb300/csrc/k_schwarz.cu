@@ -399,13 +399,19 @@ size_t gj_small_smem(int n) {
 // owned) needs 0.52 of n^3 fused multiply-adds, against 0.98.  As in
 // gj_inverse_smem, warp 0 runs one pivot step ahead of the other warps.  Panels of
 // 16 columns leave room for two thread blocks per SM, whose panels and
-// updates overlap.  5-level channel (1,364 blocks): 171 -> 93.8 ms.
+// updates overlap.  The rank-W updates themselves run on the integer pipe
+// (fix_mad: 48 wide multiply-adds and two FP64 operations per entry and panel
+// instead of 16 FP64 ones).  5-level channel (1,364 blocks): 171 ms; with the
+// work left out 93.8; with the integer updates 40.2.
 template <typename T>
 __device__ __forceinline__ unsigned long long gj_key(T a) { return abs_key((double)a); }
 template <typename T>
 __device__ __forceinline__ bool gj_nonzero(T a) { return nonzero((double)a); }
 template <>
 __device__ __forceinline__ bool gj_nonzero<float>(float a) { return (__float_as_uint(a) << 1) != 0u; }
+
+// column stride of the panel, a multiple of 16 plus 2
+__host__ __device__ __forceinline__ int gj_blk_stride(int max_n) { return (max_n + 15) / 16 * 16 + 2; }
 
 template <typename T, int W>
 __global__ void __launch_bounds__(512)
@@ -419,7 +425,8 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
   // regions sized for the largest block of the launch (max_n), so the output
   // tile (32 x 33, placed in G; the host checks max_n * W >= 32 * 33) never
   // overlaps the pivot arrays, whatever this block's n
-  const int gs = max_n | 1;                           // odd column stride of the panel (bank conflicts)
+  constexpr bool FIX = std::is_same<T, double>::value && W <= kFixTerms;
+  const int gs = gj_blk_stride(max_n);                // column stride of the panel (16-byte pairs, few bank conflicts)
   T* G = reinterpret_cast<T*>(smem_raw);              // W * gs, by columns
   T* R = G + (size_t)W * gs;                          // W * max_n
   T* f = R + (size_t)W * max_n;                       // 2 * max_n multipliers
@@ -432,6 +439,8 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
   const int nch = (n + kWarp - 1) / kWarp, mch = (max_n + kWarp - 1) / kWarp;
   uint8_t* fl = live + max_n;                         // 2 * mch: rows 32 u ..: a multiplier is not zero
   uint8_t* cl = fl + 2 * mch;                         // mch: columns 32 u ..: a pivot-row entry is not zero
+  int* er = reinterpret_cast<int*>(f);                // scales of the trailing update: rows of G, columns of R
+  int* ec = er + max_n;                               // (the multipliers are not needed any more then)
   __shared__ int s_row[2], s_sing;
   T* M = dense + dense_off[p];
   const int nown = p_nown[p];
@@ -555,6 +564,20 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
       if (used[i] != 2)
         for (int m = 0; m < wp; ++m) nz |= gj_nonzero(G[m * gs + i]);
       live[i] = nz;
+      if constexpr (FIX) {   // rows of G and columns of R in fixed point, in place
+        int eg = 0, eb = 0;
+        for (int m = 0; m < wp; ++m) {
+          eg = max(eg, fix_exp(G[m * gs + i]));
+          eb = max(eb, fix_exp(R[m * max_n + i]));
+        }
+        er[i] = eg;
+        ec[i] = eb;
+        if (eg == 2047 || eb == 2047) s_sing = 1;   // not finite: fixed point would hide it
+        for (int m = 0; m < wp; ++m) {
+          reinterpret_cast<int2*>(G)[m * gs + i] = fix_digits(G[m * gs + i], eg);
+          reinterpret_cast<int2*>(R)[m * max_n + i] = fix_digits(R[m * max_n + i], eb);
+        }
+      }
     }
     __syncthreads();
     // trailing rank-wp update, 4 rows per warp pass sharing each R load
@@ -572,15 +595,34 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
         T acc[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) acc[r] = on[r] ? M[(int64_t)(i0 + r) * n + j] : T(0);
+        if constexpr (FIX) {
+          long long hh[4] = {}, mid[4] = {};
+          const int2* Rj = reinterpret_cast<const int2*>(R) + j;
+          const int4* Gq = reinterpret_cast<const int4*>(G + i0);   // i0 and the stride are even: two rows each
 #pragma unroll 4
-        for (int m = 0; m < wp; ++m) {
-          const T rv = R[m * max_n + j];
+          for (int m = 0; m < wp; ++m) {
+            const int2 rv = Rj[m * max_n];
+            const int4 g0 = Gq[m * (gs / 2)], g1 = Gq[m * (gs / 2) + 1];
+            fix_mad(hh[0], mid[0], make_int2(g0.x, g0.y), rv);
+            fix_mad(hh[1], mid[1], make_int2(g0.z, g0.w), rv);
+            fix_mad(hh[2], mid[2], make_int2(g1.x, g1.y), rv);
+            fix_mad(hh[3], mid[3], make_int2(g1.z, g1.w), rv);
+          }
+          const int eb = ec[j];
 #pragma unroll
-          for (int r = 0; r < 4; ++r) acc[r] += Gr[m * gs + r] * rv;
+          for (int r = 0; r < 4; ++r)
+            if (on[r]) M[(int64_t)(i0 + r) * n + j] = fix_add(acc[r], hh[r], mid[r], er[i0 + r], eb);
+        } else {
+#pragma unroll 4
+          for (int m = 0; m < wp; ++m) {
+            const T rv = R[m * max_n + j];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[r] += Gr[m * gs + r] * rv;
+          }
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (on[r]) M[(int64_t)(i0 + r) * n + j] = acc[r];
         }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          if (on[r]) M[(int64_t)(i0 + r) * n + j] = acc[r];
       }
     }
     __syncthreads();
@@ -1234,7 +1276,7 @@ bool launch_patch_gj_tc_levels(const GjLevels& lv, int nblocks, int max_n, int32
 
 template <typename T, int W>
 size_t gj_blk_smem(int n) {
-  return ((size_t)W * (n | 1) + (size_t)W * n + 3 * (size_t)n) * sizeof(T) + 2 * (size_t)n * sizeof(int) +
+  return ((size_t)W * gj_blk_stride(n) + (size_t)W * n + 3 * (size_t)n) * sizeof(T) + 2 * (size_t)n * sizeof(int) +
          3 * (size_t)n + 3 * ((size_t)n / kWarp + 1) + 64;
 }
 
