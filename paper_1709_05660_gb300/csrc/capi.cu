@@ -242,7 +242,6 @@ void build_device(Ctx& c) {
   const int L = (int)c.hl.size();
   c.dl.assign(L, DevLevel());
   const int dim = c.dim, B = c.B, nloc = c.nloc, nd = c.ndofe;
-  int64_t max_dense = 0;
   for (int l = 0; l < L; ++l) {
     HostLevel& H = c.hl[l];
     DevLevel& D = c.dl[l];
@@ -312,7 +311,6 @@ void build_device(Ctx& c) {
         D.dc = dalloc<double>(c, (size_t)H.idx_total);
         D.inv = dalloc<double>(c, (size_t)H.inv_total);
       }
-      max_dense = std::max(max_dense, H.dense_total);
       std::vector<char> is_ilu(H.n_patches, 0);
       if (c.opts.local_solver == 1) {
         // fluid blocks (material of the block's elements) up to the ILU size limit
@@ -400,12 +398,11 @@ void build_device(Ctx& c) {
   ck(cudaMallocHost((void**)&c.host_small, 512 * sizeof(double)), "cudaMallocHost");
   c.stage_a = dalloc<double>(c, F.N);
   c.stage_b = dalloc<double>(c, F.N);
-  // the mixed path factors the blocks of all levels in one launch: one
-  // workspace region per level
+  // the blocks of all levels are factored in one launch: one workspace region
+  // per level
   int64_t sum_dense = 0;
   for (int l = 1; l < L; ++l) sum_dense += c.hl[l].dense_total;
-  c.dense_ws_len = std::max<int64_t>(c.mixed ? sum_dense : max_dense, 1);
-  // patch factorisation workspace: max_dense elements of the factor precision
+  c.dense_ws_len = std::max<int64_t>(sum_dense, 1);
   c.dense_ws = dalloc<double>(c, c.mixed ? ((size_t)c.dense_ws_len + 1) / 2 : (size_t)c.dense_ws_len);
   // coarse dense operator
   const int64_t n0 = c.hl[0].Ni;
@@ -834,7 +831,7 @@ bool gather_mixed(Ctx& c, GjLevels& lv, int& first, int& max_n) {
   int64_t off = 0;
   bool ok = true;
   // the gathers of all levels in one launch when the table holds them
-  GatherLevels gl{};
+  GatherLevelsT<float> gl{};
   gl.B = c.B;
   int gblocks = 0;
   const bool one_launch = L - 1 <= kGjMaxLevels;
@@ -842,7 +839,7 @@ bool gather_mixed(Ctx& c, GjLevels& lv, int& first, int& max_n) {
     DevLevel& D = c.dl[l];
     if (one_launch) {
       if (D.n_patches > 0)
-        gl.l[gl.nlev++] = GatherLevel{D.p_n,    D.p_dense_off, D.p_gmap_off, D.p_gmap,      D.p_boff_off,
+        gl.l[gl.nlev++] = GatherLevelT<float>{D.p_n,    D.p_dense_off, D.p_gmap_off, D.p_gmap,      D.p_boff_off,
                                       D.p_boff, D.p_pad_off,   D.p_padpos,   D.val,         ws + off,
                                       D.p_idx_off, D.dr32,     D.dc32,       gblocks};
       gblocks += D.n_patches;
@@ -855,7 +852,7 @@ bool gather_mixed(Ctx& c, GjLevels& lv, int& first, int& max_n) {
     off += D.dense_total;
   }
   if (one_launch && gblocks > 0) {
-    launch_patch_gather_levels(gl, gblocks, c.stream);
+    launch_patch_gather_levels<float>(gl, gblocks, c.stream);
     counted(c);
   }
   off = 0;
@@ -928,15 +925,45 @@ void schwarz_factor(Ctx& c) {
       }
     }
   }
-  for (int l = 1; l < L && !c.mixed; ++l) {
-    DevLevel& D = c.dl[l];
-    Prof pr(c, FSI_K_PATCH_FACTOR, D.factor_bytes, D.factor_flops, 2);
-    launch_patch_gather_t<double>(D.n_patches, D.p_n, D.p_dense_off, D.p_gmap_off, D.p_gmap, D.p_boff_off,
-                                  D.p_boff, D.p_pad_off, D.p_padpos, D.val, B, c.dense_ws, D.p_idx_off, D.dr, D.dc,
-                                  c.stream);
-    launch_patch_gj_t<double>(D.n_patches, D.max_n, D.p_n, D.p_nown, D.p_dense_off, D.p_own_off, D.p_own,
-                              D.p_inv_off, c.dense_ws, D.inv, c.status, true, c.stream);
-    counted(c, 2);
+  if (!c.mixed && L > 1) {
+    // the same in FP64: every level in its own workspace region, the finest
+    // first, one gather and one factorisation launch (level by level the few
+    // blocks of the coarse levels ran alone, each as long as a wave of the finest)
+    GatherLevelsT<double> gl{};
+    GjLevelsT<double> lv{};
+    gl.B = B;
+    int first = 0, max_n = 0;
+    int64_t off = 0;
+    double by = 0.0, fl = 0.0;
+    for (int l = L - 1; l >= 1; --l) {
+      DevLevel& D = c.dl[l];
+      by += D.factor_bytes;
+      fl += D.factor_flops;
+      if (D.n_patches <= 0) continue;
+      double* ws = c.dense_ws + off;
+      gl.l[gl.nlev++] = GatherLevelT<double>{D.p_n,    D.p_dense_off, D.p_gmap_off, D.p_gmap, D.p_boff_off,
+                                             D.p_boff, D.p_pad_off,   D.p_padpos,   D.val,    ws,
+                                             D.p_idx_off, D.dr,       D.dc,         first};
+      lv.l[lv.nlev++] = GjLevelT<double>{D.p_n, D.p_nown, D.p_dense_off, D.p_own_off, D.p_own, D.p_inv_off, ws,
+                                         D.inv, c.status, nullptr, first};
+      first += D.n_patches;
+      max_n = std::max(max_n, D.max_n);
+      off += D.dense_total;
+    }
+    Prof pr(c, FSI_K_PATCH_FACTOR, by, fl, 2);
+    launch_patch_gather_levels<double>(gl, first, c.stream);
+    counted(c);
+    if (launch_patch_gj_levels_f64(lv, first, max_n, c.stream)) {
+      counted(c);
+    } else {
+      for (int i = 0; i < lv.nlev; ++i) {   // blocks too large for shared memory: level by level
+        const GjLevelT<double>& v = lv.l[i];
+        const int np = (i + 1 < lv.nlev ? lv.l[i + 1].first : first) - v.first;
+        launch_patch_gj_t<double>(np, max_n, v.p_n, v.p_nown, v.dense_off, v.own_off, v.own, v.inv_off, v.dense,
+                                  v.invT, v.status, true, c.stream);
+        counted(c);
+      }
+    }
   }
 }
 
@@ -1569,7 +1596,7 @@ static int64_t estimate_device_bytes(const Ctx& c) {
   const bool mixed = c.opts.precision == FSI_MIXED;
   const double fs = mixed ? 4.0 : 8.0;
   const int B = c.B, nd = c.ndofe, m = c.opts.restart;
-  double b = 0.0, max_dense = 0.0;
+  double b = 0.0;
   const size_t L = c.hl.size();
   for (size_t l = 0; l < L; ++l) {
     const HostLevel& H = c.hl[l];
@@ -1584,7 +1611,6 @@ static int64_t estimate_device_bytes(const Ctx& c) {
            H.p_padpos.size() * 4.0 + (H.p_boff.size() + H.p_gptr.size()) * 4.0 + H.inv_total * fs +
            2.0 * H.idx_total * fs;
       if (mixed) b += H.nnzb * B * B * 4.0 + (H.P_col.size() + H.R_col.size()) * 4.0 + H.Ni * 3.0 * 4.0;
-      max_dense = std::max(max_dense, (double)H.dense_total);
     }
   }
   const HostLevel& F = c.hl.back();
@@ -1595,7 +1621,7 @@ static int64_t estimate_device_bytes(const Ctx& c) {
   if (c.dim == 3) b += (double)assemble_3d_scratch_doubles(max_assembly_batch(c)) * 8.0;
   double sum_dense = 0.0;
   for (size_t l = 1; l < L; ++l) sum_dense += (double)c.hl[l].dense_total;
-  b += (mixed ? sum_dense : max_dense) * fs + F.n_elem * (double)nd * 8.0 + 1e6;
+  b += sum_dense * fs + F.n_elem * (double)nd * 8.0 + 1e6;
   const HostLevel& H0 = c.hl[0];
   const std::vector<int64_t>& so = H0.slab_off;
   b += 2.0 * n0 * 8.0 + H0.free_map.size() * 4.0 + n0 * 4.0;   // right-hand side, row scales, free ordering

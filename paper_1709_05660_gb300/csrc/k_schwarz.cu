@@ -334,25 +334,31 @@ k_patch_gj_t(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown
 // the other's updates.  GB300, 3-level channel (2 x 2-element blocks of 112
 // unknowns): 3.3 -> 1.58 ms against the sweep that updates every
 // element in every step.
+// the level of a table that this thread block belongs to
+template <typename T>
+__device__ __forceinline__ const GjLevelT<T>& gj_level(const GjLevelsT<T>& lv) {
+  int l = 0;
+  while (l + 1 < lv.nlev && (int)blockIdx.x >= lv.l[l + 1].first) ++l;
+  return lv.l[l];
+}
+
 constexpr int kGjPad = 1;   // column stride n + 1: conflict-free transposed stores
 __global__ void __launch_bounds__(512)
-k_patch_gj_small(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown,
-                 const int64_t* __restrict__ dense_off, const int64_t* __restrict__ own_off,
-                 const int32_t* __restrict__ own, const int64_t* __restrict__ inv_off,
-                 const double* __restrict__ dense, double* __restrict__ invT, int32_t* __restrict__ status) {
+k_patch_gj_small(const GjLevelsT<double> lv) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ GjStep step;
-  const int p = blockIdx.x;
-  const int n = p_n[p], ld = n + kGjPad;
+  const GjLevelT<double>& L = gj_level(lv);
+  const int p = (int)blockIdx.x - L.first;
+  const int n = L.p_n[p], ld = n + kGjPad;
   double* M = reinterpret_cast<double*>(smem_raw);
   double* f = M + (size_t)n * ld;
   double* rd = f + 2 * n;
   int* piv = reinterpret_cast<int*>(rd + n);
   int* qinv = piv + n;
   uint8_t* isown = reinterpret_cast<uint8_t*>(qinv + n);
-  const int nown = p_nown[p];
-  const int32_t* ow = own + own_off[p];
-  const double* Mg = dense + dense_off[p];
+  const int nown = L.p_nown[p];
+  const int32_t* ow = L.own + L.own_off[p];
+  const double* Mg = L.dense + L.dense_off[p];
   for (int i = threadIdx.x; i < n; i += blockDim.x) isown[i] = 0;
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) M[(t % n) * ld + t / n] = Mg[t];
   __syncthreads();
@@ -360,7 +366,7 @@ k_patch_gj_small(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_
     if (FSI_IN(ow[o], n, FSI_SITE(1))) isown[ow[o]] = 1;
   __syncthreads();
   const bool ok = gj_inverse_smem(M, n, ld, f, rd, piv, qinv, step, isown);
-  double* out = invT + inv_off[p];
+  double* out = L.invT + L.inv_off[p];
   const int opad = own_pad(nown);
   for (int t = threadIdx.x; t < n * opad; t += blockDim.x) {
     const int c = t / opad, o = t - c * opad;
@@ -371,7 +377,7 @@ k_patch_gj_small(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_
     }
     out[t] = v;
   }
-  if (threadIdx.x == 0 && !ok) atomicExch(&status[ST_SINGULAR], 1);
+  if (threadIdx.x == 0 && !ok) atomicExch(&L.status[ST_SINGULAR], 1);
 }
 
 size_t gj_small_smem(int n) {
@@ -415,13 +421,11 @@ __host__ __device__ __forceinline__ int gj_blk_stride(int max_n) { return (max_n
 
 template <typename T, int W>
 __global__ void __launch_bounds__(512)
-k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown,
-               const int64_t* __restrict__ dense_off, const int64_t* __restrict__ own_off,
-               const int32_t* __restrict__ own, const int64_t* __restrict__ inv_off, T* __restrict__ dense,
-               T* __restrict__ invT, int32_t* __restrict__ status, int max_n) {
+k_patch_gj_blk(const GjLevelsT<T> lv, int max_n) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int p = blockIdx.x;
-  const int n = p_n[p];
+  const GjLevelT<T>& L = gj_level(lv);
+  const int p = (int)blockIdx.x - L.first;
+  const int n = L.p_n[p];
   // regions sized for the largest block of the launch (max_n), so the output
   // tile (32 x 33, placed in G; the host checks max_n * W >= 32 * 33) never
   // overlaps the pivot arrays, whatever this block's n
@@ -442,9 +446,9 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
   int* er = reinterpret_cast<int*>(f);                // scales of the trailing update: rows of G, columns of R
   int* ec = er + max_n;                               // (the multipliers are not needed any more then)
   __shared__ int s_row[2], s_sing;
-  T* M = dense + dense_off[p];
-  const int nown = p_nown[p];
-  const int32_t* ow = own + own_off[p];
+  T* __restrict__ M = L.dense + L.dense_off[p];
+  const int nown = L.p_nown[p];
+  const int32_t* ow = L.own + L.own_off[p];
   for (int i = threadIdx.x; i < n; i += blockDim.x) { used[i] = 0; isown[i] = 0; }
   if (threadIdx.x == 0) s_sing = 0;
   __syncthreads();
@@ -508,9 +512,18 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
   };
   for (int k0 = 0; k0 < n; k0 += W) {
     const int wp = min(W, n - k0);
-    for (int t = threadIdx.x; t < n * W; t += blockDim.x) {
-      const int i = t / W, m = t % W;
-      if (m < wp) G[m * gs + i] = M[(int64_t)i * n + k0 + m];
+    for (int t0 = threadIdx.x; t0 < n * W; t0 += 6 * (int)blockDim.x) {   // six loads in flight per thread
+      T v[6];
+#pragma unroll
+      for (int u = 0; u < 6; ++u) {
+        const int t = t0 + u * (int)blockDim.x;
+        v[u] = t < n * W && t % W < wp ? M[(int64_t)(t / W) * n + k0 + t % W] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 6; ++u) {
+        const int t = t0 + u * (int)blockDim.x;
+        if (t < n * W) G[(t % W) * gs + t / W] = v[u];
+      }
     }
     __syncthreads();
     if (wid == 0) prepare(0, k0);
@@ -632,7 +645,7 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
   __syncthreads();
   // owned rows of the inverse, transposed through a shared tile (reuses G)
   T* tile = G;   // 32 x 33
-  T* out = invT + inv_off[p];
+  T* out = L.invT + L.inv_off[p];
   for (int o0 = 0; o0 < own_pad(nown); o0 += 32) {
     for (int c0 = 0; c0 < n; c0 += 32) {
       for (int t = threadIdx.x; t < 32 * 32; t += blockDim.x) {
@@ -652,7 +665,7 @@ k_patch_gj_blk(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_no
       __syncthreads();
     }
   }
-  if (threadIdx.x == 0 && s_sing) atomicExch(&status[ST_SINGULAR], 1);
+  if (threadIdx.x == 0 && s_sing) atomicExch(&L.status[ST_SINGULAR], 1);
 }
 
 // FP32 panel-blocked Gauss-Jordan, same sweep as k_patch_gj_blk with:
@@ -1390,17 +1403,19 @@ __global__ void k_patch_gather_t(const int32_t* __restrict__ p_n, const int64_t*
 // block i - first of the level whose range holds i), so that the coarse
 // levels' few blocks run beside the finest level's instead of each paying a
 // launch of their own
-__global__ void __launch_bounds__(512) k_patch_gather_levels(const GatherLevels lv) {
+template <typename T>
+__global__ void __launch_bounds__(512) k_patch_gather_levels(const GatherLevelsT<T> lv) {
   int l = 0;
   while (l + 1 < lv.nlev && (int)blockIdx.x >= lv.l[l + 1].first) ++l;
-  const GatherLevel& G = lv.l[l];
-  gather_block<float>((int)blockIdx.x - G.first, G.p_n, G.dense_off, G.gmap_off, G.gmap, G.boff_off, G.boff,
+  const GatherLevelT<T>& G = lv.l[l];
+  gather_block<T>((int)blockIdx.x - G.first, G.p_n, G.dense_off, G.gmap_off, G.gmap, G.boff_off, G.boff,
                       G.pad_off, G.padpos, G.bsr_val, lv.B, G.dense, G.idx_off, G.dr, G.dc);
 }
 
-void launch_patch_gather_levels(const GatherLevels& lv, int nblocks, cudaStream_t st) {
+template <typename T>
+void launch_patch_gather_levels(const GatherLevelsT<T>& lv, int nblocks, cudaStream_t st) {
   if (nblocks <= 0 || lv.nlev < 1) return;
-  k_patch_gather_levels<<<nblocks, 512, 0, st>>>(lv);
+  k_patch_gather_levels<T><<<nblocks, 512, 0, st>>>(lv);
 }
 
 
@@ -1416,15 +1431,23 @@ void launch_patch_gather_t(int np, const int32_t* p_n, const int64_t* dense_off,
 }
 
 template <typename T, int W>
-bool try_gj_blk(int np, int max_n, const int32_t* p_n, const int32_t* p_nown, const int64_t* dense_off,
-                const int64_t* own_off, const int32_t* own, const int64_t* inv_off, T* dense, T* invT,
-                int32_t* status, cudaStream_t st) {
+bool try_gj_blk(const GjLevelsT<T>& lv, int nblocks, int max_n, cudaStream_t st) {
   const size_t smem = gj_blk_smem<T, W>(max_n);
   if (smem > 220 * 1024 || (size_t)32 * 33 > (size_t)max_n * W) return false;
   cudaFuncSetAttribute(k_patch_gj_blk<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_patch_gj_blk<T, W><<<np, 512, smem, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status,
-                                               max_n);
+  k_patch_gj_blk<T, W><<<nblocks, 512, smem, st>>>(lv, max_n);
   return true;
+}
+
+bool launch_patch_gj_levels_f64(const GjLevelsT<double>& lv, int nblocks, int max_n, cudaStream_t st) {
+  if (nblocks <= 0 || lv.nlev < 1 || lv.nlev > kGjMaxLevels) return false;
+  if (max_n <= kGjSmemMax) {
+    const size_t smem = gj_small_smem(max_n);
+    cudaFuncSetAttribute(k_patch_gj_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_patch_gj_small<<<nblocks, 512, smem, st>>>(lv);
+    return true;
+  }
+  return try_gj_blk<double, 16>(lv, nblocks, max_n, st) || try_gj_blk<double, 8>(lv, nblocks, max_n, st);
 }
 
 template <typename T>
@@ -1432,14 +1455,11 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
                        const int64_t* own_off, const int32_t* own, const int64_t* inv_off, T* dense, T* invT,
                        int32_t* status, bool n_mult4, cudaStream_t st) {
   if (np <= 0) return;
-  if (std::is_same<T, double>::value && max_n <= kGjSmemMax) {
-    const size_t smem = gj_small_smem(max_n);
-    cudaFuncSetAttribute(k_patch_gj_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_patch_gj_small<<<np, 512, smem, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off,
-                                            reinterpret_cast<const double*>(dense),
-                                            reinterpret_cast<double*>(invT), status);
-    return;
-  }
+  GjLevelsT<T> one{};
+  one.nlev = 1;
+  one.l[0] = GjLevelT<T>{p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, nullptr, 0};
+  if constexpr (std::is_same<T, double>::value)
+    if (launch_patch_gj_levels_f64(one, np, max_n, st)) return;
   // small blocks: the whole matrix fits in shared memory (unblocked sweep)
   const size_t base = (size_t)max_n * (2 * sizeof(T) + 2 * sizeof(int)) + ((max_n + 15) / 16) * 16;
   const size_t with_m = base + (size_t)max_n * max_n * sizeof(T);
@@ -1461,10 +1481,10 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
     if (try_gj_f32<32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, st)) return;
     if (try_gj_f32<16>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, st)) return;
   }
-  if (std::is_same<T, float>::value &&
-      try_gj_blk<T, 32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
-  if (try_gj_blk<T, 16>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
-  if (try_gj_blk<T, 8>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
+  if constexpr (std::is_same<T, float>::value)
+    if (try_gj_blk<T, 32>(one, np, max_n, st) || try_gj_blk<T, 16>(one, np, max_n, st) ||
+        try_gj_blk<T, 8>(one, np, max_n, st))
+      return;
   cudaFuncSetAttribute(k_patch_gj_t<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
   k_patch_gj_t<T, false><<<np, 512, base, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT,
                                                 status);
@@ -1884,6 +1904,7 @@ void launch_patch_apply_ilu(int nsel, int max_n, int max_nb, const int32_t* sel,
 }
 
 #define FSI_INST(T)                                                                                              \
+  template void launch_patch_gather_levels<T>(const GatherLevelsT<T>&, int, cudaStream_t);                        \
   template void launch_patch_gather_t<T>(int, const int32_t*, const int64_t*, const int64_t*, const int32_t*,  \
                                          const int64_t*, const int32_t*, const int64_t*, const int32_t*,        \
                                          const double*, int, T*, const int64_t*, T*, T*, cudaStream_t);         \

@@ -77,26 +77,30 @@ void launch_nonfinite_check(int64_t n, const double* v, int32_t* status, cudaStr
 // Schwarz blocks of one level for the tensor-core factorisation; several
 // levels can share one launch (blocks first .. first + n_patches - 1)
 constexpr int kGjMaxLevels = 24;   // levels of one launch (several instances may share it)
-struct GjLevel {
+template <typename T>
+struct GjLevelT {
   const int32_t* p_n;
   const int32_t* p_nown;
   const int64_t* dense_off;
   const int64_t* own_off;
   const int32_t* own;
   const int64_t* inv_off;
-  float* dense;
-  float* invT;
+  T* dense;
+  T* invT;
   int32_t* status;   // status flags of the instance the level belongs to
   const int32_t* sel; // blocks of the level to factor (nullptr: all of them)
   int first;
 };
-struct GjLevels {
+template <typename T>
+struct GjLevelsT {
   int nlev;
   // iteration limit of the first bounded wait of each block on its tensor-core
   // work (the drain waits before tensor memory is released keep their full limit)
   long long first_wait;
-  GjLevel l[kGjMaxLevels];
+  GjLevelT<T> l[kGjMaxLevels];
 };
+using GjLevel = GjLevelT<float>;
+using GjLevels = GjLevelsT<float>;
 constexpr long long kTcWaitIters = 1LL << 22;
 // Gauss-Jordan variant code: 16-column panels on 64-column tiles with 256
 // tensor-memory columns, so that two blocks share an SM (blocks <= 512 unknowns)
@@ -109,8 +113,9 @@ bool launch_patch_gj_tc_levels(const GjLevels& lv, int nblocks, int max_n, int32
 // panel width of the tensor-core variant that launch_patch_gj_tc_levels picks
 // for blocks up to max_n with preference `panel` (0: none fits)
 int gj_tc_variant(int max_n, int panel);
-// the FP32 gathers of the Schwarz levels of one instance in one launch
-struct GatherLevel {
+// the gathers of the Schwarz levels of one instance in one launch
+template <typename T>
+struct GatherLevelT {
   const int32_t* p_n;
   const int64_t* dense_off;
   const int64_t* gmap_off;
@@ -120,17 +125,22 @@ struct GatherLevel {
   const int64_t* pad_off;
   const int32_t* padpos;
   const double* bsr_val;
-  float* dense;
+  T* dense;
   const int64_t* idx_off;
-  float* dr;
-  float* dc;
+  T* dr;
+  T* dc;
   int first;   // first thread block of the level
 };
-struct GatherLevels {
+template <typename T>
+struct GatherLevelsT {
   int nlev, B;
-  GatherLevel l[kGjMaxLevels];
+  GatherLevelT<T> l[kGjMaxLevels];
 };
-void launch_patch_gather_levels(const GatherLevels& lv, int nblocks, cudaStream_t st);
+template <typename T>
+void launch_patch_gather_levels(const GatherLevelsT<T>& lv, int nblocks, cudaStream_t st);
+// FP64 blocks of the levels in one launch; false when they fit no shared-memory
+// variant (the caller then factors level by level)
+bool launch_patch_gj_levels_f64(const GjLevelsT<double>& lv, int nblocks, int max_n, cudaStream_t st);
 // boff / boff_off: per local block of a Schwarz block its dense offset * 8 + width
 template <typename T>
 void launch_patch_gather_t(int np, const int32_t* p_n, const int64_t* dense_off, const int64_t* gmap_off,
