@@ -1306,7 +1306,18 @@ void orthonormalize(Ctx& c, int j, int passes, double* h, double* hn, double* wn
   double* sm = c.small;
   double* hs = c.host_small;
   Prof pr(c, FSI_K_KRYLOV, (2.0 * passes * (j + 1) + 8.0) * n * 8.0, (4.0 * passes * (j + 1) + 4.0) * n,
-          passes == 2 ? 8 : 5);
+          j + 1 <= 32 ? 1 : (passes == 2 ? 8 : 5));
+  double* vnext = c.V + (size_t)(j + 1) * n;
+  if (launch_arnoldi_step(n, c.V, n, j + 1, passes, c.w, vnext, c.partial, nb, sm, c.stream)) {
+    counted(c);
+    ck(cudaMemcpyAsync(hs, sm, 260 * sizeof(double), cudaMemcpyDeviceToHost, c.stream), "D2H");
+    sync(c);
+    for (int i = 0; i <= j; ++i) h[i] = hs[i] + (passes == 2 ? hs[128 + i] : 0.0);
+    *hn = hs[257];
+    *wn0 = std::sqrt(hs[j + 1]);
+    return;
+  }
+  // restart lengths beyond the fused kernel's, launch by launch
   // pass 1: h1 = V^T w (with ||w||^2)
   launch_arnoldi_dots(n, c.V, n, j + 1, c.w, true, c.partial, nb, c.stream);
   launch_reduce(c.partial, j + 2, nb, sm, false, c.stream);             // h1 = sm[0..j], ||w||^2 = sm[j+1]

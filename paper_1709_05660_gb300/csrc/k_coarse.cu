@@ -304,18 +304,27 @@ __global__ void k_coarse_check(int B, int64_t nb, const int32_t* __restrict__ ro
                                const double* __restrict__ val, const double* __restrict__ v,
                                const double* __restrict__ x, double tol, const int32_t* __restrict__ pos,
                                int32_t* __restrict__ status) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb * B || pos[i] < 0) return;
-  const int64_t br = i / B;
-  const int ci = (int)(i % B);
-  double s = v[i], a = fabs(v[i]);
-  for (int32_t k = rowptr[br]; k < rowptr[br + 1]; ++k)
-    for (int c = 0; c < B; ++c) {
-      const double t = val[((int64_t)k * B + ci) * B + c] * x[(int64_t)col[k] * B + c];
-      s -= t;
-      a += fabs(t);
-    }
-  if (!(fabs(s) <= tol * a)) atomicExch(&status[ST_COARSE_RETRY], 1);
+  // eight lanes per row
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 8;
+  const int sub = threadIdx.x % 8;
+  const bool on = i < nb * B && pos[i] >= 0;
+  double s = 0.0, a = 0.0;
+  if (on) {
+    const int64_t br = i / B;
+    const int ci = (int)(i % B);
+    for (int32_t k = rowptr[br] + sub; k < rowptr[br + 1]; k += 8)
+      for (int c = 0; c < B; ++c) {
+        const double t = val[((int64_t)k * B + ci) * B + c] * x[(int64_t)col[k] * B + c];
+        s += t;
+        a += fabs(t);
+      }
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+  }
+  if (on && sub == 0 && !(fabs(v[i] - s) <= tol * (a + fabs(v[i])))) atomicExch(&status[ST_COARSE_RETRY], 1);
 }
 
 // entries in (-1, 1), none of them zero, at the unknowns of the ordering
@@ -334,7 +343,7 @@ void launch_coarse_check(int B, int64_t nb, const int32_t* rowptr, const int32_t
                          const double* v, const double* x, double tol, const int32_t* pos, int32_t* status,
                          cudaStream_t st) {
   const int64_t n = nb * B;
-  k_coarse_check<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(B, nb, rowptr, col, val, v, x, tol, pos, status);
+  k_coarse_check<<<(unsigned)((n * 8 + 255) / 256), 256, 0, st>>>(B, nb, rowptr, col, val, v, x, tol, pos, status);
 }
 
 }  // namespace fsi

@@ -238,7 +238,20 @@ __global__ void k_csr_spmv(int64_t nrows, const int32_t* __restrict__ ptr, const
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nrows) return;
   TY acc = TY(0);
-  for (int32_t k = ptr[i]; k < ptr[i + 1]; ++k) acc += TY(val[k]) * TY(x[col[k]]);
+  int32_t k = ptr[i];
+  const int32_t k1 = ptr[i + 1];
+  for (; k + 4 <= k1; k += 4) {   // the loads of four entries in flight
+    int32_t c[4];
+    TV v[4];
+    TX xv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { c[u] = col[k + u]; v[u] = val[k + u]; }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) xv[u] = x[c[u]];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc += TY(v[u]) * TY(xv[u]);
+  }
+  for (; k < k1; ++k) acc += TY(val[k]) * TY(x[col[k]]);
   y[i] = add ? y[i] + acc : acc;
 }
 
@@ -466,6 +479,103 @@ void launch_arnoldi_update_norm(int64_t n, const double* V, int64_t ldv, int nve
   else k_arnoldi_update_norm<128><<<nblk, 256, 0, st>>>(n, V, ldv, nvec, h, w, partial);
 }
 
+// One Arnoldi step in one cooperative launch: w is orthogonalised against
+// V[0 .. nvec - 1] by `passes` passes of classical Gram-Schmidt and
+// normalised into vnext.  A pass's update w -= V h is followed at once, row by
+// row, by the products of the new w that the next pass (or the norm) needs, so two
+// passes read the basis three times instead of four.  Every block adds the blocks'
+// partial sums itself, in a fixed order.  As separate launches (eight for two
+// passes) the step took 25 us on small problems, mostly launches.
+// out: h of the first pass, then ||w||^2 before it; out[128 ..]: h of the second
+// pass; out[257]: ||w|| after the passes.  partial: 3 (nvec + 1) gridDim.x doubles.
+template <int NV>
+__global__ void __launch_bounds__(256, 2) k_arnoldi_step(int64_t n, const double* __restrict__ V, int64_t ldv, int nvec,
+                                                      int passes, double* __restrict__ w,
+                                                      double* __restrict__ vnext, double* __restrict__ partial,
+                                                      double* __restrict__ out) {
+  cg::grid_group grid = cg::this_grid();
+  __shared__ double red[8 * (NV + 1)];
+  __shared__ double h[NV + 1];
+  const int lane = threadIdx.x % kWarp, wid = threadIdx.x / kWarp, nw = blockDim.x / kWarp;
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  // h[v] = sum over the blocks of region `reg`'s partial sums v (cnt of them)
+  auto gather = [&](int reg, int cnt) {
+    const double* p = partial + (int64_t)reg * (nvec + 1) * gridDim.x;
+    __syncthreads();
+    for (int v = wid; v < cnt; v += nw) {
+      double s = 0.0;
+      for (int b = lane; b < (int)gridDim.x; b += kWarp) s += __ldcg(p + (int64_t)v * gridDim.x + b);
+#pragma unroll
+      for (int o = kWarp / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) h[v] = s;
+    }
+    __syncthreads();
+  };
+  double acc[NV], nn = 0.0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+  for (int64_t i = i0; i < n; i += step) {
+    const double wi = w[i];
+    nn = fma(wi, wi, nn);
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+      if (v < nvec) acc[v] = fma(V[(int64_t)v * ldv + i], wi, acc[v]);
+  }
+  block_partials<NV>(acc, nvec, nn, true, red, partial + blockIdx.x, gridDim.x);
+  grid.sync();
+  gather(0, nvec + 1);
+  if (blockIdx.x == 0)
+    for (int v = threadIdx.x; v <= nvec; v += blockDim.x) out[v] = h[v];
+  for (int p = 1; p <= passes; ++p) {
+    const bool last = p == passes;
+    nn = 0.0;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+    for (int64_t i = i0; i < n; i += step) {
+      double wi = w[i];
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        if (v < nvec) wi = fma(-V[(int64_t)v * ldv + i], h[v], wi);
+      w[i] = wi;
+      if (last) {
+        nn = fma(wi, wi, nn);
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          if (v < nvec) acc[v] = fma(V[(int64_t)v * ldv + i], wi, acc[v]);
+      }
+    }
+    __syncthreads();
+    block_partials<NV>(acc, last ? 0 : nvec, nn, last, red, partial + (int64_t)p * (nvec + 1) * gridDim.x + blockIdx.x,
+                       gridDim.x);
+    grid.sync();
+    gather(p, last ? 1 : nvec);
+    if (!last && blockIdx.x == 0)
+      for (int v = threadIdx.x; v < nvec; v += blockDim.x) out[128 + v] = h[v];
+  }
+  const double norm = sqrt(h[0]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) out[257] = norm;
+  const double inv = 1.0 / norm;
+  for (int64_t i = i0; i < n; i += step) vnext[i] = w[i] * inv;
+}
+
+bool launch_arnoldi_step(int64_t n, const double* V, int64_t ldv, int nvec, int passes, double* w, double* vnext,
+                         double* partial, int max_blocks, double* out, cudaStream_t st) {
+  // a thread a row, up to the co-resident blocks
+  int grid = (int)std::max<int64_t>(1, std::min<int64_t>(max_blocks, (n + 255) / 256));
+  void* args[] = {(void*)&n, (void*)&V, (void*)&ldv, (void*)&nvec, (void*)&passes, (void*)&w, (void*)&vnext,
+                  (void*)&partial, (void*)&out};
+  auto go = [&](auto kern) {
+    if (cudaLaunchCooperativeKernel((const void*)kern, grid, 256, args, 0, st) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+  };
+  if (nvec <= 8) return go(k_arnoldi_step<8>);
+  if (nvec <= 16) return go(k_arnoldi_step<16>);
+  if (nvec <= 32) return go(k_arnoldi_step<32>);
+  return false;
+}
+
 // x += sum_v Z[v] coef[v]
 __global__ void k_combo(int64_t n, const double* __restrict__ Z, int64_t ldz, int nvec, const double* __restrict__ c,
                         double* __restrict__ x) {
@@ -504,17 +614,24 @@ void launch_nonfinite_check(int64_t n, const double* v, int32_t* status, cudaStr
 __global__ void k_coarse_row_scale(int B, int64_t nb, const int32_t* __restrict__ rowptr,
                                    const int32_t* __restrict__ col, const double* __restrict__ val,
                                    const int32_t* __restrict__ perm, int64_t n, double* __restrict__ dr) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb * B || perm[i] < 0 || !FSI_IN(perm[i], n, FSI_SITE(2))) return;
-  const int64_t br = i / B;
-  const int ci = (int)(i % B);
+  // eight lanes per row
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 8;
+  const int sub = threadIdx.x % 8;
   uint32_t top = 0u;   // largest exponent field
-  for (int32_t k = rowptr[br]; k < rowptr[br + 1]; ++k)
-    for (int c = 0; c < B; ++c)
-      if (perm[(int64_t)col[k] * B + c] >= 0)
-        top = max(top, (uint32_t)(abs_key(val[((int64_t)k * B + ci) * B + c]) >> 52));
+  const bool on = i < nb * B && perm[i] >= 0 && FSI_IN(perm[i], n, FSI_SITE(2));
+  if (on) {
+    const int64_t br = i / B;
+    const int ci = (int)(i % B);
+    for (int32_t k = rowptr[br] + sub; k < rowptr[br + 1]; k += 8)
+      for (int c = 0; c < B; ++c)
+        if (perm[(int64_t)col[k] * B + c] >= 0)
+          top = max(top, (uint32_t)(abs_key(val[((int64_t)k * B + ci) * B + c]) >> 52));
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
   // 2^(1023 - e) for e = 1 .. 2045 as a bit pattern; zero, tiny and non-finite rows keep their scale
-  dr[perm[i]] = top >= 1u && top <= 2045u ? __longlong_as_double((long long)(2046u - top) << 52) : 1.0;
+  if (on && sub == 0)
+    dr[perm[i]] = top >= 1u && top <= 2045u ? __longlong_as_double((long long)(2046u - top) << 52) : 1.0;
 }
 
 // Dense coarse operator in the banded ordering, rows scaled by dr, column-major:
@@ -526,13 +643,14 @@ __global__ void k_dense_gather(int B, int64_t nb, const int32_t* __restrict__ ro
   const int64_t br = blockIdx.x;
   if (br >= nb) return;
   const int BB = B * B;
-  for (int32_t k = rowptr[br]; k < rowptr[br + 1]; ++k)
-    for (int e = threadIdx.x; e < BB; e += blockDim.x) {
-      const int ci = e / B, cj = e % B;
-      if (!FSI_IN(col[k], nb, FSI_SITE(2))) continue;
-      const int64_t r = perm[br * B + ci], c = perm[(int64_t)col[k] * B + cj];
-      if (r >= 0 && c >= 0 && FSI_IN(r, n, FSI_SITE(2)) && FSI_IN(c, n, FSI_SITE(2))) A[c * n + r] = dr[r] * val[(int64_t)k * BB + e];
-    }
+  const int64_t k0 = rowptr[br], cnt = (rowptr[br + 1] - k0) * BB;
+  for (int64_t t = threadIdx.x; t < cnt; t += blockDim.x) {
+    const int64_t k = k0 + t / BB;
+    const int e = (int)(t % BB), ci = e / B, cj = e % B;
+    if (!FSI_IN(col[k], nb, FSI_SITE(2))) continue;
+    const int64_t r = perm[br * B + ci], c = perm[(int64_t)col[k] * B + cj];
+    if (r >= 0 && c >= 0 && FSI_IN(r, n, FSI_SITE(2)) && FSI_IN(c, n, FSI_SITE(2))) A[c * n + r] = dr[r] * val[k * BB + e];
+  }
 }
 
 __global__ void k_set_diag(const int32_t* __restrict__ list, int cnt, const int32_t* __restrict__ perm, int64_t n,
@@ -548,8 +666,8 @@ void launch_dense_gather(int B, int64_t nb, const int32_t* rowptr, const int32_t
                          const int32_t* pad_list, int npad, const int32_t* perm, int64_t n, double* dr, double* A,
                          cudaStream_t st) {
   cudaMemsetAsync(A, 0, (size_t)n * n * sizeof(double), st);
-  k_coarse_row_scale<<<(unsigned)((nb * B + 127) / 128), 128, 0, st>>>(B, nb, rowptr, col, val, perm, n, dr);
-  k_dense_gather<<<(unsigned)nb, 64, 0, st>>>(B, nb, rowptr, col, val, perm, n, dr, A);
+  k_coarse_row_scale<<<(unsigned)((nb * B * 8 + 255) / 256), 256, 0, st>>>(B, nb, rowptr, col, val, perm, n, dr);
+  k_dense_gather<<<(unsigned)nb, 128, 0, st>>>(B, nb, rowptr, col, val, perm, n, dr, A);
   if (npad > 0) k_set_diag<<<(npad + 255) / 256, 256, 0, st>>>(pad_list, npad, perm, n, A);
 }
 
@@ -953,13 +1071,21 @@ __global__ void __launch_bounds__(256) k_gemv_cm_part(int64_t n, const double* _
   if (threadIdx.x < c1 - c0) xs[threadIdx.x] = (double)x[map[c0 + threadIdx.x]] * dr[c0 + threadIdx.x];
   __syncthreads();
   if (i >= n) return;
+  // all 32 loads of a full chunk in flight
   double a0 = 0.0, a1 = 0.0;
-  int64_t c = c0;
-  for (; c + 1 < c1; c += 2) {
-    a0 += A[c * n + i] * xs[c - c0];
-    a1 += A[(c + 1) * n + i] * xs[c + 1 - c0];
+  if (c1 - c0 == kGemvChunk) {
+    const double* Ai = A + c0 * n + i;
+    double v[kGemvChunk];
+#pragma unroll
+    for (int u = 0; u < kGemvChunk; ++u) v[u] = __ldg(Ai + u * n);
+#pragma unroll
+    for (int u = 0; u < kGemvChunk; u += 2) {
+      a0 = fma(v[u], xs[u], a0);
+      a1 = fma(v[u + 1], xs[u + 1], a1);
+    }
+  } else {
+    for (int64_t c = c0; c < c1; ++c) a0 = fma(A[c * n + i], xs[c - c0], a0);
   }
-  if (c < c1) a0 += A[c * n + i] * xs[c - c0];
   part[(int64_t)blockIdx.y * n + i] = a0 + a1;
 }
 
@@ -971,8 +1097,19 @@ __global__ void k_gemv_cm_sum(int64_t ni, int64_t n, int nchunk, const double* _
   const int64_t r = pos[i];
   double s = 0.0;
   if (r < 0) s = (double)x[i];
-  else
-    for (int q = 0; q < nchunk; ++q) s += part[(int64_t)q * n + r];
+  else {
+    double s1 = 0.0;
+    int q = 0;
+    for (; q + 8 <= nchunk; q += 8) {   // eight loads in flight
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = part[(int64_t)(q + u) * n + r];
+      s += (v[0] + v[1]) + (v[2] + v[3]);
+      s1 += (v[4] + v[5]) + (v[6] + v[7]);
+    }
+    for (; q < nchunk; ++q) s += part[(int64_t)q * n + r];
+    s += s1;
+  }
   y[i] = TY(s);
 }
 

@@ -68,6 +68,10 @@ void launch_arnoldi_dots(int64_t n, const double* V, int64_t ldv, int nvec, cons
                          double* partial, int nblk, cudaStream_t st);
 void launch_arnoldi_update_norm(int64_t n, const double* V, int64_t ldv, int nvec, const double* h, double* w,
                                 double* partial, int nblk, cudaStream_t st);
+// one Arnoldi step in one cooperative launch (nvec <= 32; false: not launched); partial holds
+// 3 (nvec + 1) max_blocks doubles
+bool launch_arnoldi_step(int64_t n, const double* V, int64_t ldv, int nvec, int passes, double* w, double* vnext,
+                         double* partial, int max_blocks, double* out, cudaStream_t st);
 void launch_cgs_update(int64_t n, const double* V, int64_t ldv, int nvec, const double* h, double* w, cudaStream_t st);
 void launch_combo(int64_t n, const double* Z, int64_t ldz, int nvec, const double* coef, double* x, cudaStream_t st);
 void launch_norm_partial(int64_t n, const double* w, double* partial, int nblk, cudaStream_t st);
