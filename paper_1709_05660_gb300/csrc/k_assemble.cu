@@ -543,140 +543,131 @@ __global__ void k_dirichlet(const int32_t* __restrict__ dir_list, int64_t n_dir,
 // element-wise Galerkin coarsening (2D)
 // ---------------------------------------------------------------------------
 namespace {
-// weight of parent node m at the child's local node i, child side s: the
-// 1D quadratic Lagrange basis m at the parent reference coordinate
-// -1 + (2 s + i) / 2, i.e. at -1, -1/2, 0 (s = 0) or 0, 1/2, 1 (s = 1); the
-// values are exact binary fractions, tabulated so that forming the weights
-// costs one product each and no work on the FP64 pipe beyond it
-__device__ const double kQw1[2][3][3] = {{{1.0, 0.0, 0.0}, {0.375, 0.75, -0.125}, {0.0, 1.0, 0.0}},
-                                         {{0.0, 1.0, 0.0}, {-0.125, 0.75, 0.375}, {0.0, 0.0, 1.0}}};
-// nonzero pattern of kQw1: bit (3 s + i) 3 + m
-constexpr unsigned kQwNz = (1u << 0) | (7u << 3) | (1u << 7) | (1u << 10) | (7u << 12) | (1u << 17);
-__device__ __forceinline__ bool qw_nz(int s, int i, int m) { return (kQwNz >> ((3 * s + i) * 3 + m)) & 1u; }
+// Interpolation from the parent's three 1D nodes to the child's and its
+// transpose: the weight of parent node m at the child's local node i, child side
+// s, is the 1D quadratic Lagrange basis m at the parent reference coordinate
+// -1 + (2 s + i) / 2, i.e. at -1, -1/2, 0 (s = 0) or 0, 1/2, 1 (s = 1):
+//     s = 0:  (1, 0, 0)  (3/8, 3/4, -1/8)  (0, 1, 0)
+// and s = 1 is its mirror image.  x_m = sum_i w_im x_i in place: three FP64
+// operations, the weights are exact.
+__device__ __forceinline__ void quarter_1d(double& x0, double& x1, double& x2, bool side) {
+  const double l = fma(0.375, x1, side ? x2 : x0), m = fma(0.75, x1, side ? x0 : x2), r = -0.125 * x1;
+  x0 = side ? r : l;
+  x1 = m;
+  x2 = side ? l : r;
+}
+__device__ __forceinline__ void quarter_2d(double (&v)[kNloc], int sx, int sy) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) quarter_1d(v[3 * q], v[3 * q + 1], v[3 * q + 2], sx != 0);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) quarter_1d(v[q], v[q + 3], v[q + 6], sy != 0);
+}
+// a child's pressure (value and slopes) from the parent's, direction k's half
+__device__ __forceinline__ double quarter_p(double p0, double pk, int side) {
+  return fma(0.5, pk, p0 * (side ? 0.5 : -0.5));
+}
 __device__ __forceinline__ int row_kind(int cls, int slot) {
   if (cls == kFluid) return slot < kDim ? 2 : 0;
   return slot < kDim ? 0 : 1;
 }
+constexpr int kGaLd = 44;   // row stride of T: the (row, slot) lanes' 8-byte stores hit each bank once
 }  // namespace
 
-__global__ void __launch_bounds__(256)
+// Per child: T = A_c P_c in shared memory (straight from the child's matrix),
+// then C += R_c T with C in registers.  P_c and R_c interpolate each field by the
+// tensor product of the 1D weights, so a thread takes the 9 nodal values of one
+// field of one row (column): 18 FP64 operations, every lane the same number
+// (the 25 nonzero products of the weights took lists of 1 to 4).  T is double-
+// buffered: one barrier per child.  The FP64 pipe bounds it.  The five levels
+// below 65,536 elements: 1.38 ms, 3.17 with the lists.
+__global__ void __launch_bounds__(256, 4)
 k_galerkin_2d(int ncx, int ncy, const double* __restrict__ Kf, const int32_t* __restrict__ f_nodes,
               const uint8_t* __restrict__ f_class, const uint8_t* __restrict__ f_dir,
               const int32_t* __restrict__ c_nodes, const uint8_t* __restrict__ c_class,
               const uint8_t* __restrict__ c_dir, double* __restrict__ Kc) {
-  __shared__ double sA[kNdofe * kNdofe];
-  __shared__ double sT[kNdofe * kNdofe];
-  __shared__ double sC[kNdofe * kNdofe];
-  __shared__ double wP[kNN * kNloc];        // T[i][(b,s)] = sum_a A[i][(a,s)] wP[(b,s)][a]
-  __shared__ double wR[kNN * kNloc * 2];    // C[(b,sc)][J] += sum_a sum_h wR[.][a][h] T[(a, sf_h)][J]
-  __shared__ uint8_t c_cls[kNloc], c_msk[kNN], f_cls[kNloc], f_msk[kNN];
-  // nonzero entries of each table row (zero weights cost no FP64 work; adding
-  // an exact zero would not change the sums)
-  __shared__ uint8_t nP[kNN], lP[kNN][kNloc], nR[kNN], lR[kNN][2 * kNloc];
-  __shared__ uint8_t nzP[kNN * kNloc], nzR[kNN * kNloc * 2];   // the nonzero pattern of wP and wR
-  __shared__ double sQ[2][3][3];
-  if (threadIdx.x < 18) (&sQ[0][0][0])[threadIdx.x] = (&kQw1[0][0][0])[threadIdx.x];
-  const int E = blockIdx.x;
+  __shared__ double sT[2][kNdofe * kGaLd];
+  // index 0 .. 3: the children, 4: the coarse element
+  __shared__ uint8_t msk[5][kNN], cls[5][kNloc];
+  __shared__ uint8_t row[5][3][kDim][kNloc];   // row (a, slot) of a kind and component, 255: none (or Dirichlet)
+  __shared__ int s_kinds;
+  const int E = blockIdx.x, tid = threadIdx.x;
   const int cx = E % ncx, cy = E / ncx;
   const int fcx = 2 * ncx;
-  for (int t = threadIdx.x; t < kNdofe * kNdofe; t += blockDim.x) sC[t] = 0.0;
-  if (threadIdx.x < kNloc) c_cls[threadIdx.x] = c_class[c_nodes[(int64_t)E * kNloc + threadIdx.x]];
-  if (threadIdx.x < kNN) {
-    const int a = threadIdx.x / kB, s = threadIdx.x % kB;
-    c_msk[threadIdx.x] = c_dir[(int64_t)c_nodes[(int64_t)E * kNloc + a] * kB + s] ? 0 : 1;
-  }
-  for (int ch = 0; ch < 4; ++ch) {
-    const int sx = ch & 1, sy = ch >> 1;
-    const int64_t ef = (2 * cx + sx) + (int64_t)fcx * (2 * cy + sy);
-    __syncthreads();
-    for (int t = threadIdx.x; t < kNdofe * kNdofe; t += blockDim.x) sA[t] = Kf[ef * kNdofe * kNdofe + t];
-    if (threadIdx.x < kNloc) f_cls[threadIdx.x] = f_class[f_nodes[ef * kNloc + threadIdx.x]];
-    if (threadIdx.x < kNN) {
-      const int a = threadIdx.x / kB, s = threadIdx.x % kB;
-      f_msk[threadIdx.x] = f_dir[(int64_t)f_nodes[ef * kNloc + a] * kB + s] ? 0 : 1;
-    }
-    __syncthreads();
-    // weight tables of this child: coarse basis b at the child's node a
-    for (int t = threadIdx.x; t < kNN * kNloc; t += blockDim.x) {
-      const int J = t / kNloc, a = t % kNloc;        // J = (b, s)
-      const int b = J / kB, sl = J % kB;
-      const int ax = a % 3, ay = a / 3, bx = b % 3, by = b / 3;
-      const bool nq = qw_nz(sx, ax, bx) && qw_nz(sy, ay, by);
-      const double q = nq ? sQ[sx][ax][bx] * sQ[sy][ay][by] : 0.0;
-      const bool mp = nq && c_msk[J] && f_msk[a * kB + sl];
-      wP[t] = mp ? q : 0.0;
-      nzP[t] = mp;
-      const int comp = sl % kDim;
-      const int kc = row_kind(c_cls[b], sl);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int sf = h == 0 ? comp : kDim + comp;
-        const bool mr = nq && c_msk[J] && f_msk[a * kB + sf] && row_kind(f_cls[a], sf) == kc;
-        wR[t * 2 + h] = mr ? q : 0.0;
-        nzR[t * 2 + h] = mr;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x < kNN) {
-      const int J = threadIdx.x;
-      int np = 0, nq = 0;
-      for (int a = 0; a < kNloc; ++a) {
-        if (nzP[J * kNloc + a]) lP[J][np++] = (uint8_t)a;
-        for (int h = 0; h < 2; ++h)
-          if (nzR[(J * kNloc + a) * 2 + h]) lR[J][nq++] = (uint8_t)(2 * a + h);
-      }
-      nP[J] = (uint8_t)np;
-      nR[J] = (uint8_t)nq;
-    }
-    __syncthreads();
-    // T = A_c P_c
-    for (int t = threadIdx.x; t < kNdofe * kNdofe; t += blockDim.x) {
-      const int i = t / kNdofe, J = t % kNdofe;
-      const double* Ai = sA + i * kNdofe;
-      double acc = 0.0;
-      if (J < kNN) {
-        const int sl = J % kB;
-        const double* w = wP + J * kNloc;
-        for (int q = 0; q < nP[J]; ++q) {
-          const int a = lP[J][q];
-          acc += Ai[a * kB + sl] * w[a];
-        }
-      } else {
-        const int k = J - kNN;
-        // child coefficients: c0 = p0 + sum_d sig_d/2 p_d ; c_d = p_d / 2
-        if (k == 0) acc = Ai[kNN];
-        else {
-          const double sig = k == 1 ? (sx ? 0.5 : -0.5) : (sy ? 0.5 : -0.5);
-          acc = Ai[kNN] * sig + Ai[kNN + k] * 0.5;
-        }
-      }
-      sT[t] = acc;
-    }
-    __syncthreads();
-    // C += R_c T
-    for (int t = threadIdx.x; t < kNdofe * kNdofe; t += blockDim.x) {
-      const int I = t / kNdofe, J = t % kNdofe;
-      double acc = 0.0;
-      if (I < kNN) {
-        const int comp = (I % kB) % kDim;
-        const double* w = wR + I * kNloc * 2;
-        for (int q = 0; q < nR[I]; ++q) {
-          const int ah = lR[I][q], a = ah >> 1, h = ah & 1;
-          acc += w[ah] * sT[(a * kB + h * kDim + comp) * kNdofe + J];
-        }
-      } else {
-        const int k = I - kNN;
-        if (k == 0) acc = sT[kNN * kNdofe + J];
-        else {
-          const double sig = k == 1 ? (sx ? 0.5 : -0.5) : (sy ? 0.5 : -0.5);
-          acc = sT[kNN * kNdofe + J] * sig + sT[(kNN + k) * kNdofe + J] * 0.5;
-        }
-      }
-      sC[t] += acc;
-    }
+  auto child = [&](int ch) { return (2 * cx + (ch & 1)) + (int64_t)fcx * (2 * cy + (ch >> 1)); };
+  if (tid == 0) s_kinds = 0;
+  for (int t = tid; t < 5 * kNN; t += blockDim.x) {
+    const int w = t / kNN, a = t % kNN / kB, s = t % kB;
+    const int32_t nd = w == 4 ? c_nodes[(int64_t)E * kNloc + a] : f_nodes[child(w) * kNloc + a];
+    msk[w][t % kNN] = (w == 4 ? c_dir : f_dir)[(int64_t)nd * kB + s] ? 0 : 1;
+    if (s == 0) cls[w][a] = (w == 4 ? c_class : f_class)[nd];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < kNdofe * kNdofe; t += blockDim.x) Kc[(int64_t)E * kNdofe * kNdofe + t] = sC[t];
+  for (int t = tid; t < 5 * 3 * kDim * kNloc; t += blockDim.x) {
+    const int a = t % kNloc, c = t / kNloc % kDim, kind = t / (kNloc * kDim) % 3, w = t / (kNloc * kDim * 3);
+    const int sl = row_kind(cls[w][a], c) == kind ? c : (row_kind(cls[w][a], kDim + c) == kind ? kDim + c : -1);
+    const bool ok = sl >= 0 && msk[w][a * kB + sl];
+    row[w][kind][c][a] = (uint8_t)(ok ? a * kB + sl : 255);
+    if (w == 4 && ok) atomicOr(&s_kinds, 1 << kind);
+  }
+  __syncthreads();
+  // C += R T: thread (kind, component, J) for the unknowns, (k, J) from the other
+  // end for the pressures
+  const int kinds = s_kinds;
+  const int J = tid % kNdofe, c = tid / kNdofe % kDim, w = tid / (kNdofe * kDim);
+  int kind = 0;
+  for (int n = 0; kind < 3; ++kind)
+    if ((kinds >> kind) & 1 && n++ == w) break;
+  const bool unk = w < 3 && kind < 3;
+  const int pt = (int)blockDim.x - 1 - tid, pi = pt / 3, pk = pt % 3;   // T's pressure columns: row pi
+  const int pJ = pt % kNdofe, pc = pt / kNdofe;                         // C's pressure rows: row pc
+  const bool press = pt < 3 * kNdofe;
+  double acc[kNloc], pacc = 0.0;
+#pragma unroll
+  for (int b = 0; b < kNloc; ++b) acc[b] = 0.0;
+  for (int ch = 0; ch < 4; ++ch) {
+    const int sx = ch & 1, sy = ch >> 1;
+    const double* A = Kf + child(ch) * kNdofe * kNdofe;
+    double* T = sT[ch & 1];
+    if (tid < kNdofe * kB) {   // T = A P: thread (i, slot)
+      const int i = tid / kB, sl = tid % kB;
+      double v[kNloc];
+#pragma unroll
+      for (int a = 0; a < kNloc; ++a) v[a] = msk[ch][a * kB + sl] ? __ldg(A + i * kNdofe + a * kB + sl) : 0.0;
+      quarter_2d(v, sx, sy);
+#pragma unroll
+      for (int b = 0; b < kNloc; ++b) T[i * kGaLd + b * kB + sl] = msk[4][b * kB + sl] ? v[b] : 0.0;
+    }
+    if (press) {
+      const double* p = A + pi * kNdofe + kNN;
+      T[pi * kGaLd + kNN + pk] = pk == 0 ? p[0] : quarter_p(p[0], p[pk], pk == 1 ? sx : sy);
+    }
+    __syncthreads();
+    if (unk) {
+      double v[kNloc];
+#pragma unroll
+      for (int a = 0; a < kNloc; ++a) {
+        const int r = row[ch][kind][c][a];
+        v[a] = r != 255 ? T[r * kGaLd + J] : 0.0;
+      }
+      quarter_2d(v, sx, sy);
+#pragma unroll
+      for (int b = 0; b < kNloc; ++b) acc[b] += v[b];
+    }
+    if (press) {
+      const double p0 = T[kNN * kGaLd + pJ];
+      pacc += pc == 0 ? p0 : quarter_p(p0, T[(kNN + pc) * kGaLd + pJ], pc == 1 ? sx : sy);
+    }
+  }
+  double* C = Kc + (int64_t)E * kNdofe * kNdofe;
+  if (unk)
+#pragma unroll
+    for (int b = 0; b < kNloc; ++b) {
+      const int r = row[4][kind][c][b];
+      if (r != 255) C[r * kNdofe + J] = acc[b];
+    }
+  if (press) C[(kNN + pc) * kNdofe + pJ] = pacc;
+  for (int t = tid; t < kNN * kNdofe; t += blockDim.x)   // Dirichlet rows
+    if (!msk[4][t / kNdofe]) C[t] = 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -1288,14 +1279,31 @@ k_assemble_3d(const int32_t* __restrict__ elems, const int32_t* __restrict__ ele
   }
 }
 
-// Element-wise Galerkin coarsening in 3D.  Per child: T = A_c P_c is formed
-// in shared memory from the child's matrix (global, row-major), then the
-// coarse element matrix (global, accumulated over the 8 children) gets
-// R_c T.  The interpolation weights of a child are products of 1D
-// quarter-point weights; each coarse node b keeps the compact list of the
-// child nodes a with a nonzero weight (125 of the 27 x 27 pairs), built from
-// an 18-entry 1D table, so no FP64 work is spent on zero weights.
+// Element-wise Galerkin coarsening in 3D.  Per child: T = A_c P_c is formed in
+// shared memory from the child's matrix (global, row-major), then the coarse
+// element matrix (global, accumulated over the 8 children) gets R_c T.  P_c and
+// R_c interpolate each of the fields by the tensor product of the 1D table, so a
+// thread takes the 27 nodal values of one field of one row (column) in registers
+// and applies the three 1D interpolations in turn: 81 FP64 operations, against
+// 125 for the nonzero products of the three tables, and every lane the same
+// number of them.  FP64 and the loads ahead of it bound it (one block of 512
+// threads per SM: T takes the shared memory).  The two coarse
+// levels below 900,000 unknowns: 9.2 ms, 21.1 with lists of the nonzero products.
 size_t galerkin_3d_smem() { return (size_t)k3Ndofe * k3Ndofe * sizeof(double); }
+
+namespace {
+__device__ __forceinline__ void quarter_3d(double (&v)[k3Nloc], int sx, int sy, int sz) {
+#pragma unroll
+  for (int q = 0; q < 9; ++q) quarter_1d(v[3 * q], v[3 * q + 1], v[3 * q + 2], sx != 0);
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    const int o = q / 3 * 9 + q % 3;
+    quarter_1d(v[o], v[o + 3], v[o + 6], sy != 0);
+  }
+#pragma unroll
+  for (int q = 0; q < 9; ++q) quarter_1d(v[q], v[q + 9], v[q + 18], sz != 0);
+}
+}  // namespace
 
 __global__ void __launch_bounds__(512)
 k_galerkin_3d(int ncx, int ncy, int ncz, const double* __restrict__ Kf, const int32_t* __restrict__ f_nodes,
@@ -1304,122 +1312,87 @@ k_galerkin_3d(int ncx, int ncy, int ncz, const double* __restrict__ Kf, const in
               const uint8_t* __restrict__ c_dir, double* __restrict__ Kc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* T = reinterpret_cast<double*>(smem_raw);   // [i][J]
-  __shared__ double w1[2][3][3];                     // [side][fine 1D][coarse 1D]
-  __shared__ double l_w[125];
-  __shared__ uint8_t l_a[125];
-  __shared__ int l_ptr[k3Nloc + 1];
-  __shared__ uint8_t c_cls[k3Nloc], c_msk[k3NN], f_cls[k3Nloc], f_msk[k3NN];
+  // row (a, slot) of a row kind and component at a node, 255: none (another
+  // kind, or a Dirichlet row)
+  __shared__ uint8_t f_row[3][k3Dim][k3Nloc], c_row[3][k3Dim][k3Nloc];
+  __shared__ uint8_t c_msk[k3NN], f_msk[k3NN];
+  __shared__ int s_kinds;
   const int E = blockIdx.x;
   const int cx = E % ncx, cy = (E / ncx) % ncy, cz = E / (ncx * ncy);
   const int fcx = 2 * ncx, fcy = 2 * ncy;
   (void)ncz;
   double* C = Kc + (int64_t)E * k3Ndofe * k3Ndofe;
   for (int t = threadIdx.x; t < k3Ndofe * k3Ndofe; t += blockDim.x) C[t] = 0.0;
-  if (threadIdx.x < 18) (&w1[0][0][0])[threadIdx.x] = (&kQw1[0][0][0])[threadIdx.x];
-  if (threadIdx.x < k3Nloc) c_cls[threadIdx.x] = c_class[c_nodes[(int64_t)E * k3Nloc + threadIdx.x]];
-  if (threadIdx.x < k3NN) {
-    const int a = threadIdx.x / k3B, s = threadIdx.x % k3B;
-    c_msk[threadIdx.x] = c_dir[(int64_t)c_nodes[(int64_t)E * k3Nloc + a] * k3B + s] ? 0 : 1;
-  }
+  if (threadIdx.x == 0) s_kinds = 0;
+  __syncthreads();
+  // per node, kind and component: each kind has at most one slot there
+  auto row_of = [](const uint8_t* msk, int cls, int kind, int c, int a) {
+    const int sl = row_kind3(cls, c) == kind ? c : (row_kind3(cls, k3Dim + c) == kind ? k3Dim + c : -1);
+    return (uint8_t)(sl >= 0 && msk[a * k3B + sl] ? a * k3B + sl : 255);
+  };
+  auto tables = [&](const int32_t* nodes, const uint8_t* cls, const uint8_t* dir, uint8_t* msk,
+                    uint8_t (&row)[3][k3Dim][k3Nloc], bool coarse) {
+    if (threadIdx.x < k3NN)
+      msk[threadIdx.x] = dir[(int64_t)nodes[threadIdx.x / k3B] * k3B + threadIdx.x % k3B] ? 0 : 1;
+    __syncthreads();
+    if (threadIdx.x < 3 * k3NN / 2) {
+      const int a = threadIdx.x % k3Nloc, c = threadIdx.x / k3Nloc % k3Dim, kind = threadIdx.x / (k3Nloc * k3Dim);
+      row[kind][c][a] = row_of(msk, cls[nodes[a]], kind, c, a);
+      if (coarse && row[kind][c][a] != 255) atomicOr(&s_kinds, 1 << kind);
+    }
+    __syncthreads();
+  };
+  tables(c_nodes + (int64_t)E * k3Nloc, c_class, c_dir, c_msk, c_row, true);
+  const int kinds = s_kinds, nk = __popc(kinds);
   for (int ch = 0; ch < 8; ++ch) {
     const int sx = ch & 1, sy = (ch >> 1) & 1, sz = ch >> 2;
     const int64_t ef = (2 * cx + sx) + (int64_t)fcx * ((2 * cy + sy) + (int64_t)fcy * (2 * cz + sz));
     const double* A = Kf + ef * k3Ndofe * k3Ndofe;
-    __syncthreads();
-    if (threadIdx.x < k3Nloc) f_cls[threadIdx.x] = f_class[f_nodes[ef * k3Nloc + threadIdx.x]];
-    if (threadIdx.x < k3NN) {
-      const int a = threadIdx.x / k3B, s = threadIdx.x % k3B;
-      f_msk[threadIdx.x] = f_dir[(int64_t)f_nodes[ef * k3Nloc + a] * k3B + s] ? 0 : 1;
-    }
-    // nonzero pattern of the child's weights: count per coarse node
-    if (threadIdx.x < k3Nloc) {
-      const int b = threadIdx.x, mx = b % 3, my = (b / 3) % 3, mz = b / 9;
-      int n = 1;
-      const int sd[3] = {sx, sy, sz}, mm[3] = {mx, my, mz};
-      for (int d = 0; d < 3; ++d) {
-        int c = 0;
-        for (int i = 0; i < 3; ++i) c += w1[sd[d]][i][mm[d]] != 0.0;
-        n *= c;
-      }
-      l_ptr[b + 1] = n;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      l_ptr[0] = 0;
-      for (int b = 0; b < k3Nloc; ++b) l_ptr[b + 1] += l_ptr[b];
-    }
-    __syncthreads();
-    if (threadIdx.x < k3Nloc) {
-      const int b = threadIdx.x, mx = b % 3, my = (b / 3) % 3, mz = b / 9;
-      int q = l_ptr[b];
-      for (int iz = 0; iz < 3; ++iz) {
-        const double wz = w1[sz][iz][mz];
-        if (wz == 0.0) continue;
-        for (int iy = 0; iy < 3; ++iy) {
-          const double wy = w1[sy][iy][my];
-          if (wy == 0.0) continue;
-          for (int ix = 0; ix < 3; ++ix) {
-            const double wx = w1[sx][ix][mx];
-            if (wx == 0.0) continue;
-            l_a[q] = (uint8_t)(ix + 3 * iy + 9 * iz);
-            l_w[q] = wx * wy * wz;
-            ++q;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // T = A P  (J fastest: coalesced reads of A's row i)
-    for (int t = threadIdx.x; t < k3Ndofe * k3Ndofe; t += blockDim.x) {
-      const int i = t / k3Ndofe, J = t % k3Ndofe;
-      const double* Ai = A + (int64_t)i * k3Ndofe;
-      double acc = 0.0;
-      if (J < k3NN) {
-        const int b = J / k3B, sl = J % k3B;
-        if (c_msk[J])
-          for (int q = l_ptr[b]; q < l_ptr[b + 1]; ++q) {
-            const int a = l_a[q];
-            if (f_msk[a * k3B + sl]) acc += Ai[a * k3B + sl] * l_w[q];
-          }
-      } else {
-        const int k = J - k3NN;
-        if (k == 0) acc = Ai[k3NN];
-        else {
-          const int sd = k == 1 ? sx : (k == 2 ? sy : sz);
-          acc = Ai[k3NN] * (sd ? 0.5 : -0.5) + Ai[k3NN + k] * 0.5;
-        }
-      }
-      T[t] = acc;
-    }
-    __syncthreads();
-    // C += R T  (row I uniform across a warp: uniform lists and masks)
-    for (int t = threadIdx.x; t < k3Ndofe * k3Ndofe; t += blockDim.x) {
-      const int I = t / k3Ndofe, J = t % k3Ndofe;
-      double acc = 0.0;
-      if (I < k3NN) {
-        const int b = I / k3B, sc = I % k3B;
-        if (c_msk[I]) {
-          const int comp = sc % k3Dim;
-          const int kc = row_kind3(c_cls[b], sc);
-          for (int q = l_ptr[b]; q < l_ptr[b + 1]; ++q) {
-            const int a = l_a[q];
+    tables(f_nodes + ef * k3Nloc, f_class, f_dir, f_msk, f_row, false);
+    // T = A P: thread (i, slot)
+    for (int t = threadIdx.x; t < k3Ndofe * k3B; t += blockDim.x) {
+      const int i = t / k3B, sl = t % k3B;
+      const double* Ai = A + (int64_t)i * k3Ndofe + sl;
+      double v[k3Nloc];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int sf = h == 0 ? comp : k3Dim + comp;
-              if (f_msk[a * k3B + sf] && row_kind3(f_cls[a], sf) == kc) acc += l_w[q] * T[(a * k3B + sf) * k3Ndofe + J];
-            }
-          }
-        }
-      } else {
-        const int k = I - k3NN;
-        if (k == 0) acc = T[k3NN * k3Ndofe + J];
-        else {
-          const int sd = k == 1 ? sx : (k == 2 ? sy : sz);
-          acc = T[k3NN * k3Ndofe + J] * (sd ? 0.5 : -0.5) + T[(k3NN + k) * k3Ndofe + J] * 0.5;
-        }
-      }
-      C[t] += acc;
+      for (int a = 0; a < k3Nloc; ++a) v[a] = f_msk[a * k3B + sl] ? __ldg(Ai + a * k3B) : 0.0;
+      quarter_3d(v, sx, sy, sz);
+      double* Ti = T + i * k3Ndofe + sl;
+#pragma unroll
+      for (int b = 0; b < k3Nloc; ++b) Ti[b * k3B] = c_msk[b * k3B + sl] ? v[b] : 0.0;
     }
+    for (int t = threadIdx.x; t < k3Ndofe * 4; t += blockDim.x) {
+      const int i = t / 4, k = t % 4;
+      const double* Ai = A + (int64_t)i * k3Ndofe + k3NN;
+      T[i * k3Ndofe + k3NN + k] = k == 0 ? Ai[0] : quarter_p(Ai[0], Ai[k], k == 1 ? sx : (k == 2 ? sy : sz));
+    }
+    __syncthreads();
+    // C += R T: thread (kind, component, J); each row of C has one kind
+    for (int t = threadIdx.x; t < nk * k3Dim * k3Ndofe; t += blockDim.x) {
+      const int J = t % k3Ndofe, c = t / k3Ndofe % k3Dim, w = t / (k3Ndofe * k3Dim);
+      int kind = 0;
+      for (int n = 0; kind < 3; ++kind)
+        if ((kinds >> kind) & 1 && n++ == w) break;
+      double v[k3Nloc];
+#pragma unroll
+      for (int a = 0; a < k3Nloc; ++a) {
+        const int r = f_row[kind][c][a];
+        v[a] = r != 255 ? T[r * k3Ndofe + J] : 0.0;
+      }
+      quarter_3d(v, sx, sy, sz);
+#pragma unroll
+      for (int b = 0; b < k3Nloc; ++b) {
+        const int r = c_row[kind][c][b];
+        if (r != 255) C[r * k3Ndofe + J] += v[b];
+      }
+    }
+    for (int t = threadIdx.x; t < 4 * k3Ndofe; t += blockDim.x) {
+      const int k = t / k3Ndofe, J = t % k3Ndofe;
+      const double p0 = T[k3NN * k3Ndofe + J];
+      C[(k3NN + k) * k3Ndofe + J] +=
+          k == 0 ? p0 : quarter_p(p0, T[(k3NN + k) * k3Ndofe + J], k == 1 ? sx : (k == 2 ? sy : sz));
+    }
+    __syncthreads();   // T is free again
   }
 }
 
@@ -1575,10 +1548,15 @@ double assemble_flops_per_element(int dim, bool solid, int mode) {
   mode = mode < 0 ? 0 : (mode > 2 ? 2 : mode);
   return dim == 2 ? f2[solid][mode] : f3[solid][mode];
 }
-// the same count for the Galerkin kernels, per coarse element (2D: the
-// 5-level channel's finest coarsening, 4,096 coarse elements, with the
-// tabulated child weights)
-double galerkin_flops_per_coarse_element(int dim) { return dim == 2 ? 69340.0 : 3030039.0; }
+// the same count for the Galerkin kernels, per coarse element away from the
+// fluid-solid interface, from their loops: 1D interpolations of 5 operations, the
+// sums over the children and the pressures
+double galerkin_flops_per_coarse_element(int dim) {
+  const double rows = dim == 2 ? kNdofe : k3Ndofe, fields = dim == 2 ? kB : k3B, nodes = dim == 2 ? kNloc : k3Nloc;
+  const double line = dim == 2 ? 6 * 5 : 27 * 5;   // of one field's values
+  const double child = rows * fields * (2 * line + nodes) + rows * (dim * 3 + 1 + dim * 4);
+  return (dim == 2 ? 4 : 8) * child;
+}
 
 int assemble_launches(int dim, int ne) { return dim == 2 || ne <= 0 ? (ne > 0) : 2 * ((ne + k3Chunk - 1) / k3Chunk); }
 
