@@ -407,46 +407,48 @@ void launch_slab_gemm(const SlabGemm* g, int n, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 namespace {
 constexpr int kSvThreads = 512;
-constexpr int kSvRows = 16;                            // rows of a thread block's product
-constexpr int kSvCols = kSvThreads / kSvRows;          // columns in flight
+constexpr int kSvMinRows = 4;                          // rows of a thread block's part of a product (a sector)
+constexpr int kSvAhead = 16;                           // matrix entries per thread loaded ahead of the barrier
 
-// out[r0 + r] = beta y[r0 + r] + alpha sum_c A[(r0 + r) + c lda] x[c] for the
-// kSvRows rows of a thread block (the rows < nr): lanes over rows, column groups
-// over the threads, summed in a fixed order.  x is read through L2: other
-// blocks wrote it before the last grid barrier.
-__device__ __forceinline__ void block_gemv(const double* __restrict__ A, int64_t lda, int r0, int nr, int nc,
-                                           const double* x, double alpha, double beta, const double* y, double* out,
-                                           double* red) {
-  const int r = threadIdx.x % kSvRows, cgp = threadIdx.x / kSvRows;
-  const bool ok = r0 + r < nr;
-  const double* Ar = A + (ok ? r0 + r : 0);
-  double s0 = 0.0, s1 = 0.0;
-  int c = cgp;
-#pragma unroll 4
-  for (; c + kSvCols < nc; c += 2 * kSvCols) {
-    s0 = fma(__ldg(Ar + (int64_t)c * lda), __ldcg(x + c), s0);
-    s1 = fma(__ldg(Ar + (int64_t)(c + kSvCols) * lda), __ldcg(x + c + kSvCols), s1);
+// out = beta y + alpha A x, rows [0, nr) over `nb` thread blocks
+struct SvGemv {
+  const double* A;
+  int64_t lda;
+  int nr, nc, b, nb;
+  const double* x;
+  double alpha, beta;
+  const double* y;
+  double* out;
+};
+
+// A thread block's part of a product: rows [r0, r0 + rb), rb = ceil(nr / nb).
+// Threads over rows, then column groups; their sums are added in a fixed order.
+struct SvPart {
+  int rb, r0, cnt, ng, r, g;
+  const double* col;   // entry (r0 + r, g)
+  __device__ explicit SvPart(const SvGemv& j) {
+    rb = max(kSvMinRows, (j.nr + j.nb - 1) / j.nb);
+    r0 = j.b * rb;
+    cnt = min(rb, j.nr - r0);
+    ng = kSvThreads / rb;
+    r = threadIdx.x % rb;
+    g = threadIdx.x / rb;
+    if (r >= cnt) g = j.nc;   // no columns
+    col = j.A + (r0 + r) + (int64_t)g * j.lda;
   }
-  if (c < nc) s0 = fma(__ldg(Ar + (int64_t)c * lda), __ldcg(x + c), s0);
-  red[cgp * kSvRows + r] = s0 + s1;
-  __syncthreads();
-  if (threadIdx.x < kSvRows && ok) {
-    double s = 0.0;
-    for (int q = 0; q < kSvCols; ++q) s += red[q * kSvRows + threadIdx.x];
-    const double b = beta == 0.0 ? 0.0 : beta * __ldcg(y + r0 + r);
-    __stcg(out + r0 + r, fma(alpha, s, b));
-  }
-  __syncthreads();
-}
+};
 }  // namespace
 
 // x = A^{-1} b over the slab ordering (b in w, overwritten; x in x): elimination
-// from both ends, the middle slab, back substitution to both ends; each step is
+// from both ends, the middle slab, back substitution to both ends; each stage is
 // a product over the thread blocks followed by a grid barrier, the left
-// side's on the even blocks and the right side's on the odd ones.  Two products
-// per slab and direction; a step is bound by the barrier and one L2 round
-// trip (about 2.5 us) rather than by its 3.4 MB of matrix, so it is one launch
-// instead of 134: 0.4 ms against 1.5 for the 16 slabs of 652 unknowns.
+// side's on the even blocks and the right side's on the odd ones, two products
+// per slab and direction, in one launch.  A stage is a chain (barrier, x from
+// L2, products, sums), so the matrix, which no stage changes, is loaded a stage
+// ahead, the rows are spread over all blocks, and the column sums are added by 16
+// lanes a row.  16 slabs of 652 unknowns (33 stages): 0.25 ms a solve; 0.41 with 16
+// rows to a block (half of the SMs), 0.27 with the loads just before the
+// barrier, 1.5 as 134 launches.
 __global__ void __launch_bounds__(kSvThreads) k_slab_solve(SlabChain ch, const double* __restrict__ A, int64_t n,
                                                            const double* __restrict__ sinv, double* w, double* x,
                                                            double* u) {
@@ -458,71 +460,112 @@ __global__ void __launch_bounds__(kSvThreads) k_slab_solve(SlabChain ch, const d
   auto off = [&](int k) { return (int64_t)ch.off[k]; };
   auto len = [&](int k) { return ch.off[k + 1] - ch.off[k]; };
   auto inv = [&](int k) { return sinv + ch.inv[k]; };
-  // rows [0, nr) of a product over the blocks of one side
-  auto rows = [&](int nr, auto&& f) {
-    for (int r0 = b0 * kSvRows; r0 < nr; r0 += nbk * kSvRows) f(r0);
-  };
   const int steps = max(mid, K - 1 - mid);
-  for (int s = 0; s < steps; ++s) {
-    const int kl = s + 1, kr = K - 2 - s;   // slabs that take a correction
-    if (side == 0 && kl <= mid) {
-      const int m = len(kl - 1);            // u = S_{kl-1}^{-1}[P,:] w_{kl-1}
-      rows(p, [&](int r0) { block_gemv(inv(kl - 1) + (m - p), m, r0, p, m, w + off(kl - 1), 1.0, 0.0, us, us, red); });
+  // both sides correct the middle slab in the last step: the right one in a stage of its own
+  const int clash = mid > 0 && mid == K - 1 - mid ? 1 : 0;
+  const int fwd = 2 * steps + clash, total = fwd + 1 + 2 * steps;
+  // this block's side's product of stage i (nr = 0: none)
+  auto stage = [&](int i) {
+    SvGemv j{A, n, 0, 0, b0, nbk, w, 1.0, 0.0, w, w};
+    if (i < fwd) {
+      const int s = min(i / 2, steps - 1), ph = i - 2 * s;
+      const int kl = s + 1, kr = K - 2 - s;   // slabs that take a correction
+      const bool apart = clash && s == steps - 1;
+      if (side == 0 && kl <= mid) {
+        if (ph == 0) {                        // u = S_{kl-1}^{-1}[P,:] w_{kl-1}
+          const int m = len(kl - 1);
+          j = SvGemv{inv(kl - 1) + (m - p), m, p, m, b0, nbk, w + off(kl - 1), 1.0, 0.0, us, us};
+        } else if (ph == 1) {                 // w_kl -= A_{kl,kl-1}[:,P] u
+          j = SvGemv{A + (off(kl) - p) * n + off(kl), n, len(kl), p, b0, nbk, us, -1.0, 1.0, w + off(kl), w + off(kl)};
+        }
+      }
+      if (side == 1 && kr >= mid) {
+        const int m = len(kr + 1);
+        if (ph == 0) {                        // u = S_{kr+1}^{-1} w_{kr+1}
+          j = SvGemv{inv(kr + 1), m, m, m, b0, nbk, w + off(kr + 1), 1.0, 0.0, us, us};
+        } else if (ph == (apart ? 2 : 1)) {   // w_kr[P] -= A_{kr,kr+1}[P,:] u
+          const int64_t o = off(kr + 1) - p;
+          j = SvGemv{A + off(kr + 1) * n + o, n, p, m, b0, nbk, us, -1.0, 1.0, w + o, w + o};
+        }
+      }
+    } else if (i == fwd) {                    // the middle slab, over the blocks of both sides
+      const int m = len(mid);
+      j = SvGemv{inv(mid), m, m, m, (int)blockIdx.x, (int)gridDim.x, w + off(mid), 1.0, 0.0, x + off(mid), x + off(mid)};
+    } else if (i < total) {
+      const int s = (i - fwd - 1) / 2, ph = (i - fwd - 1) % 2;
+      const int k = side == 0 ? mid - 1 - s : mid + 1 + s;
+      if (k >= 0 && k < K) {
+        const int m = len(k);
+        if (ph == 1) {
+          j = SvGemv{inv(k), m, m, m, b0, nbk, w + off(k), 1.0, 0.0, x + off(k), x + off(k)};
+        } else if (side == 0) {               // w_k[P] -= A_{k,k+1}[P,:] x_{k+1}
+          const int64_t o = off(k + 1) - p;
+          j = SvGemv{A + off(k + 1) * n + o, n, p, len(k + 1), b0, nbk, x + off(k + 1), -1.0, 1.0, w + o, w + o};
+        } else {                              // w_k -= A_{k,k-1}[:,P] x_{k-1}[P]
+          j = SvGemv{A + (off(k) - p) * n + off(k), n, m, p, b0, nbk, x + off(k) - p, -1.0, 1.0, w + off(k), w + off(k)};
+        }
+      }
     }
-    if (side == 1 && kr >= mid) {
-      const int m = len(kr + 1);            // u = S_{kr+1}^{-1} w_{kr+1}
-      rows(m, [&](int r0) { block_gemv(inv(kr + 1), m, r0, m, m, w + off(kr + 1), 1.0, 0.0, us, us, red); });
+    return j;
+  };
+  auto ahead = [&](const SvGemv& j, double (&v)[kSvAhead]) {
+    const SvPart t(j);
+#pragma unroll
+    for (int q = 0; q < kSvAhead; ++q)
+      v[q] = t.g < t.ng && t.g + q * t.ng < j.nc ? __ldg(t.col + (int64_t)q * t.ng * j.lda) : 0.0;
+  };
+  double a[kSvAhead], an[kSvAhead];
+  SvGemv j = stage(0);
+  ahead(j, a);
+  for (int i = 0; i < total; ++i) {
+    const SvGemv jn = stage(i + 1);
+    ahead(jn, an);
+    const SvPart t(j);
+    if (t.cnt > 0) {
+      double s = 0.0;
+      if (t.g < t.ng) {
+        double xv[kSvAhead];
+#pragma unroll
+        for (int q = 0; q < kSvAhead; ++q) {
+          const int c = t.g + q * t.ng;
+          xv[q] = c < j.nc ? __ldcg(j.x + c) : 0.0;
+        }
+        double s1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < kSvAhead; q += 2) {
+          if (t.g + q * t.ng < j.nc) s = fma(a[q], xv[q], s);
+          if (t.g + (q + 1) * t.ng < j.nc) s1 = fma(a[q + 1], xv[q + 1], s1);
+        }
+        for (int c = t.g + kSvAhead * t.ng; c < j.nc; c += t.ng)
+          s = fma(__ldg(t.col + (int64_t)(c - t.g) * j.lda), __ldcg(j.x + c), s);
+        s += s1;
+      }
+      red[threadIdx.x] = s;
+      __syncthreads();
+      for (int e0 = threadIdx.x / 32 * 32; e0 < t.rb * 16; e0 += kSvThreads) {   // 16 lanes a row
+        const int e = e0 + threadIdx.x % 32, r = e / 16;
+        double v = 0.0;
+        if (r < t.cnt)
+          for (int g = e % 16; g < t.ng; g += 16) v += red[g * t.rb + r];
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (e % 16 == 0 && r < t.cnt) {
+          const double b = j.beta == 0.0 ? 0.0 : j.beta * __ldcg(j.y + t.r0 + r);
+          __stcg(j.out + t.r0 + r, fma(j.alpha, v, b));
+        }
+      }
     }
+    if (i + 1 == total) break;
     grid.sync();
-    // both sides correct the middle slab: the right one in the step's second half
-    const bool clash = kl == mid && kr == mid;
-    if (side == 0 && kl <= mid) {
-      const int m = len(kl);                // w_kl -= A_{kl,kl-1}[:,P] u
-      const double* B = A + (off(kl) - p) * n + off(kl);
-      rows(m, [&](int r0) { block_gemv(B, n, r0, m, p, us, -1.0, 1.0, w + off(kl), w + off(kl), red); });
-    }
-    if (clash) grid.sync();
-    if (side == 1 && kr >= mid) {
-      const int64_t o = off(kr + 1) - p;    // w_kr[P] -= A_{kr,kr+1}[P,:] u
-      rows(p, [&](int r0) {
-        block_gemv(A + off(kr + 1) * n + o, n, r0, p, len(kr + 1), us, -1.0, 1.0, w + o, w + o, red);
-      });
-    }
-    grid.sync();
-  }
-  {
-    const int m = len(mid);
-    for (int r0 = blockIdx.x * kSvRows; r0 < m; r0 += gridDim.x * kSvRows)
-      block_gemv(inv(mid), m, r0, m, m, w + off(mid), 1.0, 0.0, x + off(mid), x + off(mid), red);
-  }
-  grid.sync();
-  for (int s = 0; s < steps; ++s) {
-    const int kl = mid - 1 - s, kr = mid + 1 + s;
-    if (side == 0 && kl >= 0) {
-      const int64_t o = off(kl + 1) - p;    // w_kl[P] -= A_{kl,kl+1}[P,:] x_{kl+1}
-      rows(p, [&](int r0) {
-        block_gemv(A + off(kl + 1) * n + o, n, r0, p, len(kl + 1), x + off(kl + 1), -1.0, 1.0, w + o, w + o, red);
-      });
-    }
-    if (side == 1 && kr < K) {
-      const int m = len(kr);                // w_kr -= A_{kr,kr-1}[:,P] x_{kr-1}[P]
-      const double* B = A + (off(kr) - p) * n + off(kr);
-      rows(m, [&](int r0) { block_gemv(B, n, r0, m, p, x + off(kr) - p, -1.0, 1.0, w + off(kr), w + off(kr), red); });
-    }
-    grid.sync();
-    const int k = side == 0 ? kl : kr;
-    if (k >= 0 && k < K) {
-      const int m = len(k);
-      rows(m, [&](int r0) { block_gemv(inv(k), m, r0, m, m, w + off(k), 1.0, 0.0, x + off(k), x + off(k), red); });
-    }
-    grid.sync();
+    j = jn;
+#pragma unroll
+    for (int q = 0; q < kSvAhead; ++q) a[q] = an[q];
   }
 }
 
 int launch_slab_solve(const SlabChain& ch, const double* A, int64_t n, const double* sinv, double* w, double* x,
                       double* u, int sm_count, cudaStream_t st) {
-  // a block per 16 rows of a side's slab; more would only lengthen the barriers
-  const int grid = std::max(2, std::min(sm_count & ~1, 2 * ((ch.mmax + kSvRows - 1) / kSvRows)));
+  const int grid = std::max(2, std::min(sm_count & ~1, 2 * ((ch.mmax + kSvMinRows - 1) / kSvMinRows)));
   SlabChain c = ch;
   void* args[] = {(void*)&c, (void*)&A, (void*)&n, (void*)&sinv, (void*)&w, (void*)&x, (void*)&u};
   return cudaLaunchCooperativeKernel((const void*)k_slab_solve, grid, kSvThreads, args, 0, st) == cudaSuccess ? 0 : -2;
