@@ -263,8 +263,13 @@ __global__ void __launch_bounds__(256, sizeof(TV) == 8 ? 4 : 8) k_bsr4_residual_
 void launch_bsr_residual(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
                          const double* x, const double* b, double* y, cudaStream_t st) {
   const int64_t n = nb * B;
-  const unsigned grid4 = (unsigned)((n * 4 + 255) / 256);
-  if (B == 4) k_bsr4_residual_sub<4, double, double, double><<<grid4, 256, 0, st>>>(nb, rowptr, col, val, x, b, y);
+  // two threads a row where they fill the GPU: the rounds of two block rows fit
+  // their lengths better and the sum of a row takes one step instead of two.
+  // 314,000 rows: 68 us against 79 with four threads; 79,000: equal; 20,000: 11% slower
+  const int S = n >= 160000 ? 2 : 4;
+  const unsigned grid4 = (unsigned)((n * S + 255) / 256);
+  if (B == 4 && S == 2) k_bsr4_residual_sub<2, double, double, double><<<grid4, 256, 0, st>>>(nb, rowptr, col, val, x, b, y);
+  else if (B == 4) k_bsr4_residual_sub<4, double, double, double><<<grid4, 256, 0, st>>>(nb, rowptr, col, val, x, b, y);
   else launch_bsr6_residual<double>(nb, rowptr, col, val, x, b, y, st);
 }
 
