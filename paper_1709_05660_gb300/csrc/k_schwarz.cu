@@ -1387,19 +1387,7 @@ k_patch_apply_t(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_n
   }
 }
 
-// one Schwarz block per thread block (the level's own launch)
-template <typename T>
-__global__ void k_patch_gather_t(const int32_t* __restrict__ p_n, const int64_t* __restrict__ dense_off,
-                                 const int64_t* __restrict__ gmap_off, const int32_t* __restrict__ gmap,
-                                 const int64_t* __restrict__ boff_off, const int32_t* __restrict__ boff,
-                                 const int64_t* __restrict__ pad_off, const int32_t* __restrict__ padpos,
-                                 const double* __restrict__ bsr_val, int B, T* __restrict__ dense,
-                                 const int64_t* __restrict__ idx_off, T* __restrict__ dr, T* __restrict__ dc) {
-  gather_block<T>(blockIdx.x, p_n, dense_off, gmap_off, gmap, boff_off, boff, pad_off, padpos, bsr_val, B, dense,
-                  idx_off, dr, dc);
-}
-
-// the FP32 gathers of several levels in one launch (thread block i gathers
+// the gathers of several levels in one launch (thread block i gathers
 // block i - first of the level whose range holds i), so that the coarse
 // levels' few blocks run beside the finest level's instead of each paying a
 // launch of their own
@@ -1420,16 +1408,6 @@ void launch_patch_gather_levels(const GatherLevelsT<T>& lv, int nblocks, cudaStr
 
 
 // ---------------------------------------------------------------------------
-template <typename T>
-void launch_patch_gather_t(int np, const int32_t* p_n, const int64_t* dense_off, const int64_t* gmap_off,
-                           const int32_t* gmap, const int64_t* boff_off, const int32_t* boff, const int64_t* pad_off,
-                           const int32_t* padpos, const double* bsr_val, int B, T* dense, const int64_t* idx_off,
-                           T* dr, T* dc, cudaStream_t st) {
-  if (np <= 0) return;
-  k_patch_gather_t<T><<<np, 512, 0, st>>>(p_n, dense_off, gmap_off, gmap, boff_off, boff, pad_off, padpos, bsr_val,
-                                          B, dense, idx_off, dr, dc);
-}
-
 template <typename T, int W>
 bool try_gj_blk(const GjLevelsT<T>& lv, int nblocks, int max_n, cudaStream_t st) {
   const size_t smem = gj_blk_smem<T, W>(max_n);
@@ -1455,36 +1433,30 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
                        const int64_t* own_off, const int32_t* own, const int64_t* inv_off, T* dense, T* invT,
                        int32_t* status, bool n_mult4, cudaStream_t st) {
   if (np <= 0) return;
-  GjLevelsT<T> one{};
-  one.nlev = 1;
-  one.l[0] = GjLevelT<T>{p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, nullptr, 0};
-  if constexpr (std::is_same<T, double>::value)
-    if (launch_patch_gj_levels_f64(one, np, max_n, st)) return;
-  // small blocks: the whole matrix fits in shared memory (unblocked sweep)
   const size_t base = (size_t)max_n * (2 * sizeof(T) + 2 * sizeof(int)) + ((max_n + 15) / 16) * 16;
-  const size_t with_m = base + (size_t)max_n * max_n * sizeof(T);
-  if (with_m <= 190 * 1024) {
-    cudaFuncSetAttribute(k_patch_gj_t<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)with_m);
-    k_patch_gj_t<T, true><<<np, 512, with_m, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT,
-                                                   status);
-    return;
-  }
-  // larger blocks: panel-blocked sweep with the widest panel that fits
-  if (std::is_same<T, float>::value && n_mult4) {
-    float* d = reinterpret_cast<float*>(dense);
-    float* o = reinterpret_cast<float*>(invT);
+  if constexpr (std::is_same<T, float>::value) {
     GjLevels lv{};
     lv.nlev = 1;
     lv.first_wait = kTcWaitIters;
-    lv.l[0] = GjLevel{p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, nullptr, 0};
-    if (launch_patch_gj_tc_levels(lv, np, max_n, status, st)) return;
-    if (try_gj_f32<32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, st)) return;
-    if (try_gj_f32<16>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, d, o, status, st)) return;
-  }
-  if constexpr (std::is_same<T, float>::value)
-    if (try_gj_blk<T, 32>(one, np, max_n, st) || try_gj_blk<T, 16>(one, np, max_n, st) ||
-        try_gj_blk<T, 8>(one, np, max_n, st))
+    lv.l[0] = GjLevel{p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, nullptr, 0};
+    // small blocks: the whole matrix fits in shared memory (unblocked sweep)
+    const size_t with_m = base + (size_t)max_n * max_n * sizeof(T);
+    if (with_m <= 190 * 1024) {
+      cudaFuncSetAttribute(k_patch_gj_t<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)with_m);
+      k_patch_gj_t<T, true><<<np, 512, with_m, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT,
+                                                     status);
       return;
+    }
+    // larger blocks: panel-blocked sweep with the widest panel that fits
+    if (n_mult4) {
+      if (launch_patch_gj_tc_levels(lv, np, max_n, status, st)) return;
+      if (try_gj_f32<32>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
+      if (try_gj_f32<16>(np, max_n, p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status, st)) return;
+    }
+    if (try_gj_blk<T, 32>(lv, np, max_n, st) || try_gj_blk<T, 16>(lv, np, max_n, st) ||
+        try_gj_blk<T, 8>(lv, np, max_n, st))
+      return;
+  }
   cudaFuncSetAttribute(k_patch_gj_t<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
   k_patch_gj_t<T, false><<<np, 512, base, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT,
                                                 status);
@@ -1905,9 +1877,6 @@ void launch_patch_apply_ilu(int nsel, int max_n, int max_nb, const int32_t* sel,
 
 #define FSI_INST(T)                                                                                              \
   template void launch_patch_gather_levels<T>(const GatherLevelsT<T>&, int, cudaStream_t);                        \
-  template void launch_patch_gather_t<T>(int, const int32_t*, const int64_t*, const int64_t*, const int32_t*,  \
-                                         const int64_t*, const int32_t*, const int64_t*, const int32_t*,        \
-                                         const double*, int, T*, const int64_t*, T*, T*, cudaStream_t);         \
   template void launch_patch_gj_t<T>(int, int, const int32_t*, const int32_t*, const int64_t*, const int64_t*, \
                                      const int32_t*, const int64_t*, T*, T*, int32_t*, bool, cudaStream_t);     \
   template void launch_patch_apply_t<T>(int, int64_t, int, int, const int32_t*, const int32_t*, const int64_t*,\

@@ -125,7 +125,7 @@ struct GatherLevelT {
   const int64_t* gmap_off;
   const int32_t* gmap;
   const int64_t* boff_off;
-  const int32_t* boff;
+  const int32_t* boff;   // per local block its dense offset * 8 + width
   const int64_t* pad_off;
   const int32_t* padpos;
   const double* bsr_val;
@@ -145,12 +145,6 @@ void launch_patch_gather_levels(const GatherLevelsT<T>& lv, int nblocks, cudaStr
 // FP64 blocks of the levels in one launch; false when they fit no shared-memory
 // variant (the caller then factors level by level)
 bool launch_patch_gj_levels_f64(const GjLevelsT<double>& lv, int nblocks, int max_n, cudaStream_t st);
-// boff / boff_off: per local block of a Schwarz block its dense offset * 8 + width
-template <typename T>
-void launch_patch_gather_t(int np, const int32_t* p_n, const int64_t* dense_off, const int64_t* gmap_off,
-                           const int32_t* gmap, const int64_t* boff_off, const int32_t* boff, const int64_t* pad_off,
-                           const int32_t* padpos, const double* bsr_val, int B, T* dense, const int64_t* idx_off,
-                           T* dr, T* dc, cudaStream_t st);
 template <typename T>
 void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_nown, const int64_t* dense_off,
                        const int64_t* own_off, const int32_t* own, const int64_t* inv_off, T* dense, T* invT,
