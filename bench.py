@@ -47,6 +47,8 @@ FALLBACK_BF16_SUSTAINED_TFLOPS = 1700.0
 # FP64 ALU peak derived from the unit counts and clocks: 152 SMs x 2.07 GHz x
 # 4 FP64 flop / clock / SM (the 1.25 TFLOP/s nominal FP64 rate of the part).
 FP64_ALU_PEAK_GFLOPS = 152 * 2.07 * 4.0
+# FP64 products in fixed point: three wide integer multiply-adds (62.6 per SM and clock, measured) per multiply-add
+FIXED_POINT_PEAK_GFLOPS = 152 * 2.07 * 62.6 / 3.0 * 2.0
 # FP32 CUDA-core peak: 152 SMs x 2.07 GHz x 128 FP32 FMA / clock / SM x 2 flop.
 FP32_ALU_PEAK_GFLOPS = 152 * 2.07 * 256.0
 HBM_BOUND = {"patch_apply", "spmv", "transfer", "krylov", "scatter"}
@@ -704,6 +706,14 @@ def _roofline(kst, steps, fp32_classes=(), traffic_key=None):
                 "peak_source": f"{kind} bf16 sustained {bf16:.0f} TFLOP/s x nominal tf32/bf16 1.1/2.25",
                 "dtype": "tf32 (3xTF32 split, FP32 accumulate)",
                 "flops": "algorithmic Gauss-Jordan flops 2 n^3 per block (the tensor pipe executes 3x that)"}
+    elif dom == "patch_factor":
+        # FP64 block inverses: the trailing products run in fixed point on the integer pipe
+        achieved = d["flops"] / (d["ms"] / 1e3) / 1e9
+        roof = {"bound": "alu", "achieved": achieved / 1e3, "peak": FIXED_POINT_PEAK_GFLOPS / 1e3, "unit": "TFLOP/s",
+                "frac": achieved / FIXED_POINT_PEAK_GFLOPS,
+                "peak_source": "derived integer peak (152 SM x 2.07 GHz x 62.6 wide multiply-adds/clk, three per FP64 "
+                               "multiply-add)", "dtype": "f64",
+                "flops": "algorithmic Gauss-Jordan flops 2 n^3 per block (about half are left out as zeros or unread)"}
     else:
         achieved = d["flops"] / (d["ms"] / 1e3) / 1e9
         roof = {"bound": "alu", "achieved": achieved / 1e3, "peak": FP64_ALU_PEAK_GFLOPS / 1e3, "unit": "TFLOP/s",

@@ -1,13 +1,13 @@
 // Element-batched residual + exact Jacobian assembly and Galerkin coarsening.
 //
-// Assembly (Sec. 2.3, 2.5, 3): one thread per (element, unknown j) evaluates
-// the element residual in forward-mode dual arithmetic seeded along e_j, so
-// it produces column j of the exact element Jacobian (the derivative of the
-// discrete residual, as the paper obtains with automatic differentiation)
-// and the value of residual row j.  Element matrices are written to an
-// element-matrix buffer; a coloured scatter adds them into the block-sparse
-// Jacobian (elements of one colour share no node, so no atomics are needed
-// and the summation order is fixed).
+// Assembly (Sec. 2.3, 2.5, 3): the fluxes at a quadrature point depend on the
+// element unknowns only through a few fields (gradients and values of u and d,
+// p), so they are evaluated in forward-mode dual arithmetic along those fields
+// (the derivative of the discrete residual, as the paper obtains with automatic
+// differentiation) and contracted with the bases of trial and test functions one
+// direction after the other.  Element matrices are written to an element-matrix
+// buffer; a gather adds them into the block-sparse Jacobian, each entry over its
+// elements in a fixed order.
 //
 // Galerkin (Sec. 3.2): J_{l-1} = R J_l P is formed element by element.  A
 // coarse element matrix is sum_children R_c A_c P_c, where P_c interpolates
@@ -1541,10 +1541,10 @@ bool launch_assemble_3d(bool solid, const int32_t* elems, int ne, const double* 
 // 1 BDF, 2 Crank-Nicolson; Mooney-Rivlin adds a few percent in the solid);
 // used for the FP64-ALU fraction of the assembly in the per-class timings.
 double assemble_flops_per_element(int dim, bool solid, int mode) {
-  static const double f2[2][3] = {{113705.0, 121355.0, 155816.0}, {85909.0, 92740.0, 104785.0}};
-  // 3D: flux derivatives + columns
-  static const double f3[2][3] = {{437386.0 + 5908383.0, 539270.0 + 5908383.0, 1057103.0 + 5908383.0},
-                                  {242394.0 + 4286875.0, 313563.0 + 4286875.0, 502750.0 + 4286875.0}};
+  static const double f2[2][3] = {{58243.0, 66127.0, 100480.0}, {44932.0, 51325.0, 63655.0}};
+  // 3D: flux derivatives + sums over the quadrature points
+  static const double f3[2][3] = {{437386.0 + 839713.0, 531264.0 + 839713.0, 1057143.0 + 839713.0},
+                                  {242395.0 + 770633.0, 313568.0 + 770633.0, 502742.0 + 770633.0}};
   mode = mode < 0 ? 0 : (mode > 2 ? 2 : mode);
   return dim == 2 ? f2[solid][mode] : f3[solid][mode];
 }

@@ -1,12 +1,14 @@
 // Sparse / dense linear-algebra kernels of the Newton-step solve:
 //  * BSR residual / SpMV on the block-sparse Jacobian of each level;
 //  * scalar CSR SpMV for the grid transfers (Sec. 3.2);
-//  * coarse level (FP64): dense gather in the banded x-slab ordering, blocked
-//    banded LU with partial pivoting (cooperative), inverse columns by
-//    triangular solves, dense GEMV apply; for the slab-blocked 3D solve also
-//    dense GEMM / GEMV on column-major sub-matrices;
-//  * Krylov helpers: multi-vector dot products, classical Gram-Schmidt
-//    updates, norms, linear combinations (Sec. 4.1 FGMRES).
+//  * coarse level (FP64): row scales and dense gather over the free unknowns in
+//    the x-slab ordering; blocked banded LU with partial pivoting (cooperative)
+//    and inverse columns by triangular solves where the merged 2D inverse or the
+//    two-sided slab chain does not apply; dense GEMV apply; dense GEMM / GEMV on
+//    column-major sub-matrices;
+//  * Krylov helpers: the Arnoldi step (one cooperative launch up to 32 vectors),
+//    dot products, classical Gram-Schmidt updates, norms, linear combinations
+//    (Sec. 4.1 FGMRES).
 #include <cooperative_groups.h>
 
 #include <cmath>

@@ -7,7 +7,7 @@
 //    power-of-two row and column scales; the blocks mix rows scaled by the
 //    shear modulus, the ALE stiffness 1/V_el and the kinematic mass matrix,
 //    and without scaling an FP32 inverse loses its small entries.
-//  * k_patch_gj: in-place Gauss-Jordan with partial (row) pivoting, one thread
+//  * k_patch_gj_*: in-place Gauss-Jordan with partial (row) pivoting, one thread
 //    block per Schwarz block.  Only the rows of B_k^{-1} that belong to R^0_k
 //    are written out, transposed (column-major in the owned row index) so the
 //    smoother's batched product reads them with coalesced loads.
@@ -408,7 +408,8 @@ size_t gj_small_smem(int n) {
 // updates overlap.  The rank-W updates themselves run on the integer pipe
 // (fix_mad: 48 wide multiply-adds and two FP64 operations per entry and panel
 // instead of 16 FP64 ones).  5-level channel (1,364 blocks): 171 ms; with the
-// work left out 93.8; with the integer updates 40.2.
+// work left out 93.8; with the integer updates 40.2; with all levels in
+// one launch 31.3.
 template <typename T>
 __device__ __forceinline__ unsigned long long gj_key(T a) { return abs_key((double)a); }
 template <typename T>
