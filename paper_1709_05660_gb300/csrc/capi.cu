@@ -410,6 +410,7 @@ void build_device(Ctx& c) {
   c.c_B = dalloc<double>(c, (size_t)2 * n0);   // reciprocal pivots of the coarse LU
   c.c_piv = dalloc<int32_t>(c, n0);
   c.c_rhs = dalloc<double>(c, n0);
+  if (L == 1) c.c_val = dalloc<double>(c, (size_t)c.hl[0].nnzb * B * B);
   c.c_dr = dalloc<double>(c, n0);
   {
     const HostLevel& H0 = c.hl[0];
@@ -781,14 +782,15 @@ double coarse_slab_apply_bytes(const Ctx& c) {
 // of both vectors.  Unknowns that the ordering leaves out are identity rows
 // (x = b); their columns move to the right-hand side on a one-level instance,
 // where J_0 is the assembled operator (a Galerkin operator has none: the grid
-// transfers drop them).
+// transfers drop them).  The columns are those of the factored operator (c_val):
+// the level's own values may have been assembled or imported anew since.
 template <typename TB>
 void coarse_solve(Ctx& c, const TB* b, TB* x, double* part) {
   DevLevel& C = c.dl[0];
   const CoarseOrder& o = c.ord();
   const bool shift = c.dl.size() == 1 && o.n < C.Ni;
   if (shift) {
-    launch_coarse_rhs<TB>(c.B, C.nb, C.rowptr, C.col, C.val, o.pos, b, c.c_rhs, c.stream);
+    launch_coarse_rhs<TB>(c.B, C.nb, C.rowptr, C.col, c.c_val, o.pos, b, c.c_rhs, c.stream);
     counted(c);
   }
   if (o.slab) {
@@ -997,6 +999,9 @@ void coarse_factor(Ctx& c) {
     c.co_now = which;
     drop_vcycle_graph(c);   // the recorded V-cycle solves over the other ordering
   }
+  if (c.c_val)
+    ck(cudaMemcpyAsync(c.c_val, C.val, (size_t)C.nnzb * c.B * c.B * sizeof(double), cudaMemcpyDeviceToDevice,
+                       c.stream), "copy");
   const CoarseOrder& o = c.ord();
   if (o.slab) {
     if (o.twoway) coarse_factor_twoway(c);
@@ -1628,6 +1633,7 @@ static int64_t estimate_device_bytes(const Ctx& c) {
   const HostLevel& H0 = c.hl[0];
   const std::vector<int64_t>& so = H0.slab_off;
   b += 2.0 * n0 * 8.0 + H0.free_map.size() * 4.0 + n0 * 4.0;   // right-hand side, row scales, free ordering
+  if (L == 1) b += (double)H0.nnzb * B * B * 8.0;               // the factored operator's values
   if (c.dim == 3 && !so.empty()) {
     // dense banded-order operator + Sinv_k blocks + LU scratch + vectors
     double mm = 0.0, sum = 0.0;

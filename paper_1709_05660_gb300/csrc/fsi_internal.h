@@ -225,6 +225,7 @@ struct Ctx {
   double *c_L = nullptr, *c_Bp = nullptr, *c_gh = nullptr;   // scratch of the merged inverse
   double* c_dr = nullptr;                 // row scales of the coarse operator
   double* c_rhs = nullptr;                // right-hand side less the Dirichlet columns (one level)
+  double* c_val = nullptr;                // level 0's block values at the last factorisation (one level)
   // slab-blocked coarse solve (3D): Sinv_k blocks, LU scratch, vectors
   double *c_sinv = nullptr, *c_S = nullptr, *c_T = nullptr, *c_zb = nullptr, *c_xb = nullptr, *c_tp = nullptr;
   int32_t* c_iota = nullptr;
