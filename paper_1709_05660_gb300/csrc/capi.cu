@@ -168,7 +168,7 @@ double dev_norm(Ctx& c, int64_t n, const double* v, double* slot) {
 }
 
 // Throws for the errors of the kernels since the last call; true when only the
-// merged coarse inverse has to be redone by the banded LU.
+// coarse factorisation has to be redone by its sequential form (coarse_refactor).
 bool check_status(Ctx& c) {
   int32_t st[ST_COUNT];
   ck(cudaMemcpyAsync(st, c.status, sizeof(st), cudaMemcpyDeviceToHost, c.stream), "D2H status");
@@ -797,7 +797,7 @@ void coarse_solve(Ctx& c, const TB* b, TB* x, double* part) {
     if (shift) launch_coarse_pick<double>(o.n, o.map, c.c_dr, c.c_rhs, c.c_zb, c.stream);
     else launch_coarse_pick<TB>(o.n, o.map, c.c_dr, b, c.c_zb, c.stream);
     counted(c);
-    if (o.twoway) {
+    if (c.twoway()) {
       if (launch_slab_solve(slab_chain(o), c.c_A, o.n, c.c_sinv, c.c_zb, c.c_xb, c.s_u, c.sm_count, c.stream) != 0)
         throw ApiError(FSI_E_CUDA, "slab solve launch failed");
       counted(c);
@@ -975,12 +975,6 @@ void coarse_factor_banded(Ctx& c) {
   counted(c, 2);
 }
 
-// The merged inverse needs nonsingular slab ranges, which the LU's pivoting
-// across slabs does not; its result is therefore checked on one vector (rows
-// of A x - v against |A| |x| + |v|; both inverses measure below 1e-10 there, a
-// breakdown order 1), and factor() falls back to the LU when that fails.
-constexpr double kCoarseCheckTol = 1e-6;
-
 void drop_vcycle_graph(Ctx& c) {
   if (c.vc_exec) cudaGraphExecDestroy(c.vc_exec);
   if (c.vc_graph) cudaGraphDestroy(c.vc_graph);
@@ -989,23 +983,57 @@ void drop_vcycle_graph(Ctx& c) {
   c.vc_graph_failed = false;
 }
 
+// The 2D merged inverse needs nonsingular slab ranges, which the LU's pivoting
+// across slabs does not, and the 3D elimination from both ends needs the right
+// ends of the chain nonsingular beside the left ones.  The result is therefore
+// checked on one vector (rows of A x - v against |A| |x| + |v|; both inverses
+// measure below 1e-10 there, a breakdown order 1), and the factorisation redone by
+// the LU or the chain from one end (coarse_refactor) when that fails.
+constexpr double kCoarseCheckTol = 1e-6;
+
+void coarse_check(Ctx& c) {
+  DevLevel& C = c.dl[0];
+  const CoarseOrder& o = c.ord();
+  const double by = o.slab ? coarse_slab_apply_bytes(c) : (double)o.n * o.n * 8.0;
+  Prof pr(c, FSI_K_COARSE_FACTOR, by, by / 4.0, o.slab ? 5 : 4);
+  launch_coarse_probe(C.Ni, o.pos, C.b, c.stream);
+  coarse_solve<double>(c, C.b, C.x, c.c_part);
+  launch_coarse_check(c.B, C.nb, C.rowptr, C.col, C.val, C.b, C.x, kCoarseCheckTol, o.pos, c.status, c.stream);
+  counted(c, 2);
+}
+
+void coarse_refactor(Ctx& c) {
+  if (!c.ord().slab) {
+    coarse_factor_banded(c);
+    return;
+  }
+  c.one_sided = true;
+  drop_vcycle_graph(c);   // the recorded V-cycle solves from both ends
+  coarse_factor_slab(c);
+}
+
 // The Dirichlet rows of J_0 are identity rows, so its solve is one over the
 // free unknowns (2D 16 x 4 cells: 1,074 of 1,444; 3D 16 x 4 x 4: 10,200 of
 // 17,574, in slabs of 652 instead of 1,068), unless level 0 was imported.
 void coarse_factor(Ctx& c) {
   DevLevel& C = c.dl[0];
   const int which = c.coarse_imported ? 1 : 0;
-  if (which != c.co_now) {
+  if (which != c.co_now || c.one_sided) {
     c.co_now = which;
-    drop_vcycle_graph(c);   // the recorded V-cycle solves over the other ordering
+    c.one_sided = false;
+    drop_vcycle_graph(c);   // the recorded V-cycle solves over the other ordering, or from one end
   }
   if (c.c_val)
     ck(cudaMemcpyAsync(c.c_val, C.val, (size_t)C.nnzb * c.B * c.B * sizeof(double), cudaMemcpyDeviceToDevice,
                        c.stream), "copy");
   const CoarseOrder& o = c.ord();
   if (o.slab) {
-    if (o.twoway) coarse_factor_twoway(c);
-    else coarse_factor_slab(c);
+    if (o.twoway) {
+      coarse_factor_twoway(c);
+      coarse_check(c);
+    } else {
+      coarse_factor_slab(c);
+    }
   } else if (o.tree) {
     double flops = 0.0;
     const CoarseTree& t = *o.tree;
@@ -1015,15 +1043,15 @@ void coarse_factor(Ctx& c) {
       const double w = t.merge[i].b - t.merge[i].a;
       flops += 2.0 * p * w * (w + t.merge[i].s + 2.0 * p);
     }
-    Prof pr(c, FSI_K_COARSE_FACTOR, (double)o.n * o.n * 8.0 * 3.0, flops, 6);
-    coarse_gather(c);
-    const int rc = launch_coarse_merge(t, o.n, o.p, o.tree_leaf, o.tree_s, c.c_A, c.c_L, c.c_Bp, c.c_gh, c.c_inv,
-                                       c.status, c.sm_count, c.stream);
-    if (rc != 0) throw ApiError(FSI_E_CUDA, "merged coarse inverse launch failed (" + std::to_string(rc) + ")");
-    launch_coarse_probe(C.Ni, o.pos, C.b, c.stream);
-    launch_gemv<double, double>(C.Ni, o.n, c.c_inv, o.pos, o.map, c.c_dr, C.b, C.x, c.c_part, c.stream);
-    launch_coarse_check(c.B, C.nb, C.rowptr, C.col, C.val, C.b, C.x, kCoarseCheckTol, o.pos, c.status, c.stream);
-    counted(c, 5);
+    {
+      Prof pr(c, FSI_K_COARSE_FACTOR, (double)o.n * o.n * 8.0 * 3.0, flops, 3);
+      coarse_gather(c);
+      const int rc = launch_coarse_merge(t, o.n, o.p, o.tree_leaf, o.tree_s, c.c_A, c.c_L, c.c_Bp, c.c_gh, c.c_inv,
+                                         c.status, c.sm_count, c.stream);
+      if (rc != 0) throw ApiError(FSI_E_CUDA, "merged coarse inverse launch failed (" + std::to_string(rc) + ")");
+      counted(c);
+    }
+    coarse_check(c);
   } else {
     coarse_factor_banded(c);
   }
@@ -1078,7 +1106,7 @@ void factor(Ctx& c) {
   if (fork) cudaStreamWaitEvent(c.stream, c.ev_join, 0);
   else coarse_factor(c);
   if (check_status(c)) {
-    coarse_factor_banded(c);
+    coarse_refactor(c);
     check_status(c);
   }
   c.factored = true;
@@ -1101,7 +1129,7 @@ void coarse_grid(Ctx& c, const T* b, T* x) {
   const CoarseOrder& o = c.ord();
   const double n = (double)o.n, io = 2.0 * (double)c.dl[0].Ni * sizeof(T);
   const double by = o.slab ? coarse_slab_apply_bytes(c) : n * n * 8.0;
-  Prof pr(c, FSI_K_TRANSFER, by + io, by / 4.0, o.twoway ? 3 : (o.slab ? 2 + 8 * ((int)o.slab_off.size() - 1) : 2));
+  Prof pr(c, FSI_K_TRANSFER, by + io, by / 4.0, c.twoway() ? 3 : (o.slab ? 2 + 8 * ((int)o.slab_off.size() - 1) : 2));
   coarse_solve<T>(c, b, x, c.c_part);
 }
 
@@ -2044,7 +2072,7 @@ int fsi_factor_schwarz_batch(fsi_ctx* const* ctxs, int n) {
     for (int i = 0; i < n; ++i) {
       Ctx& c = *ctxs[i];
       if (check_status(c)) {
-        coarse_factor_banded(c);
+        coarse_refactor(c);
         check_status(c);
       }
       c.factored = true;

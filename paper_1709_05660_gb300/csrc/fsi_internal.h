@@ -222,6 +222,8 @@ struct Ctx {
   int co_now = 0;                         // ordering of the last factorisation
   bool coarse_imported = false;           // level 0 was imported since the last assembly
   const CoarseOrder& ord() const { return co[co_now]; }
+  bool one_sided = false;                 // 3D: the elimination from both ends failed its check
+  bool twoway() const { return ord().twoway && !one_sided; }
   double *c_L = nullptr, *c_Bp = nullptr, *c_gh = nullptr;   // scratch of the merged inverse
   double* c_dr = nullptr;                 // row scales of the coarse operator
   double* c_rhs = nullptr;                // right-hand side less the Dirichlet columns (one level)
@@ -264,8 +266,8 @@ struct Ctx {
 };
 
 // status flag slots
-// (ST_COARSE_RETRY: the merged coarse inverse broke down or failed its check;
-// the host then factors the coarse operator by the banded LU)
+// (ST_COARSE_RETRY: the merged coarse inverse or the 3D elimination from both ends
+// broke down or failed its check; the host then factors by the banded LU or from one end)
 enum { ST_SINGULAR = 0, ST_TANGLED = 1, ST_NONFINITE = 2, ST_TIMEOUT = 3, ST_COARSE_RETRY = 4, ST_COUNT = 5 };
 
 }  // namespace fsi

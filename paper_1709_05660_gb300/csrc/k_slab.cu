@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int 
       out[r] = __ldcg(J.rd + pr) * X[(size_t)c * ms + pr];
     }
   }
-  if (tid == 0 && s_sing) atomicExch(&status[ST_SINGULAR], 1);
+  if (tid == 0 && s_sing) atomicExch(&status[ST_COARSE_RETRY], 1);
 }
 
 namespace {

@@ -240,7 +240,7 @@ size_t slab_gj_scratch(int m);
 int slab_gj_panels(int m);
 bool slab_gj_fits(int m, int sm_count);
 // inverses of up to two slab complements at once; epoch: another one on every call with the same flags.
-// A zero pivot raises ST_SINGULAR, a wait that ran out ST_TIMEOUT
+// A zero pivot raises ST_COARSE_RETRY, a wait that ran out ST_TIMEOUT
 int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_count, cudaStream_t st);
 void launch_slab_gemm(const SlabGemm* g, int n, cudaStream_t st);   // n <= 2 products
 // x = A^{-1} w (w is overwritten); u: 2 mmax doubles
