@@ -986,10 +986,12 @@ void drop_vcycle_graph(Ctx& c) {
 // The 2D merged inverse needs nonsingular slab ranges, which the LU's pivoting
 // across slabs does not, and the 3D elimination from both ends needs the right
 // ends of the chain nonsingular beside the left ones.  The result is therefore
-// checked on one vector (rows of A x - v against |A| |x| + |v|; both inverses
-// measure below 1e-10 there, a breakdown order 1), and the factorisation redone by
-// the LU or the chain from one end (coarse_refactor) when that fails.
-constexpr double kCoarseCheckTol = 1e-6;
+// checked on one vector, and the factorisation redone by the LU or the chain from one
+// end (coarse_refactor) when that fails.  Largest row of |A x - v| / (|A| |x| + |v|)
+// over 200 problems of 2 to 4 levels on GB300: 2D 3e-14 to 1.5e-9 (the LU of the
+// same operators 2e-12 to 5e-9), 3D 9e-13 to 2.6e-8 (from one end 2e-11 to 2.3e-8), so
+// the operators' conditioning sets it and the limit lies above the largest.
+constexpr double kCoarseCheckTol = 1e-7;
 
 void coarse_check(Ctx& c) {
   DevLevel& C = c.dl[0];

@@ -85,8 +85,9 @@ def _solve(s, apply, b):
     return x.cpu().numpy()
 
 
-@pytest.mark.parametrize("delta", [0.0, 1e-12])
-@pytest.mark.parametrize("dim,slab", [(2, 1), (2, 4), (2, 6), (3, 4)])
+# (the last one: an error of 3e-7 in the probe's row, where sound inverses stay below 3e-8)
+@pytest.mark.parametrize("dim,slab,delta", [(2, 1, 0.0), (2, 4, 0.0), (2, 6, 0.0), (3, 4, 0.0), (2, 1, 1e-12),
+                                            (2, 4, 1e-12), (2, 6, 1e-12), (3, 4, 1e-12), (2, 6, 2e-11)])
 def test_one_level(dim, slab, delta):
     s = _instance(dim, 1)
     try:
