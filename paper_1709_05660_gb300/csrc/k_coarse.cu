@@ -260,7 +260,7 @@ template <int COLS>
 int run_merge(const CoarseTree& tr, int64_t n, int p, size_t smem, double* A, double* Lbuf, double* Bbuf, double* gh,
               double* Ainv, int32_t* status, int sm_count, cudaStream_t st) {
   const auto kern = k_coarse_merge<COLS>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (!allow_dynamic_smem(kern)) return -1;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMergeThreads, smem);
   if (per_sm < 1) return -1;

@@ -1081,7 +1081,7 @@ int launch_coarse_lu_inverse(int64_t n, int kl, int ku, double* M, double* rdiag
   void* args[] = {(void*)&n,     (void*)&kl,     (void*)&ku, (void*)&M, (void*)&piv, (void*)&rdiag,
                   (void*)&status, (void*)&cw};
   auto go = [&](auto kern, size_t smem) -> int {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem(kern);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (per_sm < 1) return -1;
@@ -1101,10 +1101,10 @@ int launch_coarse_lu_inverse(int64_t n, int kl, int ku, double* M, double* rdiag
   if (ismem > 200 * 1024) return -4;
   const unsigned nblk = (unsigned)((n + wpb - 1) / wpb);
   if ((int64_t)kl + ku <= 32 * 8) {   // narrow band: register prefetch of the next factor column
-    cudaFuncSetAttribute(k_band_inv_pf<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem);
+    allow_dynamic_smem(k_band_inv_pf<8>);
     k_band_inv_pf<8><<<nblk, wpb * kWarp, ismem, st>>>(n, kl, ku, M, piv, rdiag, perm, pinv, Ainv);
   } else {
-    cudaFuncSetAttribute(k_band_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ismem);
+    allow_dynamic_smem(k_band_inv);
     k_band_inv<<<nblk, wpb * kWarp, ismem, st>>>(n, kl, ku, M, piv, rdiag, perm, pinv, Ainv);
   }
   return 0;

@@ -864,7 +864,7 @@ bool try_gj_f32(int np, int max_n, const int32_t* p_n, const int32_t* p_nown, co
                 int32_t* status, cudaStream_t st) {
   const size_t smem = gj_f32_smem(max_n, W);
   if (smem > 225 * 1024 || max_n % 4 != 0 || (size_t)max_n * (W + 1) < 32 * 33) return false;
-  cudaFuncSetAttribute(k_patch_gj_f32<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k_patch_gj_f32<W>);
   k_patch_gj_f32<W><<<np, 1024, smem, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT, status,
                                             max_n);
   return true;
@@ -1257,7 +1257,7 @@ bool fits_gj_tc(int max_n) {
 template <int W, int TN, int NC = 512>
 void run_gj_tc(const GjLevels& lv, int nblocks, int max_n, int32_t* status, cudaStream_t st) {
   const size_t smem = gj_tc_smem<W, TN, NC>(max_n);
-  cudaFuncSetAttribute(k_patch_gj_tc<W, TN, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k_patch_gj_tc<W, TN, NC>);
   k_patch_gj_tc<W, TN, NC><<<nblocks, gj_tc_threads<W, TN, NC>(), smem, st>>>(lv, status, max_n);
 }
 
@@ -1413,7 +1413,7 @@ template <typename T, int W>
 bool try_gj_blk(const GjLevelsT<T>& lv, int nblocks, int max_n, cudaStream_t st) {
   const size_t smem = gj_blk_smem<T, W>(max_n);
   if (smem > 220 * 1024 || (size_t)32 * 33 > (size_t)max_n * W) return false;
-  cudaFuncSetAttribute(k_patch_gj_blk<T, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_dynamic_smem(k_patch_gj_blk<T, W>);
   k_patch_gj_blk<T, W><<<nblocks, 512, smem, st>>>(lv, max_n);
   return true;
 }
@@ -1422,7 +1422,7 @@ bool launch_patch_gj_levels_f64(const GjLevelsT<double>& lv, int nblocks, int ma
   if (nblocks <= 0 || lv.nlev < 1 || lv.nlev > kGjMaxLevels) return false;
   if (max_n <= kGjSmemMax) {
     const size_t smem = gj_small_smem(max_n);
-    cudaFuncSetAttribute(k_patch_gj_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem(k_patch_gj_small);
     k_patch_gj_small<<<nblocks, 512, smem, st>>>(lv);
     return true;
   }
@@ -1443,7 +1443,7 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
     // small blocks: the whole matrix fits in shared memory (unblocked sweep)
     const size_t with_m = base + (size_t)max_n * max_n * sizeof(T);
     if (with_m <= 190 * 1024) {
-      cudaFuncSetAttribute(k_patch_gj_t<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)with_m);
+      allow_dynamic_smem(k_patch_gj_t<T, true>);
       k_patch_gj_t<T, true><<<np, 512, with_m, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT,
                                                      status);
       return;
@@ -1458,7 +1458,7 @@ void launch_patch_gj_t(int np, int max_n, const int32_t* p_n, const int32_t* p_n
         try_gj_blk<T, 8>(lv, np, max_n, st))
       return;
   }
-  cudaFuncSetAttribute(k_patch_gj_t<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base);
+  allow_dynamic_smem(k_patch_gj_t<T, false>);
   k_patch_gj_t<T, false><<<np, 512, base, st>>>(p_n, p_nown, dense_off, own_off, own, inv_off, dense, invT,
                                                 status);
 }
@@ -1571,7 +1571,7 @@ void launch_patch_apply_t(int np, int64_t nv, int max_n, int max_nown, const int
     const int threads = a.vps * a.groups;
     const size_t smem = ((size_t)((max_n + 3) & ~3) + (size_t)a.groups * a.vps * VecT<T>::W) * sizeof(T);
     if (smem > 48 * 1024)   // large blocks (e.g. 16 x 16 elements): opt in to more shared memory
-      cudaFuncSetAttribute(k_patch_apply_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      allow_dynamic_smem(k_patch_apply_rows<T>);
     k_patch_apply_rows<T><<<(unsigned)((int64_t)np * a.slices), threads, smem, st>>>(
         p_n, p_nown, idx_off, idx, own_off, own, inv_off, invT, r, x, T(omega), dr, dc, a.slices, a.vps, a.groups,
         sel, nv);
@@ -1584,7 +1584,7 @@ void launch_patch_apply_t(int np, int64_t nv, int max_n, int max_nown, const int
   const int threads = vstride * CG;
   const size_t smem = ((size_t)((max_n + 3) & ~3) + (size_t)CG * vstride * VecT<T>::W) * sizeof(T);
   if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_patch_apply_t<T, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_dynamic_smem(k_patch_apply_t<T, CG>);
   k_patch_apply_t<T, CG><<<np, threads, smem, st>>>(p_n, p_nown, idx_off, idx, own_off, own, inv_off, invT, r, x,
                                                     T(omega), dr, dc, vstride, sel, nv);
 }

@@ -315,7 +315,7 @@ int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_coun
   for (int i = 0; i < jobs.n; ++i) mmax = std::max(mmax, jobs.j[i].m);
   ng = std::min(ng, slab_gj_panels(mmax));
   const size_t smem = slab_gj_smem(mmax, ng);
-  if (cudaFuncSetAttribute(k_slab_gj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (!allow_dynamic_smem(k_slab_gj)) return -1;
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_slab_gj, kSlabThreads, smem);
   if (per_sm < 1) return -1;

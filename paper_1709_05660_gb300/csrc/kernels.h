@@ -9,6 +9,18 @@
 
 namespace fsi {
 
+// Lets launches of a kernel take dynamic shared memory up to what an SM has for
+// one thread block (227 KB less the kernel's static arrays).  The limit belongs to the
+// kernel, not to the launch: were it set to each launch's own amount, another host
+// thread's smaller launch could lower it between this one's setting and its launch.
+template <typename K>
+inline bool allow_dynamic_smem(K kern) {
+  cudaFuncAttributes a;
+  return cudaFuncGetAttributes(&a, kern) == cudaSuccess &&
+         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              227 * 1024 - (int)a.sharedSizeBytes) == cudaSuccess;
+}
+
 struct PhysParams {
   double rho_f, mu_f, rho_s, mu_s;
   int ale_op;
