@@ -926,7 +926,7 @@ void schwarz_factor(Ctx& c) {
     GatherLevelsT<double> gl{};
     GjLevelsT<double> lv{};
     gl.B = B;
-    int first = 0, max_n = 0;
+    int first = 0, max_n = 0, level_max_n[kGjMaxLevels];
     int64_t off = 0;
     double by = 0.0, fl = 0.0;
     for (int l = L - 1; l >= 1; --l) {
@@ -938,6 +938,7 @@ void schwarz_factor(Ctx& c) {
       gl.l[gl.nlev++] = GatherLevelT<double>{D.p_n,    D.p_dense_off, D.p_gmap_off, D.p_gmap, D.p_boff_off,
                                              D.p_boff, D.p_pad_off,   D.p_padpos,   D.val,    ws,
                                              D.p_idx_off, D.dr,       D.dc,         first};
+      level_max_n[lv.nlev] = D.max_n;
       lv.l[lv.nlev++] = GjLevelT<double>{D.p_n, D.p_nown, D.p_dense_off, D.p_own_off, D.p_own, D.p_inv_off, ws,
                                          D.inv, c.status, nullptr, first};
       first += D.n_patches;
@@ -949,12 +950,17 @@ void schwarz_factor(Ctx& c) {
     counted(c);
     if (launch_patch_gj_levels_f64(lv, first, max_n, c.stream)) {
       counted(c);
-    } else {
-      for (int i = 0; i < lv.nlev; ++i) {   // blocks too large for shared memory: level by level
-        const GjLevelT<double>& v = lv.l[i];
+    } else {   // a level whose blocks are too large for shared memory: each by itself, as its own size allows
+      for (int i = 0; i < lv.nlev; ++i) {
+        GjLevelsT<double> one{};
+        GjLevelT<double>& v = one.l[0];
+        one.nlev = 1;
+        v = lv.l[i];
         const int np = (i + 1 < lv.nlev ? lv.l[i + 1].first : first) - v.first;
-        launch_patch_gj_t<double>(np, max_n, v.p_n, v.p_nown, v.dense_off, v.own_off, v.own, v.inv_off, v.dense,
-                                  v.invT, v.status, true, c.stream);
+        v.first = 0;
+        if (!launch_patch_gj_levels_f64(one, np, level_max_n[i], c.stream))
+          launch_patch_gj_t<double>(np, level_max_n[i], v.p_n, v.p_nown, v.dense_off, v.own_off, v.own, v.inv_off,
+                                    v.dense, v.invT, v.status, true, c.stream);
         counted(c);
       }
     }

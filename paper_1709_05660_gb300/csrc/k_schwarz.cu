@@ -1418,6 +1418,10 @@ bool try_gj_blk(const GjLevelsT<T>& lv, int nblocks, int max_n, cudaStream_t st)
   return true;
 }
 
+// The widest panel that fits in shared memory: 16 columns up to 768 unknowns, 8 up to
+// 1,376, 4 up to 2,272; larger blocks take k_patch_gj_t's sweep in device memory.  Factorisation
+// of a 16 x 12-element mesh in blocks of up to 1,348 unknowns (8 columns): 149 ms;
+// 1,394 (4 columns): 210 ms, 694 by the sweep; 1,508 (4 columns): 268 ms, 922 by the sweep.
 bool launch_patch_gj_levels_f64(const GjLevelsT<double>& lv, int nblocks, int max_n, cudaStream_t st) {
   if (nblocks <= 0 || lv.nlev < 1 || lv.nlev > kGjMaxLevels) return false;
   if (max_n <= kGjSmemMax) {
@@ -1426,7 +1430,8 @@ bool launch_patch_gj_levels_f64(const GjLevelsT<double>& lv, int nblocks, int ma
     k_patch_gj_small<<<nblocks, 512, smem, st>>>(lv);
     return true;
   }
-  return try_gj_blk<double, 16>(lv, nblocks, max_n, st) || try_gj_blk<double, 8>(lv, nblocks, max_n, st);
+  return try_gj_blk<double, 16>(lv, nblocks, max_n, st) || try_gj_blk<double, 8>(lv, nblocks, max_n, st) ||
+         try_gj_blk<double, 4>(lv, nblocks, max_n, st);
 }
 
 template <typename T>
