@@ -56,11 +56,13 @@ __device__ __forceinline__ void fix_mad(long long& hh, long long& mid, int2 a, i
   mid += (long long)a.y * b.x;
 }
 
-// c + the sum of products, for the exponent fields of the two scales
+// c + the sum of products, for the exponent fields of the two scales (a sum beyond
+// the FP64 range is infinite, as the sum of the products would be)
 __device__ __forceinline__ double fix_add(double c, long long hh, long long mid, int ea, int eb) {
+  const long long s = hh + ((mid + (1ll << 28)) >> 29);
   const int se = ea + eb - 1077;
-  const double scale = __hiloint2double(se > 0 ? se << 20 : 0, 0);
-  return fma((double)(hh + ((mid + (1ll << 28)) >> 29)), scale, c);
+  const double scale = __hiloint2double(se <= 0 ? 0 : (se < 2047 ? se << 20 : 2047 << 20), 0);
+  return s != 0 ? fma((double)s, scale, c) : c;
 }
 }  // namespace
 }  // namespace fsi
