@@ -150,7 +150,10 @@ int fsi_set_stream(fsi_ctx* ctx, void* stream);
  * `levels` entries, level 0 = coarse) and the device bytes held by ctx (for a
  * planned ctx: the bytes fsi_build_hierarchy would allocate).  The counts are
  * those of the Q2-P1disc spaces of Sec. 2.5 on each mesh of Sec. 3.2 (the
- * unknown counts of the table in Sec. 4); any pointer may be NULL. */
+ * unknown counts of the table in Sec. 4); any pointer may be NULL.  An FP64
+ * instance that does not fit the free device memory (or a server's budget) in
+ * that size is built with one workspace region for the Schwarz blocks of all
+ * levels instead of one a level, and factors them level by level. */
 int fsi_get_sizes(const fsi_ctx* ctx, int64_t* n_per_level, int64_t* nnz_per_level,
                   int64_t* hbm_bytes);
 

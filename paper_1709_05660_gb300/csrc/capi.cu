@@ -399,10 +399,13 @@ void build_device(Ctx& c) {
   c.stage_a = dalloc<double>(c, F.N);
   c.stage_b = dalloc<double>(c, F.N);
   // the blocks of all levels are factored in one launch: one workspace region
-  // per level
-  int64_t sum_dense = 0;
-  for (int l = 1; l < L; ++l) sum_dense += c.hl[l].dense_total;
-  c.dense_ws_len = std::max<int64_t>(sum_dense, 1);
+  // per level, unless memory is tight
+  int64_t sum_dense = 0, max_dense = 0;
+  for (int l = 1; l < L; ++l) {
+    sum_dense += c.hl[l].dense_total;
+    max_dense = std::max(max_dense, c.hl[l].dense_total);
+  }
+  c.dense_ws_len = std::max<int64_t>(c.tight ? max_dense : sum_dense, 1);
   c.dense_ws = dalloc<double>(c, c.mixed ? ((size_t)c.dense_ws_len + 1) / 2 : (size_t)c.dense_ws_len);
   // coarse dense operator
   const int64_t n0 = c.hl[0].Ni;
@@ -943,14 +946,18 @@ void schwarz_factor(Ctx& c) {
                                          D.inv, c.status, nullptr, first};
       first += D.n_patches;
       max_n = std::max(max_n, D.max_n);
-      off += D.dense_total;
+      if (!c.tight) off += D.dense_total;
     }
-    Prof pr(c, FSI_K_PATCH_FACTOR, by, fl, 2);
-    launch_patch_gather_levels<double>(gl, first, c.stream);
-    counted(c);
-    if (launch_patch_gj_levels_f64(lv, first, max_n, c.stream)) {
+    Prof pr(c, FSI_K_PATCH_FACTOR, by, fl, c.tight ? 2 * lv.nlev : 2);
+    if (!c.tight) {
+      launch_patch_gather_levels<double>(gl, first, c.stream);
       counted(c);
-    } else {   // a level whose blocks are too large for shared memory: each by itself, as its own size allows
+    }
+    if (!c.tight && launch_patch_gj_levels_f64(lv, first, max_n, c.stream)) {
+      counted(c);
+    } else {
+      // one workspace region, or a level whose blocks are too large for shared memory: each level by itself, as
+      // its own size allows
       for (int i = 0; i < lv.nlev; ++i) {
         GjLevelsT<double> one{};
         GjLevelT<double>& v = one.l[0];
@@ -958,6 +965,15 @@ void schwarz_factor(Ctx& c) {
         v = lv.l[i];
         const int np = (i + 1 < lv.nlev ? lv.l[i + 1].first : first) - v.first;
         v.first = 0;
+        if (c.tight) {
+          GatherLevelsT<double> g{};
+          g.B = B;
+          g.nlev = 1;
+          g.l[0] = gl.l[i];
+          g.l[0].first = 0;
+          launch_patch_gather_levels<double>(g, np, c.stream);
+          counted(c);
+        }
         if (!launch_patch_gj_levels_f64(one, np, level_max_n[i], c.stream))
           launch_patch_gj_t<double>(np, level_max_n[i], v.p_n, v.p_nown, v.dense_off, v.own_off, v.own, v.inv_off,
                                     v.dense, v.invT, v.status, true, c.stream);
@@ -1636,7 +1652,7 @@ static int max_assembly_batch(const Ctx& c) {
   return (int)std::max(F.n_fluid_elem, F.n_elem - F.n_fluid_elem);
 }
 
-static int64_t estimate_device_bytes(const Ctx& c) {
+static int64_t estimate_device_bytes(const Ctx& c, bool tight) {
   const bool mixed = c.opts.precision == FSI_MIXED;
   const double fs = mixed ? 4.0 : 8.0;
   const int B = c.B, nd = c.ndofe, m = c.opts.restart;
@@ -1663,9 +1679,12 @@ static int64_t estimate_device_bytes(const Ctx& c) {
   if (mixed) b += F.Ni * 8.0;   // the widened preconditioned vector
   if (c.desc.transient != 0) b += F.Ni * 8.0;
   if (c.dim == 3) b += (double)assemble_3d_scratch_doubles(max_assembly_batch(c)) * 8.0;
-  double sum_dense = 0.0;
-  for (size_t l = 1; l < L; ++l) sum_dense += (double)c.hl[l].dense_total;
-  b += sum_dense * fs + F.n_elem * (double)nd * 8.0 + 1e6;
+  double sum_dense = 0.0, max_dense = 0.0;
+  for (size_t l = 1; l < L; ++l) {
+    sum_dense += (double)c.hl[l].dense_total;
+    max_dense = std::max(max_dense, (double)c.hl[l].dense_total);
+  }
+  b += (tight && !mixed ? max_dense : sum_dense) * fs + F.n_elem * (double)nd * 8.0 + 1e6;
   const HostLevel& H0 = c.hl[0];
   const std::vector<int64_t>& so = H0.slab_off;
   b += 2.0 * n0 * 8.0 + H0.free_map.size() * 4.0 + n0 * 4.0;   // right-hand side, row scales, free ordering
@@ -1711,7 +1730,8 @@ static void plan(fsi_ctx* c, const fsi_problem_desc* desc, const fsi_solver_opts
   c->B = 2 * desc->dim;
   c->nloc = desc->dim == 2 ? 9 : 27;
   c->ndofe = c->B * c->nloc + desc->dim + 1;
-  c->est_bytes = estimate_device_bytes(*c);
+  c->est_bytes = estimate_device_bytes(*c, false);
+  c->est_tight = estimate_device_bytes(*c, true);
 }
 
 int fsi_plan_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opts, fsi_ctx** out) {
@@ -1732,6 +1752,15 @@ int fsi_plan_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opts
 }
 
 int fsi_build_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opts, void* stream, fsi_ctx** out) {
+  return build_hierarchy(desc, opts, stream, false, out);
+}
+
+}  // extern "C"
+
+int64_t fsi::tight_bytes(const fsi_ctx* c) { return c->est_tight; }
+
+int fsi::build_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opts, void* stream, bool tight,
+                         fsi_ctx** out) {
   if (!desc || !opts || !out) return FSI_E_INVALID;
   *out = nullptr;
   fsi_ctx* c = new (std::nothrow) fsi_ctx();
@@ -1749,6 +1778,9 @@ int fsi_build_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opt
     int coop = 0;
     ck(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev), "attr");
     if (!coop) throw ApiError(FSI_E_CUDA, "device lacks cooperative launch");
+    size_t room = 0, total = 0;
+    ck(cudaMemGetInfo(&room, &total), "cudaMemGetInfo");
+    c->tight = !c->mixed && (tight || c->est_bytes > (int64_t)room);
     build_device(*c);
     c->tmp_re = dalloc<double>(*c, (size_t)c->hl.back().n_elem * c->ndofe);
     if (c->dim == 3) {
@@ -1768,6 +1800,8 @@ int fsi_build_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opt
   *out = c;
   return FSI_OK;
 }
+
+extern "C" {
 
 void fsi_destroy(fsi_ctx* c) {
   if (!c) return;

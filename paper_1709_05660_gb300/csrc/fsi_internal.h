@@ -182,6 +182,7 @@ struct Ctx {
   std::vector<void*> allocs;
   int64_t bytes = 0;
   int64_t est_bytes = 0;                  // planned device bytes (before building)
+  int64_t est_tight = 0;                  // the same with `tight`
   std::string err;
   int64_t launches = 0;
   int dim = 2, B = 4, nloc = 9, ndofe = 39;
@@ -202,6 +203,7 @@ struct Ctx {
   double *stage_a = nullptr, *stage_b = nullptr;  // canonical staging vectors
   double* dense_ws = nullptr;             // patch factorisation workspace
   int64_t dense_ws_len = 0;
+  bool tight = false;                     // FP64: one region for every level's blocks, factored level by level
   int32_t *piv_ws = nullptr;              // per-patch pivots
   // coarse dense inverse
   double *c_A = nullptr, *c_B = nullptr, *c_inv = nullptr;
@@ -269,5 +271,12 @@ struct Ctx {
 // (ST_COARSE_RETRY: the merged coarse inverse or the 3D elimination from both ends
 // broke down or failed its check; the host then factors by the banded LU or from one end)
 enum { ST_SINGULAR = 0, ST_TANGLED = 1, ST_NONFINITE = 2, ST_TIMEOUT = 3, ST_COARSE_RETRY = 4, ST_COUNT = 5 };
+
+// Device bytes of a planned ctx, and its build, with one workspace region for the FP64
+// Schwarz blocks of all levels (factored level by level) instead of one a level:
+// what the server takes for an instance that fits its budget no other way.
+int64_t tight_bytes(const fsi_ctx* planned);
+int build_hierarchy(const fsi_problem_desc* desc, const fsi_solver_opts* opts, void* stream, bool tight,
+                    fsi_ctx** out);
 
 }  // namespace fsi

@@ -16,7 +16,7 @@
 
 #include <cuda_runtime.h>
 
-#include "../../include/fsi.h"
+#include "fsi_internal.h"
 
 namespace {
 
@@ -38,6 +38,7 @@ struct Instance {
   fsi_problem_desc desc{};
   fsi_solver_opts opts{};
   uint64_t last_use = 0;
+  bool tight = false;              // fits the budget only with the smaller FP64 workspace
   bool free_after = false;         // its last request was cancelled while a step ran
 };
 
@@ -49,6 +50,7 @@ struct Ticket {
   fsi_result res{};
   Clock::time_point t_submit, t_start, t_end;
   int state = 0;                   // 0 queued, 1 running, 2 done
+  bool tight = false;              // of that instance: planned with the smaller FP64 workspace
   int64_t planned = 0;             // planned bytes when the request creates the instance
   int64_t reserved = 0;            // bytes reserved at admission (new or evicted instance)
 };
@@ -157,8 +159,9 @@ struct fsi_server {
     if (!again) {
       in->desc = t->req.desc;
       in->opts = t->req.opts;
+      in->tight = t->tight;
     }
-    int rc = fsi_build_hierarchy(&in->desc, &in->opts, stream, &in->ctx);
+    int rc = fsi::build_hierarchy(&in->desc, &in->opts, stream, in->tight, &in->ctx);
     if (rc == FSI_OK) {
       int64_t nl[16], hb = 0;
       fsi_get_sizes(in->ctx, nl, nullptr, &hb);
@@ -358,6 +361,10 @@ int fsi_serve_submit(fsi_server* s, const fsi_request* req, uint64_t* ticket) {
     int64_t nl[16], hb = 0;
     fsi_get_sizes(plan, nl, nullptr, &hb);
     const int64_t n = nl[req->desc.levels - 1];
+    if (s->budget > 0 && hb > s->budget && fsi::tight_bytes(plan) <= s->budget) {
+      t->tight = true;
+      hb = fsi::tight_bytes(plan);
+    }
     fsi_destroy(plan);
     if (s->budget > 0 && hb > s->budget) return FSI_E_INVALID;
     if (!req->noise) return FSI_E_INVALID;
@@ -419,6 +426,7 @@ int fsi_serve_cancel(fsi_server* s, uint64_t ticket) {
     if (!t->noise.empty() && first) {
       first->noise.swap(t->noise);
       first->planned = t->planned;
+      first->tight = t->tight;
     }
     // a cancelled last request: the instance ends after its latest queued
     // request, else after the step that runs now, else at once
