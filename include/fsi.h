@@ -299,8 +299,9 @@ int fsi_import_csr(fsi_ctx* ctx, int level, const double* val);
  * factorisation on its tensor-core work (mixed precision).  When it runs out
  * the block waits (with the full limit) for the work it has already issued,
  * releases its tensor memory and reports FSI_E_TIMEOUT from
- * fsi_factor_schwarz; the ctx stays usable.  iters < 0 restores the built-in
- * limit (2^22).  A diagnostic of the time-out path; no counterpart in the
+ * fsi_factor_schwarz; the ctx stays usable.  The same limit holds for the waits
+ * of a 3D coarse slab's inverse for its panels (a message of their own).
+ * iters < 0 restores the built-in limits (2^22, 2^21).  A diagnostic of the time-out path; no counterpart in the
  * paper. */
 int fsi_set_tc_wait_limit(fsi_ctx* ctx, long long iters);
 /* y = J_level x (level's canonical numbering). */

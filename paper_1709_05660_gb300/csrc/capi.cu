@@ -179,6 +179,7 @@ bool check_status(Ctx& c) {
     if (site) throw ApiError(FSI_E_CUDA, "index out of range at bounds-check site " + std::to_string(site));
 #endif
   if (st[ST_TIMEOUT]) throw ApiError(FSI_E_TIMEOUT, "a bounded wait on the tensor core gave up");
+  if (st[ST_SLAB_TIMEOUT]) throw ApiError(FSI_E_TIMEOUT, "a bounded wait for a panel of a coarse slab inverse gave up");
   if (st[ST_TANGLED]) throw ApiError(FSI_E_MESH_TANGLED, "det F <= 0 at a quadrature point");
   if (st[ST_NONFINITE]) throw ApiError(FSI_E_NONFINITE, "non-finite values");
   if (st[ST_SINGULAR]) throw ApiError(FSI_E_SINGULAR, "zero or non-finite pivot in a Schwarz block or coarse LU");
@@ -732,7 +733,8 @@ void coarse_factor_twoway(Ctx& c) {
       }
       counted(c, last && ng == 2 ? 3 : 2);
     }
-    const int rc = launch_slab_gj(jobs, ++c.s_epoch, c.status, c.sm_count, c.stream);
+    const int rc = launch_slab_gj(jobs, ++c.s_epoch, c.tc_first_wait >= 0 ? c.tc_first_wait : kSlabWaitIters, c.status,
+                                  c.sm_count, c.stream);
     if (rc != 0) throw ApiError(FSI_E_CUDA, "slab inverse launch failed (" + std::to_string(rc) + ")");
     counted(c);
   }

@@ -269,8 +269,10 @@ struct Ctx {
 
 // status flag slots
 // (ST_COARSE_RETRY: the merged coarse inverse or the 3D elimination from both ends
-// broke down or failed its check; the host then factors by the banded LU or from one end)
-enum { ST_SINGULAR = 0, ST_TANGLED = 1, ST_NONFINITE = 2, ST_TIMEOUT = 3, ST_COARSE_RETRY = 4, ST_COUNT = 5 };
+// broke down or failed its check; the host then factors by the banded LU or from one end.
+// ST_TIMEOUT: a wait on the tensor core, ST_SLAB_TIMEOUT: one for a panel of a slab inverse)
+enum { ST_SINGULAR = 0, ST_TANGLED = 1, ST_NONFINITE = 2, ST_TIMEOUT = 3, ST_COARSE_RETRY = 4,
+       ST_SLAB_TIMEOUT = 5, ST_COUNT = 6 };
 
 // Device bytes of a planned ctx, and its build, with one workspace region for the FP64
 // Schwarz blocks of all levels (factored level by level) instead of one a level:

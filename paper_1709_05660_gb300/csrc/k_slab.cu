@@ -26,7 +26,6 @@ constexpr int kSlabThreads = 512;
 constexpr int kSlabRows = 2;                 // rows per thread: slabs of at most 1,024 unknowns
 constexpr int kSlabW = 4;                    // panel width
 constexpr int kSlabWarps = kSlabThreads / kWarp;
-constexpr long long kSlabWait = 1LL << 21;   // iteration limit of a wait for a panel
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
@@ -56,9 +55,9 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 // banded LU kernels.
 //
 // The launch is cooperative (all blocks resident), the waits are bounded: a
-// block whose wait runs out raises ST_TIMEOUT and returns, and so do those
+// block whose wait runs out raises ST_SLAB_TIMEOUT and returns, and so do those
 // that wait for it.
-__global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int ng, int epoch,
+__global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int ng, int epoch, long long wait,
                                                              int32_t* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SlabJob& J = jobs.j[blockIdx.x / ng];
@@ -245,12 +244,12 @@ __global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int 
       __syncthreads();
       if (tid == 0) {
         long long it = 0;
-        while (ld_acquire(J.flag + k) != epoch && it < kSlabWait) ++it;
-        if (it >= kSlabWait) s_abort = 1;
+        while (it < wait && ld_acquire(J.flag + k) != epoch) ++it;
+        if (it >= wait) s_abort = 1;
       }
       __syncthreads();
       if (s_abort) {
-        if (tid == 0) atomicExch(&status[ST_TIMEOUT], 1);
+        if (tid == 0) atomicExch(&status[ST_SLAB_TIMEOUT], 1);
         return;
       }
       const double2* src = reinterpret_cast<const double2*>(J.T + (size_t)k * kSlabW * ms);
@@ -310,7 +309,7 @@ bool slab_gj_fits(int m, int sm_count) {
   return m <= kSlabThreads * kSlabRows && sm_count >= 4 && slab_gj_smem(m, sm_count / 2) <= 200 * 1024;
 }
 
-int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_count, cudaStream_t st) {
+int launch_slab_gj(const SlabJobs& jobs, int epoch, long long wait, int32_t* status, int sm_count, cudaStream_t st) {
   int ng = jobs.n == 1 ? sm_count : sm_count / 2, mmax = 0;
   for (int i = 0; i < jobs.n; ++i) mmax = std::max(mmax, jobs.j[i].m);
   ng = std::min(ng, slab_gj_panels(mmax));
@@ -320,7 +319,7 @@ int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_coun
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_slab_gj, kSlabThreads, smem);
   if (per_sm < 1) return -1;
   SlabJobs jb = jobs;
-  void* args[] = {(void*)&jb, (void*)&ng, (void*)&epoch, (void*)&status};
+  void* args[] = {(void*)&jb, (void*)&ng, (void*)&epoch, (void*)&wait, (void*)&status};
   return cudaLaunchCooperativeKernel((const void*)k_slab_gj, ng * jobs.n, kSlabThreads, args, smem, st) == cudaSuccess
              ? 0 : -2;
 }

@@ -252,8 +252,10 @@ size_t slab_gj_scratch(int m);
 int slab_gj_panels(int m);
 bool slab_gj_fits(int m, int sm_count);
 // inverses of up to two slab complements at once; epoch: another one on every call with the same flags.
-// A zero pivot raises ST_COARSE_RETRY, a wait that ran out ST_TIMEOUT
-int launch_slab_gj(const SlabJobs& jobs, int epoch, int32_t* status, int sm_count, cudaStream_t st);
+// wait: iteration limit of a wait for a panel.  A zero pivot raises ST_COARSE_RETRY, a wait that ran out
+// ST_SLAB_TIMEOUT
+constexpr long long kSlabWaitIters = 1LL << 21;
+int launch_slab_gj(const SlabJobs& jobs, int epoch, long long wait, int32_t* status, int sm_count, cudaStream_t st);
 void launch_slab_gemm(const SlabGemm* g, int n, cudaStream_t st);   // n <= 2 products
 // x = A^{-1} w (w is overwritten); u: 2 mmax doubles
 int launch_slab_solve(const SlabChain& ch, const double* A, int64_t n, const double* sinv, double* w, double* x,
