@@ -1356,8 +1356,11 @@ void orthonormalize(Ctx& c, int j, int passes, double* h, double* hn, double* wn
   const int nb = nblk_red(c);
   double* sm = c.small;
   double* hs = c.host_small;
-  Prof pr(c, FSI_K_KRYLOV, (2.0 * passes * (j + 1) + 8.0) * n * 8.0, (4.0 * passes * (j + 1) + 4.0) * n,
-          j + 1 <= 32 ? 1 : (passes == 2 ? 8 : 5));
+  // fused step: the basis once for the first products and once per pass (a pass's update and the next products share
+  // a sweep), w read, updated per pass and read once more for v_{j+1}; separate launches: the basis twice per pass
+  const bool fused = j + 1 <= 32;
+  Prof pr(c, FSI_K_KRYLOV, (fused ? (passes + 1.0) * (j + 1) + 2.0 * passes + 3.0 : 2.0 * passes * (j + 1) + 8.0) * n * 8.0,
+          (4.0 * passes * (j + 1) + 4.0) * n, fused ? 1 : (passes == 2 ? 8 : 5));
   double* vnext = c.V + (size_t)(j + 1) * n;
   if (launch_arnoldi_step(n, c.V, n, j + 1, passes, c.w, vnext, c.partial, nb, sm, c.stream)) {
     counted(c);
