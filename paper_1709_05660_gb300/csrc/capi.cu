@@ -175,7 +175,7 @@ bool check_status(Ctx& c) {
   sync(c);
   ck(cudaMemsetAsync(c.status, 0, sizeof(st), c.stream), "memset");
 #ifdef FSI_BOUNDS_CHECK
-  for (int site : {bounds_site_schwarz(), bounds_site_linalg()})
+  for (int site : {bounds_site_schwarz(), bounds_site_linalg(), bounds_site_coarse(), bounds_site_slab()})
     if (site) throw ApiError(FSI_E_CUDA, "index out of range at bounds-check site " + std::to_string(site));
 #endif
   if (st[ST_TIMEOUT]) throw ApiError(FSI_E_TIMEOUT, "a bounded wait on the tensor core gave up");
@@ -799,8 +799,8 @@ void coarse_solve(Ctx& c, const TB* b, TB* x, double* part) {
     counted(c);
   }
   if (o.slab) {
-    if (shift) launch_coarse_pick<double>(o.n, o.map, c.c_dr, c.c_rhs, c.c_zb, c.stream);
-    else launch_coarse_pick<TB>(o.n, o.map, c.c_dr, b, c.c_zb, c.stream);
+    if (shift) launch_coarse_pick<double>(C.Ni, o.n, o.map, c.c_dr, c.c_rhs, c.c_zb, c.stream);
+    else launch_coarse_pick<TB>(C.Ni, o.n, o.map, c.c_dr, b, c.c_zb, c.stream);
     counted(c);
     if (c.twoway()) {
       if (launch_slab_solve(slab_chain(o), c.c_A, o.n, c.c_sinv, c.c_zb, c.c_xb, c.s_u, c.sm_count, c.stream) != 0)

@@ -5,6 +5,7 @@
 
 #include <cstdint>
 
+#include "bounds.cuh"
 #include "fp64_util.cuh"
 
 namespace fsi {
@@ -72,7 +73,7 @@ __device__ bool gj_inverse_smem(double* M, int n, int ld, double* f, double* rd,
       if (u < nu && !((used >> u) & 1u) && lane + u * kWarp < n && abs_key(v[u]) == best) row = lane + u * kWarp;
     const int bi = (int)__reduce_min_sync(0xffffffffu, row);
     double rp = 0.0;
-    if (lane == 0) {
+    if (lane == 0 && FSI_IN(bi, n, FSI_SITE(5))) {
       double pv = Mk[bi];
       if (best == 0ull || best >= 0x7FF0000000000000ull) {
         st.sing = 1;
@@ -129,6 +130,7 @@ __device__ bool gj_inverse_smem(double* M, int n, int ld, double* f, double* rd,
   for (int k = 0; k < n; ++k) {
     __syncthreads();
     const int pr = st.row[k & 1];
+    if (!FSI_IN(pr, n, FSI_SITE(5))) break;   // the whole block
     const uint32_t live = st.live[k & 1];
     double fr[kGjU];
 #pragma unroll

@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(kMergeThreads) k_coarse_merge(CoarseTree tr, i
     double* out = tr.nlev > 0 ? A : Ainv;
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
       const int c = e / m, r = e % m;
-      out[(o + c) * n + o + r] = rd[piv[r]] * M[piv[r] + qinv[c] * m];
+      if (FSI_IN(piv[r], m, FSI_SITE(3)) && FSI_IN(qinv[c], m, FSI_SITE(3)))
+        out[(o + c) * n + o + r] = rd[piv[r]] * M[piv[r] + qinv[c] * m];
     }
     __syncthreads();
   }
@@ -191,7 +192,9 @@ __global__ void __launch_bounds__(kMergeThreads) k_coarse_merge(CoarseTree tr, i
           const int j = e / p, q = e % p;
           double acc = 0.0;
           if (j < nc)
-            for (int k = 0; k < p; ++k) acc = fma(H[piv[q] + qinv[k] * p], R[j * p + k], acc);
+            for (int k = 0; k < p; ++k)
+              if (FSI_IN(piv[q], p, FSI_SITE(3)) && FSI_IN(qinv[k], p, FSI_SITE(3)))
+                acc = fma(H[piv[q] + qinv[k] * p], R[j * p + k], acc);
           Ut[q * kMergeCols + j] = acc * rd[piv[q]];
         }
         __syncthreads();
@@ -314,6 +317,7 @@ __global__ void k_coarse_check(int B, int64_t nb, const int32_t* __restrict__ ro
     const int ci = (int)(i % B);
     for (int32_t k = rowptr[br] + sub; k < rowptr[br + 1]; k += 8)
       for (int c = 0; c < B; ++c) {
+        if (!FSI_IN(col[k], nb, FSI_SITE(3))) continue;
         const double t = val[((int64_t)k * B + ci) * B + c] * x[(int64_t)col[k] * B + c];
         s += t;
         a += fabs(t);
@@ -345,5 +349,7 @@ void launch_coarse_check(int B, int64_t nb, const int32_t* rowptr, const int32_t
   const int64_t n = nb * B;
   k_coarse_check<<<(unsigned)((n * 8 + 255) / 256), 256, 0, st>>>(B, nb, rowptr, col, val, v, x, tol, pos, status);
 }
+
+FSI_BOUNDS_READER(bounds_site_coarse)
 
 }  // namespace fsi

@@ -681,7 +681,7 @@ __global__ void k_coarse_row_scale(int B, int64_t nb, const int32_t* __restrict_
     const int64_t br = i / B;
     const int ci = (int)(i % B);
     for (int32_t k = rowptr[br] + sub; k < rowptr[br + 1]; k += 8)
-      for (int c = 0; c < B; ++c)
+      for (int c = 0; c < B && FSI_IN(col[k], nb, FSI_SITE(2)); ++c)
         if (perm[(int64_t)col[k] * B + c] >= 0)
           top = max(top, (uint32_t)(abs_key(val[((int64_t)k * B + ci) * B + c]) >> 52));
   }
@@ -1119,14 +1119,17 @@ int launch_coarse_lu_inverse(int64_t n, int kl, int ku, double* M, double* rdiag
 constexpr int kGemvChunk = 32;
 
 template <typename TX>
-__global__ void __launch_bounds__(256) k_gemv_cm_part(int64_t n, const double* __restrict__ A,
+__global__ void __launch_bounds__(256) k_gemv_cm_part(int64_t ni, int64_t n, const double* __restrict__ A,
                                                       const int32_t* __restrict__ map, const double* __restrict__ dr,
                                                       const TX* __restrict__ x, double* __restrict__ part) {
   __shared__ double xs[kGemvChunk];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t c0 = (int64_t)blockIdx.y * kGemvChunk;
   const int64_t c1 = min(n, c0 + kGemvChunk);
-  if (threadIdx.x < c1 - c0) xs[threadIdx.x] = (double)x[map[c0 + threadIdx.x]] * dr[c0 + threadIdx.x];
+  if (threadIdx.x < c1 - c0) {
+    const int32_t m = map[c0 + threadIdx.x];
+    xs[threadIdx.x] = FSI_IN(m, ni, FSI_SITE(2)) ? (double)x[m] * dr[c0 + threadIdx.x] : 0.0;
+  }
   __syncthreads();
   if (i >= n) return;
   // all 32 loads of a full chunk in flight
@@ -1155,7 +1158,7 @@ __global__ void k_gemv_cm_sum(int64_t ni, int64_t n, int nchunk, const double* _
   const int64_t r = pos[i];
   double s = 0.0;
   if (r < 0) s = (double)x[i];
-  else {
+  else if (FSI_IN(r, n, FSI_SITE(2))) {
     double s1 = 0.0;
     int q = 0;
     for (; q + 8 <= nchunk; q += 8) {   // eight loads in flight
@@ -1175,7 +1178,7 @@ template <typename TX, typename TY>
 void launch_gemv(int64_t ni, int64_t n, const double* A, const int32_t* pos, const int32_t* map, const double* dr,
                  const TX* x, TY* y, double* part, cudaStream_t st) {
   const int nchunk = (int)((n + kGemvChunk - 1) / kGemvChunk);
-  k_gemv_cm_part<TX><<<dim3((unsigned)((n + 255) / 256), nchunk), 256, 0, st>>>(n, A, map, dr, x, part);
+  k_gemv_cm_part<TX><<<dim3((unsigned)((n + 255) / 256), nchunk), 256, 0, st>>>(ni, n, A, map, dr, x, part);
   k_gemv_cm_sum<TX, TY><<<(unsigned)((ni + 255) / 256), 256, 0, st>>>(ni, n, nchunk, part, pos, x, y);
 }
 template void launch_gemv<double, double>(int64_t, int64_t, const double*, const int32_t*, const int32_t*, const double*,
@@ -1221,21 +1224,22 @@ template <typename TB, typename TY>
 __global__ void k_coarse_scatter(int64_t ni, const int32_t* __restrict__ pos, const double* __restrict__ x,
                                  const TB* __restrict__ b, TY* __restrict__ y) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ni) y[i] = TY(pos[i] >= 0 ? x[pos[i]] : (double)b[i]);
+  if (i < ni && (pos[i] < 0 || FSI_IN(pos[i], ni, FSI_SITE(2)))) y[i] = TY(pos[i] >= 0 ? x[pos[i]] : (double)b[i]);
 }
 template <typename TB>
-__global__ void k_coarse_pick(int64_t n, const int32_t* __restrict__ map, const double* __restrict__ dr,
+__global__ void k_coarse_pick(int64_t ni, int64_t n, const int32_t* __restrict__ map, const double* __restrict__ dr,
                               const TB* __restrict__ b, double* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = (double)b[map[i]] * dr[i];
+  if (i < n && FSI_IN(map[i], ni, FSI_SITE(2))) out[i] = (double)b[map[i]] * dr[i];
 }
 template <typename TB, typename TY>
 void launch_coarse_scatter(int64_t ni, const int32_t* pos, const double* x, const TB* b, TY* y, cudaStream_t st) {
   k_coarse_scatter<TB, TY><<<(unsigned)((ni + 255) / 256), 256, 0, st>>>(ni, pos, x, b, y);
 }
 template <typename TB>
-void launch_coarse_pick(int64_t n, const int32_t* map, const double* dr, const TB* b, double* out, cudaStream_t st) {
-  k_coarse_pick<TB><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, map, dr, b, out);
+void launch_coarse_pick(int64_t ni, int64_t n, const int32_t* map, const double* dr, const TB* b, double* out,
+                        cudaStream_t st) {
+  k_coarse_pick<TB><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ni, n, map, dr, b, out);
 }
 template void launch_coarse_scatter<double, double>(int64_t, const int32_t*, const double*, const double*, double*,
                                                     cudaStream_t);
@@ -1243,8 +1247,8 @@ template void launch_coarse_scatter<double, float>(int64_t, const int32_t*, cons
                                                    cudaStream_t);
 template void launch_coarse_scatter<float, float>(int64_t, const int32_t*, const double*, const float*, float*,
                                                   cudaStream_t);
-template void launch_coarse_pick<double>(int64_t, const int32_t*, const double*, const double*, double*, cudaStream_t);
-template void launch_coarse_pick<float>(int64_t, const int32_t*, const double*, const float*, double*, cudaStream_t);
+template void launch_coarse_pick<double>(int64_t, int64_t, const int32_t*, const double*, const double*, double*, cudaStream_t);
+template void launch_coarse_pick<float>(int64_t, int64_t, const int32_t*, const double*, const float*, double*, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // slab-blocked coarse solve (3D): dense FP64 building blocks on column-major

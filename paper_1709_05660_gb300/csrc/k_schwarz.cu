@@ -531,6 +531,7 @@ k_patch_gj_blk(const GjLevelsT<T> lv, int max_n) {
     for (int m = 0; m < wp; ++m) {
       __syncthreads();
       const int pr = s_row[m & 1];
+      if (!FSI_IN(pr, n, FSI_SITE(1))) break;   // the whole block
       const T* fk = f + (m & 1) * max_n;
       const uint8_t* flk = fl + (m & 1) * mch;
       if (wid == 0) {
@@ -553,6 +554,7 @@ k_patch_gj_blk(const GjLevelsT<T> lv, int max_n) {
     __syncthreads();
     // old pivot rows, the column groups they reach, panel write-back
     for (int m = wid; m < wp; m += nw) {
+      if (!FSI_IN(piv[k0 + m], n, FSI_SITE(1))) continue;
       const T* Mp = M + (int64_t)piv[k0 + m] * n;
       for (int j = lane; j < n; j += kWarp) R[m * max_n + j] = Mp[j];
     }

@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int 
       for (int t = tid; t < kSlabW * ms / 2; t += kSlabThreads) dst[t] = __ldcg(src + t);
       if (tid < kSlabW) {
         const int pr = k * kSlabW + tid < m ? __ldcg(J.piv + k * kSlabW + tid) : 0;
-        s_piv[b][tid] = pr;
-        if (k * kSlabW + tid < m) s_used[pr] = 1;
+        s_piv[b][tid] = FSI_IN(pr, m, FSI_SITE(4)) ? pr : 0;
+        if (k * kSlabW + tid < m && FSI_IN(pr, m, FSI_SITE(4))) s_used[pr] = 1;
       }
     }
     // the next panel first, if it is this block's
@@ -286,10 +286,12 @@ __global__ void __launch_bounds__(kSlabThreads, 1) k_slab_gj(SlabJobs jobs, int 
   for (int c = wid; c < slots * kSlabW; c += kSlabWarps) {
     const int col = ((c / kSlabW) * ng + g) * kSlabW + c % kSlabW;
     if (col >= m) continue;
-    double* out = J.X + (size_t)__ldcg(J.piv + col) * m;
+    const int oc = __ldcg(J.piv + col);
+    if (!FSI_IN(oc, m, FSI_SITE(4))) continue;
+    double* out = J.X + (size_t)oc * m;
     for (int r = lane; r < m; r += kWarp) {
       const int pr = __ldcg(J.piv + r);
-      out[r] = __ldcg(J.rd + pr) * X[(size_t)c * ms + pr];
+      if (FSI_IN(pr, m, FSI_SITE(4))) out[r] = __ldcg(J.rd + pr) * X[(size_t)c * ms + pr];
     }
   }
   if (tid == 0 && s_sing) atomicExch(&status[ST_COARSE_RETRY], 1);
@@ -569,5 +571,7 @@ int launch_slab_solve(const SlabChain& ch, const double* A, int64_t n, const dou
   void* args[] = {(void*)&c, (void*)&A, (void*)&n, (void*)&sinv, (void*)&w, (void*)&x, (void*)&u};
   return cudaLaunchCooperativeKernel((const void*)k_slab_solve, grid, kSvThreads, args, 0, st) == cudaSuccess ? 0 : -2;
 }
+
+FSI_BOUNDS_READER(bounds_site_slab)
 
 }  // namespace fsi

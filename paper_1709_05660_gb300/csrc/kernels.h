@@ -36,6 +36,8 @@ struct PhysParams {
 // 100000 + line; 0: none), cleared by the read; always 0 in the normal build
 int bounds_site_schwarz();
 int bounds_site_linalg();
+int bounds_site_coarse();
+int bounds_site_slab();
 
 // k_assemble.cu
 // scratch: 3D only, assemble_3d_scratch_doubles(scratch_ne) doubles (2D: unused); false (nothing
@@ -271,7 +273,8 @@ template <typename TX>
 void launch_coarse_rhs(int B, int64_t nb, const int32_t* rowptr, const int32_t* col, const double* val,
                        const int32_t* pos, const TX* b, double* out, cudaStream_t st);
 template <typename TB>
-void launch_coarse_pick(int64_t n, const int32_t* map, const double* dr, const TB* b, double* out, cudaStream_t st);
+void launch_coarse_pick(int64_t ni, int64_t n, const int32_t* map, const double* dr, const TB* b, double* out,
+                        cudaStream_t st);
 template <typename TB, typename TY>
 void launch_coarse_scatter(int64_t ni, const int32_t* pos, const double* x, const TB* b, TY* y, cudaStream_t st);
 // slab-blocked coarse solve: column-major FP64 sub-matrices with leading dimensions
