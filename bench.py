@@ -457,6 +457,7 @@ def _measure(args, prec, stream, barrier, dist, world, local, rtol=None, steps=N
            "steps": steps, "warmup": warmup, "rtol": opts.rtol, "error_vs_oracle": err,
            "profiled_ms_per_step": ms_prof / prof_steps, "prof_steps": prof_steps,
            "iters": iters, "rel_res": max(rel_res), "rel_step": rel, "kst": kst, "launches": launches,
+           "max_block": max((len(d) for lev in range(1, prob.levels) for d, _ in s.export_patches(lev)), default=0),
            "clocks": clk, "hbm_bytes": s.hbm_bytes, "tuned": s.tuning is not None,
            "phase_ms": {"assemble": st.t_assemble_ms, "factor": st.t_factor_ms, "solve": st.t_solve_ms}}
     if e2e:
@@ -683,7 +684,12 @@ def _measure_transient_3d(args, stream):
             "kernel_classes": classes}
 
 
-def _roofline(kst, steps, fp32_classes=(), traffic_key=None):
+# Largest FP64 Schwarz block that is inverted in shared memory on the FP64 pipe; larger ones form their trailing
+# products in fixed point on the integer pipe.
+FP64_SMALL_BLOCK = 160
+
+
+def _roofline(kst, steps, fp32_classes=(), traffic_key=None, max_block=None):
     peaks, kind = _peaks()
     hbm_peak = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS)) if peaks else FALLBACK_HBM_GBS
     dom = max(kst, key=lambda k: kst[k]["ms"])
@@ -706,7 +712,7 @@ def _roofline(kst, steps, fp32_classes=(), traffic_key=None):
                 "peak_source": f"{kind} bf16 sustained {bf16:.0f} TFLOP/s x nominal tf32/bf16 1.1/2.25",
                 "dtype": "tf32 (3xTF32 split, FP32 accumulate)",
                 "flops": "algorithmic Gauss-Jordan flops 2 n^3 per block (the tensor pipe executes 3x that)"}
-    elif dom == "patch_factor":
+    elif dom == "patch_factor" and (max_block is None or max_block > FP64_SMALL_BLOCK):
         # FP64 block inverses: the trailing products run in fixed point on the integer pipe
         achieved = d["flops"] / (d["ms"] / 1e3) / 1e9
         roof = {"bound": "alu", "achieved": achieved / 1e3, "peak": FIXED_POINT_PEAK_GFLOPS / 1e3, "unit": "TFLOP/s",
@@ -806,7 +812,8 @@ def run_gpu(args, rank, world):
             "e2e": main["e2e"], "gpu_launches": main["launches"], "clocks": main["clocks"],
         }
         if fp64 is not None:
-            r64, c64 = _roofline(fp64["kst"], fp64["prof_steps"], traffic_key=f"{args.config} fp64")
+            r64, c64 = _roofline(fp64["kst"], fp64["prof_steps"], traffic_key=f"{args.config} fp64",
+                                 max_block=fp64["max_block"])
             line["fp64_path"] = {"value": fp64["value"], "ms_per_step": fp64["per_step"], "steps": fp64["steps"],
                                  "rtol": fp64["rtol"], "error_vs_oracle": fp64["error_vs_oracle"],
                                  "fgmres_iters": fp64["iters"], "max_true_rel_residual": fp64["rel_res"],
