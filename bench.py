@@ -759,11 +759,13 @@ DETAIL_KEYS = ("oracle_xstar", "rtol_sweep", "kernel_classes", "kernel_classes_p
 
 def split_line(full):
     """(headline, detail) of a full result: the detail keys, the FP64 path beyond its headline and the CPU baseline's
-    breakdown move to the detail."""
+    breakdown move to the detail; the served rate and latencies stay in the headline too."""
     line, detail = {}, {}
     for k, v in full.items():
         if k in DETAIL_KEYS:
             detail[k] = v
+            if k == "served" and isinstance(v.get("mixed"), dict):
+                line[k] = {q: v["mixed"]["poisson"][q] for q in ("solves_per_s", "p50_ms", "p99_ms", "requests")}
         elif k == "fp64_path":
             detail[k] = v
             line[k] = {q: v[q] for q in ("value", "ms_per_step", "steps", "rtol", "error_vs_oracle") if q in v}

@@ -27,5 +27,11 @@ def test_line_is_short_and_nothing_is_lost():
     assert all(line[k] == full[k] for k in HEADLINE)
     assert line["fp64_path"]["value"] == 1.5 and line["cpu_baseline"]["cores"] == 1
     assert {k: detail.get(k, line.get(k)) for k in full} == full
+    poisson = {"solves_per_s": 6.0, "p50_ms": 250.0, "p99_ms": 3000.0, "requests": 256, "failed_instances": [[1.0]] * 99}
+    line, detail = b.split_line({"value": 1.0, "served": {"mixed": {"poisson": poisson}}})
+    assert line["served"] == {k: v for k, v in poisson.items() if k != "failed_instances"}
+    assert detail["served"]["mixed"]["poisson"] == poisson
+    line, detail = b.split_line({"value": 1.0, "served": {"error": "x"}})
+    assert line == {"value": 1.0} and detail == {"served": {"error": "x"}}
     line, detail = b.split_line({"value": 1.0, "cpu_baseline": None})
     assert line == {"value": 1.0, "cpu_baseline": None} and detail == {}
