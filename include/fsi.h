@@ -92,7 +92,11 @@ typedef struct {
   double rtol;         /* krylov 0: stop when ||b - J x|| <= rtol ||b|| (true residual);
                           krylov 1: when ||P^{-1}(b - J x)|| < rtol ||P^{-1}(b - J x0)|| */
   int max_iters;       /* total Krylov iterations */
-  int precision;       /* FSI_FP64, or FSI_MIXED: FP32 V-cycle and Schwarz inverses, FP64 elsewhere */
+  int precision;       /* FSI_FP64, or FSI_MIXED: FP32 V-cycle and Schwarz inverses, FP64 elsewhere.
+                          On the FP64 path the trailing products of Schwarz inverses of more than 160
+                          unknowns are summed in 57-bit fixed point under one power of two per row (column)
+                          and panel: errors in the norm and by row as with FP64 products, but entries far
+                          below their row's largest keep fewer digits (none below 2^-62 of it) */
   int krylov;          /* FSI_FGMRES (0): right-preconditioned flexible GMRES, true-residual test;
                           FSI_GMRES_LEFT (1): left-preconditioned GMRES, the paper's setting (Sec. 4.1) */
   int gs_passes;       /* classical Gram-Schmidt passes per Arnoldi step: 1 or 2 (0: 2 for FGMRES,

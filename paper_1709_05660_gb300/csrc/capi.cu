@@ -907,8 +907,7 @@ void schwarz_factor(Ctx& c) {
       by += D.factor_bytes;
       fl += D.factor_flops;
     }
-    // launches: one gather for all levels (one per level past the table's
-    // capacity) and the tensor-core factorisation
+    // launches: one gather and one tensor-core factorisation for all levels
     Prof pr(c, FSI_K_PATCH_FACTOR, by, fl, 2);
     const bool all = gather_mixed(c, lv, first, max_n);
     if (all && (lv.nlev == 0 || launch_patch_gj_tc_levels(lv, first, max_n, c.status, c.stream, c.gj_panel))) {
@@ -1012,7 +1011,7 @@ void drop_vcycle_graph(Ctx& c) {
 // ends of the chain nonsingular beside the left ones.  The result is therefore
 // checked on one vector, and the factorisation redone by the LU or the chain from one
 // end (coarse_refactor) when that fails.  Largest row of |A x - v| / (|A| |x| + |v|)
-// over 200 problems of 2 to 4 levels on GB300: 2D 3e-14 to 1.5e-9 (the LU of the
+// over 144 factorisations (2 to 4 levels) on GB300: 2D 3e-14 to 1.5e-9 (the LU of the
 // same operators 2e-12 to 5e-9), 3D 9e-13 to 2.6e-8 (from one end 2e-11 to 2.3e-8), so
 // the operators' conditioning sets it and the limit lies above the largest.
 constexpr double kCoarseCheckTol = 1e-7;

@@ -31,7 +31,13 @@ __device__ __forceinline__ bool key_wins(unsigned long long ok, int oi, unsigned
 // both exact in 64 bits for up to 32 terms.  What is left out (the lo lo
 // products, the rounding of X and of MID / 2^29) is below 2^-55 of the product
 // of the two largest entries per term, where FP64 rounds each product to
-// 2^-53 of itself: the same normwise accuracy or better.
+// 2^-53 of itself.  (Exact integer products of a two-digit split, the family of
+// Ozaki, Ogita, Oishi and Rump's splittings for accurate matrix products.)  Inverses of
+// 73 Schwarz blocks of 204 to 372 unknowns against a refined extended-precision one,
+// relative to the sweep with FP64 products: error in the norm 0.91 (worst block 7.5e-15
+// against 5.0e-14), worst row 0.89, median entry 0.93.  Entries far below their row's
+// largest lose: one solid block of 204 unknowns has its median entry 13 times worse
+// (8e-14), with the norm and the rows better.
 // ---------------------------------------------------------------------------
 constexpr int kFixTerms = 32;
 

@@ -276,14 +276,16 @@ int run_merge(const CoarseTree& tr, int64_t n, int p, size_t smem, double* A, do
 }  // namespace
 
 bool coarse_merge_fits(int max_leaf, int p, int max_s) {
-  // 2 KB of the 227 KB are left to the static shared memory
+  // leaves and planes as gj_inverse_smem takes them (16 x 8 cells, slabs of 144: coarse factor 3.2 ms; 16 x 9, slabs
+  // of 163, by the banded LU: 27.8); 2 KB of the 227 KB are left to the static shared memory
   return max_leaf <= kGjSmemMax && p <= kGjSmemMax && p % 2 == 0 &&
          merge_smem(max_leaf, p, max_s, kMaxMergeCols) <= 225 * 1024;
 }
 
 // Columns per task: the last level's n columns as one task per SM where the
-// accumulators allow it (an unused accumulator costs as much as a used one:
-// 1,444 columns, 10 instead of 12: last level 250 -> 215 us)
+// accumulators allow it (the 16 x 4 grid's 1,074: 8).  An unused accumulator costs as
+// much as a used one: over all 1,444 unknowns of that grid, before the Dirichlet ones
+// were left out, the last level took 215 us with 10 columns a task and 250 with 12.
 int launch_coarse_merge(const CoarseTree& tr, int64_t n, int p, int max_leaf, int max_s, double* A, double* Lbuf,
                         double* Bbuf, double* gh, double* Ainv, int32_t* status, int sm_count,
                         cudaStream_t st) {

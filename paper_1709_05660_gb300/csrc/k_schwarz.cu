@@ -328,12 +328,6 @@ k_patch_gj_t(const int32_t* __restrict__ p_n, const int32_t* __restrict__ p_nown
   if (threadIdx.x == 0 && s_sing) atomicExch(&status[ST_SINGULAR], 1);
 }
 
-// FP64 blocks of at most kGjSmemMax unknowns: the whole block in shared memory
-// (transposed on the way in: columns contiguous), gj_inverse_smem.  Two thread
-// blocks share an SM up to about 110 unknowns, so one's pivot chain runs beside
-// the other's updates.  GB300, 3-level channel (2 x 2-element blocks of 112
-// unknowns): 3.3 -> 1.58 ms against the sweep that updates every
-// element in every step.
 // the level of a table that this thread block belongs to
 template <typename T>
 __device__ __forceinline__ const GjLevelT<T>& gj_level(const GjLevelsT<T>& lv) {
@@ -342,6 +336,12 @@ __device__ __forceinline__ const GjLevelT<T>& gj_level(const GjLevelsT<T>& lv) {
   return lv.l[l];
 }
 
+// FP64 blocks of at most kGjSmemMax unknowns: the whole block in shared memory
+// (transposed on the way in: columns contiguous), gj_inverse_smem.  Two thread
+// blocks share an SM up to about 110 unknowns, so one's pivot chain runs beside
+// the other's updates.  GB300, 3-level channel (2 x 2-element blocks of 112
+// unknowns): 3.3 -> 1.58 ms against the sweep that updates every
+// element in every step.
 constexpr int kGjPad = 1;   // column stride n + 1: conflict-free transposed stores
 __global__ void __launch_bounds__(512)
 k_patch_gj_small(const GjLevelsT<double> lv) {

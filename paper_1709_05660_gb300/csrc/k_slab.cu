@@ -307,6 +307,8 @@ size_t slab_gj_smem(int m, int ng) {
 size_t slab_gj_scratch(int m) { return (size_t)((m + kSlabW - 1) / kSlabW) * kSlabW * ((m + 1) & ~1); }
 int slab_gj_panels(int m) { return (m + kSlabW - 1) / kSlabW; }
 
+// Two rows per thread, and the block's panels in shared memory.  16 x 5 x 4 cells (slabs of
+// 836): coarse factor 36 ms; 16 x 5 x 5 (1,072, from one end by the banded LU kernels): 188.
 bool slab_gj_fits(int m, int sm_count) {
   return m <= kSlabThreads * kSlabRows && sm_count >= 4 && slab_gj_smem(m, sm_count / 2) <= 200 * 1024;
 }
